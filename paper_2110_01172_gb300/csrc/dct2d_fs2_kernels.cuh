@@ -37,6 +37,8 @@
 #include "dct2d_kernels.cuh"
 #include "fft_soa.cuh"
 #include "l2_hint.cuh"
+#include "launch_dep.cuh"
+#include "row_pairs.cuh"
 
 #include <type_traits>
 
@@ -680,21 +682,6 @@ __device__ __forceinline__ void fwd_rows_of(const Dct2dArgs& a, const float2* Zw
   *m = Zw + (long long)fs2_prow(row_mirror(k, a.n1), a.fsA, a.fsB) * (L / 2);
 }
 
-// First-stage butterfly of thread g of a group of TPS threads, arranged so that
-// the butterfly t and its mirror TPS-1-t sit in lanes l and l^m of one warp
-// (m = 16, or 15 when a warp holds two 16-thread groups).
-template <int TPS>
-__device__ __forceinline__ int mirror_lane_butterfly(int g) {
-  if constexpr (TPS >= 32) {
-    const int w = g >> 5, l = g & 31;
-    return l < 16 ? 16 * w + l : TPS + 15 - 16 * w - l;
-  } else {
-    return g;
-  }
-}
-template <int TPS>
-constexpr int mirror_lane_mask() { return TPS >= 32 ? 16 : TPS - 1; }
-
 // Forward split of two items from the workspace into SoA registers: point
 // n2 = t + TPS j of u = V_col(k1, :) is (z(p) + conj m(p)) / 2 for n2 < L/2
 // (p = n2) and (z(p) - conj m(p)) / 2i above (p = L-1-n2); the 1/2 is left out
@@ -722,7 +709,7 @@ __device__ __forceinline__ void fwd_split_x2(const float2* __restrict__ za, cons
                                              const float2* __restrict__ zb, const float2* __restrict__ mb, int t,
                                              bool packed, soa::C2* v) {
   constexpr int TPS = fft_tps(L);
-  constexpr int MASK = mirror_lane_mask<TPS>();
+  constexpr int MASK = rowp::rev_lane_mask<TPS>();
   const uint64_t pol = l2::evict_first();  // last use of the workspace
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -734,63 +721,46 @@ __device__ __forceinline__ void fwd_split_x2(const float2* __restrict__ za, cons
   }
 }
 
-// Forward combine (Section III-B, Eqs. four-elements / s-t) of both items from
-// the row spectra Y in s, one column pair (c, L-c) per thread and iteration:
-// u = aP + conj(aM), w = aP - conj(aM) (P = Y(c), M = Y(L-c)); with s = b u,
-// t = b w (b/2 in the table): y(k1,c) = Re s, y(kmir,c) = -Im t,
-// y(k1,L-c) = -Im s, y(kmir,L-c) = -Re t.  Packed lane a: a = 1 for row 0
-// and w = sqrt(1/2) (M.x - P.x, -(P.y + M.y)) for row N1/2.
-template <int L, int ST = 1>
-__device__ __forceinline__ void fwd_post_x2(const float4* __restrict__ s, const Dct2dArgs& a, float* y, int k1,
-                                            int kb, bool packed, int g) {
-  constexpr int TPS = fft_tps(L);
-  constexpr float RH = 0.70710678118654752f;
+// Forward postprocess of both items (rowp::fwd_post) into the output rows k1,
+// N1-k1 (lane a; rows 0 and N1/2 of the packed item) and kb, N1-kb (lane b).
+// GENERAL: plans with the DST-II order or a magnitude threshold.
+template <int L, bool GENERAL, bool FIRST>
+__device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, float* y, int k1, int kb, bool packed,
+                                            int g) {
   const int N1 = a.n1;
   const float2 fa0 = __ldg(a.fa + k1), fa1 = __ldg(a.fa + kb);
   // 1/2 of the split folded into the a-twiddle (not for the packed item)
   const float2 avr = make_float2(packed ? 1.f : 0.5f * fa0.x, 0.5f * fa1.x);
   const float2 avi = make_float2(packed ? 0.f : 0.5f * fa0.y, 0.5f * fa1.y);
-  const bool rev = a.vkind == 1;  // DST-II: output (k1, k2) goes to (N1-1-k1, N2-1-k2)
+  const bool rev = GENERAL && a.vkind == 1;  // DST-II: output (k1, k2) goes to (N1-1-k1, N2-1-k2)
   const int kma = row_mirror(k1, N1), kmb = row_mirror(kb, N1);
-  float* ya0 = y + (long long)(rev ? N1 - 1 - k1 : k1) * L;
-  float* ya1 = y + (long long)(rev ? N1 - 1 - kma : kma) * L;
-  float* yb0 = y + (long long)(rev ? N1 - 1 - kb : kb) * L;
-  float* yb1 = y + (long long)(rev ? N1 - 1 - kmb : kmb) * L;
-  const uint64_t pol = l2::evict_first();  // the output is streamed out
-  // magnitude threshold of Section V-A, Eq. image-compression (0: off)
-  const float eps = a.thresh;
-  auto st = [&](float* p, float v) { l2::st(p, (eps > 0.f && fabsf(v) < eps) ? 0.f : v, pol); };
-  auto column = [&](int c) {
-    const soa::C2 P = soa::unpack(s[ST * soa::pidx4(c)]);
-    const soa::C2 M = soa::unpack(s[ST * soa::pidx4((L - c) & (L - 1))]);
-    const soa::C2 aP = soa::mulw(P, avr, avi), aM = soa::mulw(M, avr, avi);
-    const soa::C2 u{soa::add2(aP.re, aM.re), soa::sub2(aP.im, aM.im)};
-    soa::C2 w{soa::sub2(aP.re, aM.re), soa::add2(aP.im, aM.im)};
-    if (packed) {
-      w.re.x = RH * (M.re.x - P.re.x);
-      w.im.x = -RH * (P.im.x + M.im.x);
-    }
-    const float2 bt = __ldg(a.fb + c);
-    const soa::C2 sv = soa::mulw(u, soa::bc(bt.x), soa::bc(bt.y));
-    const soa::C2 tv = soa::mulw(w, soa::bc(bt.x), soa::bc(bt.y));
-    const int c0 = rev ? L - 1 - c : c, c1 = rev ? c - 1 : L - c;  // stored columns of c and L-c
-    st(ya0 + c0, sv.re.x);
-    st(yb0 + c0, sv.re.y);
-    st(ya1 + c0, -tv.im.x);
-    st(yb1 + c0, -tv.im.y);
-    if (c != 0 && c != L / 2) {
-      st(ya0 + c1, -sv.im.x);
-      st(yb0 + c1, -sv.im.y);
-      st(ya1 + c1, -tv.re.x);
-      st(yb1 + c1, -tv.re.y);
-    }
-  };
-#pragma unroll 2
-  for (int r = 0; r < L / 2 / TPS; ++r) column(g + TPS * r);
-  if (g == 0) column(L / 2);
+  rowp::FwdOut<L, GENERAL> out;
+  out.a0 = y + (long long)(rev ? N1 - 1 - k1 : k1) * L;
+  out.a1 = y + (long long)(rev ? N1 - 1 - kma : kma) * L;
+  out.b0 = y + (long long)(rev ? N1 - 1 - kb : kb) * L;
+  out.b1 = y + (long long)(rev ? N1 - 1 - kmb : kmb) * L;
+  out.pol = l2::evict_first();  // the output is streamed out
+  out.eps = a.thresh;           // magnitude threshold of Section V-A, Eq. image-compression (0: off)
+  out.rev = rev;
+  rowp::fwd_post<L, FIRST, GENERAL>(v, out, avr, avi, a.fb4, g, packed);
 }
 
-template <int L>
+// Row FFT of both items from registers (v: points t + TPS j of the thread's
+// first-stage butterfly t) and the postprocess.
+template <int L, bool GENERAL>
+__device__ __forceinline__ void fwd_fft_post_x2(soa::C2* v, float4* s, const Dct2dArgs& a, float* y, int k1, int kb,
+                                                bool packed, int t, int g, int group) {
+  constexpr int TPS = fft_tps(L);
+  soa::first_stage<L, false>(v, s, t);
+  rowp::stages_to_regs<L, 16, false, true>(s, g, group, a.tw2x, v);
+  pdl::launch_dependents();
+  if (rowp::warp_has_first<TPS>(packed))
+    fwd_post_x2<L, GENERAL, true>(v, a, y, k1, kb, packed, g);
+  else
+    fwd_post_x2<L, GENERAL, false>(v, a, y, k1, kb, false, g);
+}
+
+template <int L, bool GENERAL>
 __global__ void __launch_bounds__(RowX2Geom<L>::THREADS, RowX2Geom<L>::MINB) k_fs2_rows_fwd_x2(Dct2dArgs a) {
   using R = RowX2Geom<L>;
   extern __shared__ float4 sxf[];
@@ -803,21 +773,19 @@ __global__ void __launch_bounds__(RowX2Geom<L>::THREADS, RowX2Geom<L>::MINB) k_f
   fwd_rows_of<L>(a, Zw, k1 + 1, &zb, &mb);
   soa::C2 v[16];
   const bool packed = (k1 == 0);
-  const int t = mirror_lane_butterfly<R::TPS>(g);
-  fwd_split_x2<L>(za, ma, zb, mb, t, packed, v);
-  soa::first_stage<L, false>(v, s, t);
-  __syncthreads();
-  soa::stages<L, 16, false>(s, g, a.tw2x);
-  fwd_post_x2<L>(s, a, a.out + (long long)blockIdx.z * a.out_bstride, k1, k1 + 1, packed, g);
+  const int t = rowp::rev_lane_butterfly<R::TPS>(g);
+  if (rowp::warp_has_first<R::TPS>(packed))
+    fwd_split_x2<L>(za, ma, zb, mb, t, packed, v);
+  else
+    fwd_split_x2<L>(za, ma, zb, mb, t, false, v);
+  fwd_fft_post_x2<L, GENERAL>(v, s, a, a.out + (long long)blockIdx.z * a.out_bstride, k1, k1 + 1, packed, t, g, pi);
 }
 
 // Inverse four-read preprocess (Eq. 2d_idct_pre, conjugated twiddle, 1/(N1 N2)
-// in the a-table) of one item at the thread's points k2 = g + TPS j, as
-// (x, ia) pairs: x = (c1 - c2, -(c3 + c4)) b_k2 for a normal item, where
-// c1 = C(k1,k2), c3 = C(kmir,k2), c4 = C(k1,N2-k2), c2 = C(kmir,N2-k2) (zero
-// past the edge).  The kind's maps are folded into the reads: DST-II reads rows
-// N1-1-k and columns reversed; IDCT_IDXST swaps the reads at k2 and N2-k2
-// (column 0 zero); IDXST_IDCT swaps the item's two rows (row 0 zero).
+// in the a-table) of one item, from C(k1,k2), C(kmir,k2), C(k1,N2-k2) and
+// C(kmir,N2-k2) (zero past the edge).  The kind's maps are folded into the reads:
+// DST-II reads rows N1-1-k and columns reversed; IDCT_IDXST swaps the reads at
+// k2 and N2-k2 (column 0 zero); IDXST_IDCT swaps the item's two rows (row 0 zero).
 struct InvRows {
   const float* ra;  // row of c1 / c4 (null: zero row)
   const float* rb;  // row of c3 / c2
@@ -855,57 +823,41 @@ __device__ __forceinline__ float inv_ld(const float* p, uint64_t pol) {
   }
 }
 
-// The four reads c1, c3, c4, c2 of point k2 of one item.
-template <int L, bool MAPPED, bool STAGED = false>
-__device__ __forceinline__ float4 inv_reads(const InvRows& r, int k2, bool rev, bool swapc, uint64_t pol) {
-  const int km = (L - k2) & (L - 1);
-  float c1, c3, c4, c2;
+// The reads of columns k2 and km = L - k2 of one item (edge: k2 = 0, whose
+// mirror reads are zero); ROW0: the item's first row may be null (a zero row).
+template <int L, bool MAPPED, bool STAGED, bool ROW0>
+__device__ __forceinline__ rowp::Quad inv_quad(const InvRows& r, int k2, int km, bool edge, bool rev, bool swapc,
+                                               uint64_t pol) {
+  const bool has = !ROW0 || r.ra;
+  rowp::Quad q;
   if constexpr (!MAPPED) {
-    c1 = r.ra ? inv_ld<STAGED>(r.ra + k2, pol) : 0.f;
-    c3 = inv_ld<STAGED>(r.rb + k2, pol);
-    c4 = (k2 && r.ra) ? inv_ld<STAGED>(r.ra + km, pol) : 0.f;
-    c2 = k2 ? inv_ld<STAGED>(r.rb + km, pol) : 0.f;
+    q.c1 = has ? inv_ld<STAGED>(r.ra + k2, pol) : 0.f;
+    q.c3 = inv_ld<STAGED>(r.rb + k2, pol);
+    q.c4 = (has && !edge) ? inv_ld<STAGED>(r.ra + km, pol) : 0.f;
+    q.c2 = !edge ? inv_ld<STAGED>(r.rb + km, pol) : 0.f;
   } else {
     const int ka = swapc ? km : k2, kb = swapc ? k2 : km;
     const int pa = rev ? L - 1 - ka : ka, pb = rev ? L - 1 - kb : kb;
-    const bool z0 = swapc && !k2;
-    c1 = (!r.ra || z0) ? 0.f : inv_ld<STAGED>(r.ra + pa, pol);
-    c3 = z0 ? 0.f : inv_ld<STAGED>(r.rb + pa, pol);
-    c4 = (k2 && r.ra) ? inv_ld<STAGED>(r.ra + pb, pol) : 0.f;
-    c2 = k2 ? inv_ld<STAGED>(r.rb + pb, pol) : 0.f;
+    const bool z0 = swapc && edge;
+    q.c1 = (has && !z0) ? inv_ld<STAGED>(r.ra + pa, pol) : 0.f;
+    q.c3 = !z0 ? inv_ld<STAGED>(r.rb + pa, pol) : 0.f;
+    q.c4 = (has && !edge) ? inv_ld<STAGED>(r.ra + pb, pol) : 0.f;
+    q.c2 = !edge ? inv_ld<STAGED>(r.rb + pb, pol) : 0.f;
   }
-  return make_float4(c1, c3, c4, c2);
+  return q;
 }
 
-template <int L, bool MAPPED, bool PACKED, bool STAGED = false>
-__device__ __forceinline__ void inv_pre_x2(const Dct2dArgs& a, const InvRows& A, const InvRows& B, int k1, int kb,
-                                           int g, soa::C2* v) {
-  constexpr int TPS = fft_tps(L);
+// Preprocess of both items: points t + TPS j of the returned butterfly t in v.
+template <int L, bool MAPPED, bool FIRST, bool STAGED = false>
+__device__ __forceinline__ int inv_pre_x2(const Dct2dArgs& a, const InvRows& A, const InvRows& B, int k1, int kb,
+                                          bool packed, int g, soa::C2* v) {
   const bool rev = MAPPED && a.vkind == 1, swapc = MAPPED && a.vkind == 2;
-  const float2 iaA = __ldg(a.ia + k1), iaB = __ldg(a.ia + kb);
-  const float2 ih = __ldg(a.ia + a.n1 / 2);
-  const float2 iar = make_float2(iaA.x, iaB.x), iai = make_float2(iaA.y, iaB.y);
   const uint64_t pol = l2::evict_first();  // the input is streamed in
-  // points j and 15 - j back to back: the value read at N2 - k2 is read again
-  // as the k2 point of the mirror thread TPS - g at iteration 15 - j, so the
-  // two reads of every input value fall close together and the second hits L1
-#pragma unroll
-  for (int jj = 0; jj < 16; ++jj) {
-    const int j = (jj & 1) ? 15 - (jj >> 1) : (jj >> 1);
-    const int k2 = g + TPS * j;
-    const float4 ca = inv_reads<L, MAPPED, STAGED>(A, k2, rev, swapc, pol);
-    const float4 cb = inv_reads<L, MAPPED, STAGED>(B, k2, rev, swapc, pol);
-    const float2 bk = __ldg(a.ib + k2);
-    // x = (c1 - c2, -(c3 + c4)), v = x b ia
-    const soa::C2 x{make_float2(ca.x - ca.w, cb.x - cb.w), make_float2(-(ca.y + ca.z), -(cb.y + cb.z))};
-    v[j] = soa::mulw(soa::mulw(x, soa::bc(bk.x), soa::bc(bk.y)), iar, iai);
-    if constexpr (PACKED) {  // lane a: rows 0 and N1/2 packed as re / im of one sequence
-      const float2 v0 = cmul(cmul(make_float2(ca.x, -ca.z), bk), iaA);
-      const float2 vh = cmul(cmul(make_float2(ca.y - ca.w, -(ca.y + ca.w)), bk), ih);
-      v[j].re.x = v0.x - vh.y;
-      v[j].im.x = v0.y + vh.x;
-    }
-  }
+  auto quads = [&](int k2, int km, bool edge, rowp::Quad& qa, rowp::Quad& qb) {
+    qa = inv_quad<L, MAPPED, STAGED, FIRST>(A, k2, km, edge, rev, swapc, pol);
+    qb = inv_quad<L, MAPPED, STAGED, false>(B, k2, km, edge, rev, swapc, pol);
+  };
+  return rowp::inv_pre<L, FIRST>(quads, a.ib, __ldg(a.ia + k1), __ldg(a.ia + kb), __ldg(a.ia + a.n1 / 2), packed, g, v);
 }
 
 // Inverse pairing of both items: row IFFT u in s -> workspace rows k1 and its
@@ -913,23 +865,21 @@ __device__ __forceinline__ void inv_pre_x2(const Dct2dArgs& a, const InvRows& A,
 // one column p per thread and iteration; packed lane a: the real and imaginary
 // parts go to rows 0 and N1/2.
 template <int L>
-__device__ __forceinline__ void inv_pair_x2(const float4* __restrict__ s, const Dct2dArgs& a, float2* Zw, int k1,
-                                            bool packed, int g) {
-  constexpr int TPS = fft_tps(L);
+__device__ __forceinline__ void inv_pair_x2(const soa::C2* v, const Dct2dArgs& a, float2* Zw, int k1, bool packed,
+                                            int g) {
   float2* za = Zw + (long long)fs2_prow(k1, a.fsA, a.fsB) * (L / 2);
   float2* ma = Zw + (long long)fs2_prow(row_mirror(k1, a.n1), a.fsA, a.fsB) * (L / 2);
   float2* zb = Zw + (long long)fs2_prow(k1 + 1, a.fsA, a.fsB) * (L / 2);
   float2* mb = Zw + (long long)fs2_prow(row_mirror(k1 + 1, a.n1), a.fsA, a.fsB) * (L / 2);
   const uint64_t pol = l2::evict_last();  // read again by the next column step
-#pragma unroll 2
-  for (int r = 0; r < L / 2 / TPS; ++r) {
-    const int p = g + TPS * r;
-    const soa::C2 u = soa::unpack(s[soa::pidx4(p)]), w = soa::unpack(s[soa::pidx4(L - 1 - p)]);
-    l2::st(zb + p, make_float2(u.re.y - w.im.y, u.im.y + w.re.y), pol);
-    l2::st(mb + p, make_float2(u.re.y + w.im.y, w.re.y - u.im.y), pol);
-    l2::st(za + p, packed ? make_float2(u.re.x, w.re.x) : make_float2(u.re.x - w.im.x, u.im.x + w.re.x), pol);
-    l2::st(ma + p, packed ? make_float2(u.im.x, w.im.x) : make_float2(u.re.x + w.im.x, w.re.x - u.im.x), pol);
-  }
+  rowp::inv_pairs<L>(v, g, [&](int base, int off, const soa::C2& u, const soa::C2& w) {
+    l2::st(zb + base + off, make_float2(u.re.y - w.im.y, u.im.y + w.re.y), pol);
+    l2::st(mb + base + off, make_float2(u.re.y + w.im.y, w.re.y - u.im.y), pol);
+    l2::st(za + base + off,
+           packed ? make_float2(u.re.x, w.re.x) : make_float2(u.re.x - w.im.x, u.im.x + w.re.x), pol);
+    l2::st(ma + base + off,
+           packed ? make_float2(u.im.x, w.im.x) : make_float2(u.re.x + w.im.x, w.re.x - u.im.x), pol);
+  });
 }
 
 // MAPPED: the DST-II / IDCT_IDXST index maps folded into the reads (a separate
@@ -945,14 +895,18 @@ __global__ void __launch_bounds__(RowX2Geom<L>::THREADS, RowX2Geom<L>::MINB_INV)
   const InvRows A = inv_rows_of(a, C, k1, L), B = inv_rows_of(a, C, k1 + 1, L);
   const bool packed = (k1 == 0);
   soa::C2 v[16];
-  if (packed)
-    inv_pre_x2<L, MAPPED, true>(a, A, B, k1, k1 + 1, g, v);
+  int t;
+  if (rowp::warp_has_first<R::TPS>(packed))
+    t = inv_pre_x2<L, MAPPED, true>(a, A, B, k1, k1 + 1, packed, g, v);
   else
-    inv_pre_x2<L, MAPPED, false>(a, A, B, k1, k1 + 1, g, v);
-  soa::first_stage<L, true>(v, s, g);
-  __syncthreads();
-  soa::stages<L, 16, true>(s, g, a.tw2x);
-  inv_pair_x2<L>(s, a, a.work + (long long)blockIdx.z * a.work_bstride, k1, packed, g);
+    t = inv_pre_x2<L, MAPPED, false>(a, A, B, k1, k1 + 1, false, g, v);
+  soa::first_stage<L, true>(v, s, t);
+  rowp::stages_to_regs<L, 16, true, false>(s, g, pi, a.tw2x, v);
+  float2* Zw = a.work + (long long)blockIdx.z * a.work_bstride;
+  if (rowp::warp_has_first<R::TPS>(packed))
+    inv_pair_x2<L>(v, a, Zw, k1, packed, g);
+  else
+    inv_pair_x2<L>(v, a, Zw, k1, false, g);
 }
 
 }  // namespace gbdct

@@ -50,6 +50,7 @@ struct Dct2dArgs {
   const float2* tw2;  // stage twiddles for length N2
   const float2* fa;   // a_k1, k1 in [0, N1/2]
   const float2* fb;   // b_k2 / 2, k2 in [0, N2)
+  const float4* fb4;  // b_k2 / 2 as (br, br, bi, bi) (two-item row passes)
   const float2* ia;   // conj(a_k1) / (N1 N2), k1 in [0, N1/2]
   const float2* ib;   // conj(b_k2), k2 in [0, N2)
   int seq_per_cta;    // B

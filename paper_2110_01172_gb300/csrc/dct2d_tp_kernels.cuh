@@ -195,11 +195,11 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
   soa::C2 v[16];
 #pragma unroll
   for (int j = 0; j < 16; ++j) {
-    const int m = g + TPS * j;
+    const int m = g + TPS * j;  // in the first half for j < 8
     if constexpr (!INV) {
-      float4 q = buf[NP * (m < HALF ? m : 3 * HALF - 1 - m) + pi];
+      float4 q = j < 8 ? buf[NP * m + pi] : buf[NP * (3 * HALF - 1 - TPS * j) + pi - NP * g];
       if (a.vkind == 1) {  // DST-II: (-1)^(n1 + n2); rows of the first half even, second half odd
-        const float sr = m < HALF ? 1.f : -1.f;
+        const float sr = j < 8 ? 1.f : -1.f;
         q = vsign(q, sr, -sr);
       }
       v[j] = aos_to_soa(q);
@@ -268,11 +268,33 @@ struct TpRows {
   static constexpr int MINB = THREADS >= 512 ? 1 : 512 / THREADS;  // up to 128 registers
 };
 
-template <int L, bool NARROW>
+// The thread's points of both items in v, straight from the group's four
+// workspace rows (w1, w2: the radix-2 twiddles on O[c] and O[kb]).
+template <int L, bool FIRST>
+__device__ __forceinline__ void tp_fwd_load(const float2* e1r, const float2* o1r, const float2* e2r, const float2* o2r,
+                                            float2 w1, float2 w2, bool first, int t, soa::C2* v) {
+  constexpr int TPS = fft_tps(L);
+  constexpr int MASK = rowp::rev_lane_mask<TPS>();
+  const uint64_t pol = l2::evict_first();  // last use of the workspace
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int p = t + TPS * j;
+    const float2 e1 = l2::ld_once(e1r + p, pol), e2 = l2::ld_once(e2r + p, pol);
+    const float2 o1 = cmul(l2::ld_once(o1r + p, pol), w1), o2 = cmul(l2::ld_once(o2r + p, pol), w2);
+    const float2 P = cadd(e1, o1), Q = csub(e1, o1), Rr = cadd(e2, o2), S = csub(e2, o2);
+    // (z_a, m_a, z_b, m_b) = (V[c], V[N1-c], V[M-c], V[M+c]); first group:
+    // (V[0], V[M], V[M/2], V[3M/2])
+    const bool f = FIRST && first;
+    const float2 Am = f ? Q : Rr, B = f ? Rr : S, Bm = f ? S : Q;
+    split_point<MASK>(P, Am, B, Bm, f, v[j], v[15 - j]);
+  }
+}
+
+// GENERAL: plans with the DST-II order or a magnitude threshold (row_pairs.cuh).
+template <int L, bool NARROW, bool GENERAL>
 __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>::MINB) k_tp_rows_fwd(Dct2dArgs a) {
   using R = TpRows<L, NARROW>;
   constexpr int TPS = R::TPS;
-  constexpr int MASK = mirror_lane_mask<TPS>();
   extern __shared__ float4 sxt[];
   const int pi = threadIdx.x / TPS, g = threadIdx.x % TPS;
   float4* s = sxt + pi * R::LP;
@@ -289,70 +311,53 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
   const float2 w = __ldg(a.r2w + c);
   const float2 w1 = first ? make_float2(1.f, 0.f) : w;
   const float2 w2 = first ? __ldg(a.r2w + M / 2) : conjf2(w);
-  const int t = mirror_lane_butterfly<TPS>(g);
-  const uint64_t pol = l2::evict_first();  // last use of the workspace
+  const int t = rowp::rev_lane_butterfly<TPS>(g);
   pdl::wait_prior_grid();
   soa::C2 v[16];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int p = t + TPS * j;
-    const float2 e1 = l2::ld_once(e1r + p, pol), e2 = l2::ld_once(e2r + p, pol);
-    const float2 o1 = cmul(l2::ld_once(o1r + p, pol), w1), o2 = cmul(l2::ld_once(o2r + p, pol), w2);
-    const float2 P = cadd(e1, o1), Q = csub(e1, o1), Rr = cadd(e2, o2), S = csub(e2, o2);
-    // (z_a, m_a, z_b, m_b) = (V[c], V[N1-c], V[M-c], V[M+c]); first group:
-    // (V[0], V[M], V[M/2], V[3M/2])
-    const float2 Am = first ? Q : Rr, B = first ? Rr : S, Bm = first ? S : Q;
-    split_point<MASK>(P, Am, B, Bm, first, v[j], v[15 - j]);
-  }
-  soa::first_stage<L, false>(v, s, t);
-  __syncthreads();
-  soa::stages<L, 16, false>(s, g, a.tw2x);
-  pdl::launch_dependents();
-  fwd_post_x2<L>(s, a, a.out + (long long)blockIdx.z * a.out_bstride, c, kb, first, g);
+  if (rowp::warp_has_first<TPS>(first))
+    tp_fwd_load<L, true>(e1r, o1r, e2r, o2r, w1, w2, first, t, v);
+  else
+    tp_fwd_load<L, false>(e1r, o1r, e2r, o2r, w1, w2, false, t, v);
+  fwd_fft_post_x2<L, GENERAL>(v, s, a, a.out + (long long)blockIdx.z * a.out_bstride, c, kb, first, t, g, pi);
 }
 
-// Inverse pairing of both items into E' / O' rows: from the row IFFT u in s,
+// Inverse pairing of both items into E' / O' rows: from the row IFFT u in v,
 // Z(k, p) of the items' rows as in the four-step family's pairing, then
 //   E'[c] = V[c] + V[M+c],      O'[c] = conj(w) (V[c] - V[M+c])
 //   E'[M-c] = V[M-c] + V[N1-c], O'[M-c] = w (V[N1-c] - V[M-c])
 // and for the first group E'[0], O'[0] from V[0] +- V[M], E'[M/2] = V[M/2] +
 // V[3M/2], O'[M/2] = i (V[M/2] - V[3M/2]).
 template <int L>
-__device__ __forceinline__ void tp_inv_pair(const float4* __restrict__ s, const Dct2dArgs& a, float2* Zw, int c,
-                                            int kb, bool first, int g) {
-  constexpr int TPS = fft_tps(L);
+__device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a, float2* Zw, int c, int kb, bool first,
+                                            int g) {
   const int M = a.n1 / 2;
   float2* e1r = Zw + (long long)c * (L / 2);
   float2* o1r = Zw + (long long)(M + c) * (L / 2);
   float2* e2r = Zw + (long long)kb * (L / 2);
   float2* o2r = Zw + (long long)(M + kb) * (L / 2);
-  const float2 w = __ldg(a.r2w + c);
+  const float2 cw = __ldg(a.r2w + c);
   const uint64_t pol = l2::evict_last();  // read again by the column pass
-#pragma unroll 2
-  for (int r = 0; r < L / 2 / TPS; ++r) {
-    const int p = g + TPS * r;
-    const soa::C2 u = soa::unpack(s[soa::pidx4(p)]), wv = soa::unpack(s[soa::pidx4(L - 1 - p)]);
-    const float2 zb0 = make_float2(u.re.y - wv.im.y, u.im.y + wv.re.y);  // V[kb]
-    const float2 zb1 = make_float2(u.re.y + wv.im.y, wv.re.y - u.im.y);  // V[mirror of kb]
-    const float2 za0 = first ? make_float2(u.re.x, wv.re.x) : make_float2(u.re.x - wv.im.x, u.im.x + wv.re.x);
-    const float2 za1 = first ? make_float2(u.im.x, wv.im.x) : make_float2(u.re.x + wv.im.x, wv.re.x - u.im.x);
+  rowp::inv_pairs<L>(v, g, [&](int base, int off, const soa::C2& u, const soa::C2& w) {
+    const float2 zb0 = make_float2(u.re.y - w.im.y, u.im.y + w.re.y);  // V[kb]
+    const float2 zb1 = make_float2(u.re.y + w.im.y, w.re.y - u.im.y);  // V[mirror of kb]
+    const float2 za0 = first ? make_float2(u.re.x, w.re.x) : make_float2(u.re.x - w.im.x, u.im.x + w.re.x);
+    const float2 za1 = first ? make_float2(u.im.x, w.im.x) : make_float2(u.re.x + w.im.x, w.re.x - u.im.x);
     const float2 x1 = first ? za1 : zb1;  // V[c + M]
     const float2 x2 = first ? zb1 : za1;  // V[kb + M]
     const float2 d1 = csub(za0, x1);
     const float2 d2 = csub(zb0, x2);
-    const float2 o1 = first ? d1 : cmulc(d1, w);
-    const float2 o2 = first ? make_float2(-d2.y, d2.x) : cmul(make_float2(-d2.x, -d2.y), w);
-    l2::st(e1r + p, cadd(za0, x1), pol);
-    l2::st(o1r + p, o1, pol);
-    l2::st(e2r + p, cadd(zb0, x2), pol);
-    l2::st(o2r + p, o2, pol);
-  }
+    const float2 o1 = first ? d1 : cmulc(d1, cw);
+    const float2 o2 = first ? make_float2(-d2.y, d2.x) : cmul(make_float2(-d2.x, -d2.y), cw);
+    l2::st(e1r + base + off, cadd(za0, x1), pol);
+    l2::st(o1r + base + off, o1, pol);
+    l2::st(e2r + base + off, cadd(zb0, x2), pol);
+    l2::st(o2r + base + off, o2, pol);
+  });
 }
 
 // STAGED: the group's (up to) four input rows are first copied whole into its
 // shared buffer by contiguous bulk copies (one mbarrier per group, bounded
-// wait as in the column pass), so the preprocess reads each value from shared
-// memory instead of twice from global memory (at k2 and at N2 - k2); the
+// wait as in the column pass), so few registers hold loads in flight; the
 // buffer (17 L bytes) holds the 16 L bytes of the rows until the first FFT
 // stage overwrites it.  Device buffers only.
 
@@ -369,6 +374,7 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
   const float* C = a.in + (long long)blockIdx.z * a.in_bstride;
   const InvRows A = inv_rows_of(a, C, c, L), B = inv_rows_of(a, C, kb, L);
   soa::C2 v[16];
+  int t;
   if constexpr (STAGED) {
     uint64_t* bar = reinterpret_cast<uint64_t*>(sxti + R::NP * R::LP) + pi;
     int* flag = reinterpret_cast<int*>(reinterpret_cast<uint64_t*>(sxti + R::NP * R::LP) + R::NP);
@@ -401,23 +407,26 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
     if (!*flag) return;
     tma::test_wait(bar, 0);  // completed: every thread observes the copied rows
     const InvRows As{A.ra ? st : nullptr, st + L}, Bs{B.ra ? st + 2 * L : nullptr, st + 3 * L};
-    if (first)
-      inv_pre_x2<L, MAPPED, true, true>(a, As, Bs, c, kb, g, v);
+    if (rowp::warp_has_first<R::TPS>(first))
+      t = inv_pre_x2<L, MAPPED, true, true>(a, As, Bs, c, kb, first, g, v);
     else
-      inv_pre_x2<L, MAPPED, false, true>(a, As, Bs, c, kb, g, v);
-    __syncthreads();  // the first stage overwrites the staged rows
+      t = inv_pre_x2<L, MAPPED, false, true>(a, As, Bs, c, kb, false, g, v);
+    rowp::group_sync<R::TPS>(pi);  // the first stage overwrites the staged rows
   } else {
     pdl::wait_prior_grid();
-    if (first)
-      inv_pre_x2<L, MAPPED, true>(a, A, B, c, kb, g, v);
+    if (rowp::warp_has_first<R::TPS>(first))
+      t = inv_pre_x2<L, MAPPED, true>(a, A, B, c, kb, first, g, v);
     else
-      inv_pre_x2<L, MAPPED, false>(a, A, B, c, kb, g, v);
+      t = inv_pre_x2<L, MAPPED, false>(a, A, B, c, kb, false, g, v);
   }
-  soa::first_stage<L, true>(v, s, g);
-  __syncthreads();
-  soa::stages<L, 16, true>(s, g, a.tw2x);
+  soa::first_stage<L, true>(v, s, t);
+  rowp::stages_to_regs<L, 16, true, false>(s, g, pi, a.tw2x, v);
   pdl::launch_dependents();
-  tp_inv_pair<L>(s, a, a.work + (long long)blockIdx.z * a.work_bstride, c, kb, first, g);
+  float2* Zw = a.work + (long long)blockIdx.z * a.work_bstride;
+  if (rowp::warp_has_first<R::TPS>(first))
+    tp_inv_pair<L>(v, a, Zw, c, kb, first, g);
+  else
+    tp_inv_pair<L>(v, a, Zw, c, kb, false, g);
 }
 
 }  // namespace gbdct

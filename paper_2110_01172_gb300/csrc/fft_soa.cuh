@@ -166,51 +166,48 @@ __device__ __forceinline__ C2 apply(C2 u, C2 w) {
   return INV ? mulwc(u, w.re, w.im) : mulw(u, w.re, w.im);
 }
 
-// u[j] *= w^j (conjugated for the inverse), j = 1 .. R-1, where entry (j-1)*NS
-// of twp is w^j.  Only the power-of-two powers are read (w, w^2, w^4, w^8 for
-// R = 16); the other powers are products of at most three of them (a few ulp
-// from the exactly rounded values), which keeps the table reads (and
-// registers) low.
-template <int R, bool INV>
-__device__ __forceinline__ void twiddle(C2* u, const float4* __restrict__ twp, int NS) {
-  if constexpr (R == 16) {
-    const C2 w1 = ldw(twp), w2 = ldw(twp + NS), w4 = ldw(twp + 3 * NS), w8 = ldw(twp + 7 * NS);
-    const C2 w3 = wmul(w1, w2);
-    u[1] = apply<INV>(u[1], w1);
-    u[2] = apply<INV>(u[2], w2);
-    u[3] = apply<INV>(u[3], w3);
-    u[4] = apply<INV>(u[4], w4);
-    u[5] = apply<INV>(u[5], wmul(w1, w4));
-    u[6] = apply<INV>(u[6], wmul(w2, w4));
-    const C2 w7 = wmul(w3, w4);
-    u[7] = apply<INV>(u[7], w7);
-    u[8] = apply<INV>(u[8], w8);
-    u[9] = apply<INV>(u[9], wmul(w1, w8));
-    u[10] = apply<INV>(u[10], wmul(w2, w8));
-    u[11] = apply<INV>(u[11], wmul(w3, w8));
-    const C2 w12 = wmul(w4, w8);
-    u[12] = apply<INV>(u[12], w12);
-    u[13] = apply<INV>(u[13], wmul(w1, w12));
-    u[14] = apply<INV>(u[14], wmul(w2, w12));
-    u[15] = apply<INV>(u[15], wmul(w7, w8));
-  } else if constexpr (R == 8) {  // w, w^2, w^4 read; the rest are their products
-    const C2 w1 = ldw(twp), w2 = ldw(twp + NS), w4 = ldw(twp + 3 * NS);
-    const C2 w3 = wmul(w1, w2);
-    u[1] = apply<INV>(u[1], w1);
-    u[2] = apply<INV>(u[2], w2);
-    u[3] = apply<INV>(u[3], w3);
-    u[4] = apply<INV>(u[4], w4);
-    u[5] = apply<INV>(u[5], wmul(w1, w4));
-    u[6] = apply<INV>(u[6], wmul(w2, w4));
-    u[7] = apply<INV>(u[7], wmul(w3, w4));
-  } else if constexpr (R == 4) {
-    const C2 w1 = ldw(twp), w2 = ldw(twp + NS);
-    u[1] = apply<INV>(u[1], w1);
-    u[2] = apply<INV>(u[2], w2);
-    u[3] = apply<INV>(u[3], wmul(w1, w2));
-  } else {
+// Stage twiddles of one butterfly: the power-of-two powers of w (w, w^2, w^4,
+// w^8 for R = 16), entry (j-1)*NS of twp being w^j.  The other powers are
+// products of at most three of them (a few ulp from the exactly rounded
+// values), which keeps the table reads (and registers) low.
+template <int R>
+struct Tw {
+  static constexpr int N = R == 16 ? 4 : R == 8 ? 3 : R == 4 ? 2 : 1;
+  C2 w[N];
+  __device__ __forceinline__ void load(const float4* __restrict__ twp, int NS) {
 #pragma unroll
-    for (int j = 1; j < R; ++j) u[j] = apply<INV>(u[j], ldw(twp + (j - 1) * NS));
+    for (int i = 0; i < N; ++i) w[i] = ldw(twp + ((1 << i) - 1) * NS);
+  }
+};
+
+// u[j] *= w^j (conjugated for the inverse), j = 1 .. R-1.
+template <int R, bool INV>
+__device__ __forceinline__ void twiddle(C2* u, const Tw<R>& t) {
+  static_assert(R == 2 || R == 4 || R == 8 || R == 16, "stage radices");
+  const C2 w1 = t.w[0];
+  u[1] = apply<INV>(u[1], w1);
+  if constexpr (R >= 4) {
+    const C2 w2 = t.w[1], w3 = wmul(w1, w2);
+    u[2] = apply<INV>(u[2], w2);
+    u[3] = apply<INV>(u[3], w3);
+    if constexpr (R >= 8) {
+      const C2 w4 = t.w[2], w7 = wmul(w3, w4);
+      u[4] = apply<INV>(u[4], w4);
+      u[5] = apply<INV>(u[5], wmul(w1, w4));
+      u[6] = apply<INV>(u[6], wmul(w2, w4));
+      u[7] = apply<INV>(u[7], w7);
+      if constexpr (R >= 16) {
+        const C2 w8 = t.w[3], w12 = wmul(w4, w8);
+        u[8] = apply<INV>(u[8], w8);
+        u[9] = apply<INV>(u[9], wmul(w1, w8));
+        u[10] = apply<INV>(u[10], wmul(w2, w8));
+        u[11] = apply<INV>(u[11], wmul(w3, w8));
+        u[12] = apply<INV>(u[12], w12);
+        u[13] = apply<INV>(u[13], wmul(w1, w12));
+        u[14] = apply<INV>(u[14], wmul(w2, w12));
+        u[15] = apply<INV>(u[15], wmul(w7, w8));
+      }
+    }
   }
 }
 
@@ -218,31 +215,51 @@ __device__ __forceinline__ void twiddle(C2* u, const float4* __restrict__ twp, i
 // radix-16 DFT, outputs g*16 + m stored to s.  Point i of the sequence pair
 // lives at s[ST * pidx4(i)]: ST > 1 interleaves ST sequence pairs point by
 // point (the column passes of the two-pass family, whose warps span pairs).
+//
+// Addresses: every access of a stage is one per-thread base plus a multiple of
+// a compile-time step, because pidx4(i + 16 n) = pidx4(i) + 17 n; written that
+// way the steps become immediate offsets of the loads and stores (left to the
+// compiler, the shift in pidx4 costs about four integer instructions for each
+// of them, a quarter of all instructions of a column pass).
 template <int L, bool INV, int ST = 1>
 __device__ __forceinline__ void first_stage(C2* v, float4* __restrict__ s, int g) {
   constexpr int R = stage_radix(L, 1);
   dft<R, INV>(v);
+  float4* o = s + ST * pidx4(g * R);
 #pragma unroll
-  for (int m = 0; m < R; ++m) s[ST * pidx4(g * R + m)] = pack(v[m]);
+  for (int m = 0; m < R; ++m) o[ST * m] = pack(v[m]);
 }
 
-// Shared-memory slot of output point k of the last stage: OUT = 0 the padded
-// layout (pidx4), OUT = 1 dense (k), OUT = 2 dense with the upper half
+// Shared-memory form of the outputs of the last stage: OUT = 0 the padded
+// layout (pidx4), OUT = 1 dense (slot k), OUT = 2 dense with the upper half
 // reversed (L/2 + (L-1-k) for k >= L/2), the order in which a bulk tensor
 // store writes the rows of the two reorder residues.  Consecutive k of a
 // stage's last writes stay on distinct banks in all three.  The dense forms
 // are read by bulk tensor stores, so their slots hold the global-memory
 // layout (pack_aos) instead of the engine's two-lane layout (pack).
-template <int L, int OUT>
-__device__ __forceinline__ int out_slot(int k) {
-  if constexpr (OUT == 0) return pidx4(k);
-  else if constexpr (OUT == 1) return k;
-  else return k < L / 2 ? k : (3 * L / 2 - 1 - k);
+
+// The stage starting at NS of butterfly t of length L, as a pointer to its
+// first input and the step to the next (L/R is a multiple of 16 from the
+// second stage on).
+template <int L, int NS, int ST>
+__device__ __forceinline__ void load_butterfly(C2* u, const float4* __restrict__ s, int t) {
+  constexpr int R = stage_radix(L, NS), STRIDE = L / R;
+  static_assert(STRIDE % 16 == 0, "stage strides keep the padding step constant");
+  const float4* p = s + ST * pidx4(t);
+#pragma unroll
+  for (int j = 0; j < R; ++j) u[j] = unpack(p[ST * j * (STRIDE + STRIDE / 16)]);
+}
+template <int L, int NS, int ST>
+__device__ __forceinline__ void store_butterfly(const C2* u, float4* __restrict__ s, int t) {
+  constexpr int R = stage_radix(L, NS);
+  float4* p = s + ST * pidx4(stage_out_index<L, NS>(t, 0));
+#pragma unroll
+  for (int m = 0; m < R; ++m) p[ST * m * (NS + NS / 16)] = pack(u[m]);
 }
 
 // Stages NS .. L through shared memory (natural order in and out); every
 // thread of the CTA calls this (it contains __syncthreads).  The last stage
-// writes its outputs at out_slot<L, OUT>.
+// writes its outputs in the form OUT.
 template <int L, int NS, bool INV, int ST = 1, int OUT = 0>
 __device__ __forceinline__ void stages(float4* __restrict__ s, int g, const float4* __restrict__ tw) {
   if constexpr (NS < L) {
@@ -250,29 +267,30 @@ __device__ __forceinline__ void stages(float4* __restrict__ s, int g, const floa
     constexpr int P = fft_points(L);
     constexpr int TPS = fft_tps(L);
     constexpr int NB = P / R;
-    constexpr int STRIDE = L / R;
     C2 v[P];
 #pragma unroll
-    for (int q = 0; q < NB; ++q) {
-      const int t = g + q * TPS;
-#pragma unroll
-      for (int j = 0; j < R; ++j) v[q * R + j] = unpack(s[ST * pidx4(t + j * STRIDE)]);
-    }
+    for (int q = 0; q < NB; ++q) load_butterfly<L, NS, ST>(v + q * R, s, g + q * TPS);
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int t = g + q * TPS;
       C2* u = v + q * R;
-      const int k = t & (NS - 1);
-      twiddle<R, INV>(u, tw + tw_offset(L, NS) + k, NS);
+      Tw<R> w;
+      w.load(tw + tw_offset(L, NS) + (t & (NS - 1)), NS);
+      twiddle<R, INV>(u, w);
       dft<R, INV>(u);
-      if constexpr (NS * R < L) {
+      if constexpr (NS * R < L || OUT == 0) {
+        store_butterfly<L, NS, ST>(u, s, t);
+      } else {  // last stage: output m of butterfly t is point t + m NS
+        float4* p = s + ST * t;
 #pragma unroll
-        for (int m = 0; m < R; ++m) s[ST * pidx4(stage_out_index<L, NS>(t, m))] = pack(u[m]);
-      } else {
-#pragma unroll
-        for (int m = 0; m < R; ++m)
-          s[ST * out_slot<L, OUT>(stage_out_index<L, NS>(t, m))] = OUT ? pack_aos(u[m]) : pack(u[m]);
+        for (int m = 0; m < R; ++m) {
+          if (OUT == 1 || m < R / 2) {
+            p[ST * m * NS] = pack_aos(u[m]);
+          } else {
+            s[ST * (3 * L / 2 - 1 - m * NS) - ST * t] = pack_aos(u[m]);
+          }
+        }
       }
     }
     __syncthreads();

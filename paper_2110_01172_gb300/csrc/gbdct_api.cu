@@ -473,7 +473,7 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   const size_t ta = round_up(n1 / 2 + 1, 2);
   const size_t tb = round_up(n2, 2);
   const size_t tf = four_step ? round_up(n1, 2) : 0;
-  const size_t tx = two_item_rows ? 2 * t2 : 0;  // float4 copy of the N2 stage twiddles
+  const size_t tx = two_item_rows ? 2 * t2 + 2 * tb : 0;  // float4 copies of the N2 stage twiddles and of b / 2
   // two-pass family: stage twiddles of length N1/2 (float2 and float4 copies)
   // and the radix-2 twiddles W_N1^k
   const int totm = two_pass ? gbdct::tw_size_p(n1 / 2, p->pmax) : 0;
@@ -493,6 +493,7 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   float2* ib = fb + tb;
   p->fstw = four_step ? ib + tb : nullptr;
   float4* tw2x = two_item_rows ? reinterpret_cast<float4*>(ib + tb + tf) : nullptr;
+  float4* fb4 = two_item_rows ? tw2x + t2 : nullptr;
   float2* twm = two_pass ? ib + tb + tf + tx : nullptr;
   float4* tw1x = two_pass ? reinterpret_cast<float4*>(ib + tb + tf + tx + tm) : nullptr;
   float2* r2w = two_pass ? ib + tb + tf + tx + 3 * tm : nullptr;
@@ -522,6 +523,7 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   }
   if (p->fstw) k_gen_fs_twiddles<<<(n1 + 255) / 256, 256>>>(p->fstw, n1, fsA, fsB);
   if (tw2x && tot2 > 0) k_expand_twiddles<<<(tot2 + 255) / 256, 256>>>(tw2, tw2x, tot2);
+  if (fb4) k_expand_twiddles<<<(n2 + 255) / 256, 256>>>(fb, fb4, n2);
   if (two_pass) {
     if (totm > 0) {
       k_gen_stage_twiddles<<<(totm + 255) / 256, 256>>>(twm, n1 / 2, p->pmax, totm);
@@ -552,6 +554,7 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   a.r2w = r2w;
   a.fa = fa;
   a.fb = fb;
+  a.fb4 = fb4;
   a.ia = ia;
   a.ib = ib;
   a.fstw = p->fstw;

@@ -11,8 +11,11 @@ cudaError_t row_launch(bool inverse, const Dct2dArgs& a, int batch, cudaStream_t
   if constexpr (L <= 8192) {  // two items per thread group (packed two-lane arithmetic)
     using R = RowX2Geom<L>;
     if (prepare) {
-      cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_fs2_rows_fwd_x2<L>),
+      cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_fs2_rows_fwd_x2<L, false>),
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R::SMEM);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_fs2_rows_fwd_x2<L, true>),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R::SMEM);
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_fs2_rows_inv_x2<L, false>),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R::SMEM);
@@ -26,8 +29,10 @@ cudaError_t row_launch(bool inverse, const Dct2dArgs& a, int batch, cudaStream_t
       k_fs2_rows_inv_x2<L, true><<<grid, R::THREADS, R::SMEM, s>>>(a);
     else if (inverse)
       k_fs2_rows_inv_x2<L, false><<<grid, R::THREADS, R::SMEM, s>>>(a);
+    else if (a.vkind == 1 || a.thresh > 0.f)
+      k_fs2_rows_fwd_x2<L, true><<<grid, R::THREADS, R::SMEM, s>>>(a);
     else
-      k_fs2_rows_fwd_x2<L><<<grid, R::THREADS, R::SMEM, s>>>(a);
+      k_fs2_rows_fwd_x2<L, false><<<grid, R::THREADS, R::SMEM, s>>>(a);
     return cudaGetLastError();
   } else {
     using R = RowGeom<L>;

@@ -11,7 +11,8 @@ template <int L, bool NARROW>
 cudaError_t row_launch_g(bool inverse, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
   using R = TpRows<L, NARROW>;
   if (prepare) {
-    const void* plain[] = {reinterpret_cast<const void*>(k_tp_rows_fwd<L, NARROW>),
+    const void* plain[] = {reinterpret_cast<const void*>(k_tp_rows_fwd<L, NARROW, false>),
+                           reinterpret_cast<const void*>(k_tp_rows_fwd<L, NARROW, true>),
                            reinterpret_cast<const void*>(k_tp_rows_inv<L, false, false, NARROW>),
                            reinterpret_cast<const void*>(k_tp_rows_inv<L, true, false, NARROW>)};
     const void* staged[] = {reinterpret_cast<const void*>(k_tp_rows_inv<L, false, true, NARROW>),
@@ -36,8 +37,10 @@ cudaError_t row_launch_g(bool inverse, const Dct2dArgs& a, int batch, cudaStream
     return pdl::launch(k_tp_rows_inv<L, true, false, NARROW>, grid, dim3(R::THREADS), R::SMEM, s, a);
   else if (inverse)
     return pdl::launch(k_tp_rows_inv<L, false, false, NARROW>, grid, dim3(R::THREADS), R::SMEM, s, a);
+  else if (a.vkind == 1 || a.thresh > 0.f)
+    return pdl::launch(k_tp_rows_fwd<L, NARROW, true>, grid, dim3(R::THREADS), R::SMEM, s, a);
   else
-    return pdl::launch(k_tp_rows_fwd<L, NARROW>, grid, dim3(R::THREADS), R::SMEM, s, a);
+    return pdl::launch(k_tp_rows_fwd<L, NARROW, false>, grid, dim3(R::THREADS), R::SMEM, s, a);
 }
 
 // Narrow (64-thread) CTAs when wide ones would give fewer than two CTAs per SM.
