@@ -293,9 +293,11 @@ gbdct_status gbdct_multi_destroy(gbdct_multi_t m);
  *   xi1  = IDCT_IDXST(a wv / (wu^2 + wv^2))              field along axis 1
  * with wu = pi u / N1, wv = pi v / N2 and the (0,0) term set to zero (the paper
  * only says "scaled a1, a2"; these are the eigenfrequencies of the cosine
- * basis in grid units).  The solver owns three plans (DCT2, IDXST_IDCT,
- * IDCT_IDXST), the wu / wv tables and an N1 x N2 table of the eigenvalue
- * denominators 1 / (wu^2 + wv^2), all evaluated in FP64 at creation and
+ * basis in grid units).  Where the two-pass kernels apply (both sides between 64
+ * and 4096, and some with a side of 8192) the three inverses run as one batch
+ * over the one spectrum; other shapes run three plans (DCT2, IDXST_IDCT,
+ * IDCT_IDXST).  The solver owns the workspaces, the wu / wv tables and an
+ * N1 x N2 table of the eigenvalue denominators 1 / (wu^2 + wv^2), all evaluated in FP64 at creation and
  * rounded once to FP32.  Calls switch to the solver's device for their
  * duration.
  */

@@ -791,16 +791,16 @@ struct InvRows {
   const float* rb;  // row of c3 / c2
 };
 
-__device__ __forceinline__ InvRows inv_rows_of(const Dct2dArgs& a, const float* C, int k, int L) {
+__device__ __forceinline__ InvRows inv_rows_of(const Dct2dArgs& a, const float* C, int k, int L, int vkind) {
   const int N1 = a.n1;
   const int kmir = row_mirror(k, N1);
   int r0 = k, r1 = kmir;
-  if (a.vkind == 1) {
+  if (vkind == 1) {
     r0 = N1 - 1 - k;
     r1 = N1 - 1 - kmir;
   }
   InvRows r{C + (long long)r0 * L, C + (long long)r1 * L};
-  if (a.vkind == 3) {
+  if (vkind == 3) {
     if (k) {
       const float* t = r.ra;
       r.ra = r.rb;
@@ -812,50 +812,49 @@ __device__ __forceinline__ InvRows inv_rows_of(const Dct2dArgs& a, const float* 
   return r;
 }
 
-// One input value: from global memory with the L2 policy, or (STAGED) from a
-// copy of the row already in shared memory.
+// Reads of one item's two rows, first (c1, c4) and second (c3, c2), at a column:
+// from global memory with the L2 policy, or (STAGED) from copies of the rows
+// already in shared memory.
 template <bool STAGED>
-__device__ __forceinline__ float inv_ld(const float* p, uint64_t pol) {
-  if constexpr (STAGED) {
-    return *p;
-  } else {
-    return l2::ld(p, pol);
-  }
-}
+struct RowReads {
+  InvRows r;
+  uint64_t pol;
+  __device__ __forceinline__ bool has_a() const { return r.ra != nullptr; }
+  __device__ __forceinline__ float a(int c) const { return STAGED ? r.ra[c] : l2::ld(r.ra + c, pol); }
+  __device__ __forceinline__ float b(int c) const { return STAGED ? r.rb[c] : l2::ld(r.rb + c, pol); }
+};
 
 // The reads of columns k2 and km = L - k2 of one item (edge: k2 = 0, whose
-// mirror reads are zero); ROW0: the item's first row may be null (a zero row).
-template <int L, bool MAPPED, bool STAGED, bool ROW0>
-__device__ __forceinline__ rowp::Quad inv_quad(const InvRows& r, int k2, int km, bool edge, bool rev, bool swapc,
-                                               uint64_t pol) {
-  const bool has = !ROW0 || r.ra;
+// mirror reads are zero); ROW0: the item's first row may be missing (zero).
+template <int L, bool MAPPED, bool ROW0, typename Reads>
+__device__ __forceinline__ rowp::Quad inv_quad(const Reads& r, int k2, int km, bool edge, bool rev, bool swapc) {
+  const bool has = !ROW0 || r.has_a();
   rowp::Quad q;
   if constexpr (!MAPPED) {
-    q.c1 = has ? inv_ld<STAGED>(r.ra + k2, pol) : 0.f;
-    q.c3 = inv_ld<STAGED>(r.rb + k2, pol);
-    q.c4 = (has && !edge) ? inv_ld<STAGED>(r.ra + km, pol) : 0.f;
-    q.c2 = !edge ? inv_ld<STAGED>(r.rb + km, pol) : 0.f;
+    q.c1 = has ? r.a(k2) : 0.f;
+    q.c3 = r.b(k2);
+    q.c4 = (has && !edge) ? r.a(km) : 0.f;
+    q.c2 = !edge ? r.b(km) : 0.f;
   } else {
     const int ka = swapc ? km : k2, kb = swapc ? k2 : km;
     const int pa = rev ? L - 1 - ka : ka, pb = rev ? L - 1 - kb : kb;
     const bool z0 = swapc && edge;
-    q.c1 = (has && !z0) ? inv_ld<STAGED>(r.ra + pa, pol) : 0.f;
-    q.c3 = !z0 ? inv_ld<STAGED>(r.rb + pa, pol) : 0.f;
-    q.c4 = (has && !edge) ? inv_ld<STAGED>(r.ra + pb, pol) : 0.f;
-    q.c2 = !edge ? inv_ld<STAGED>(r.rb + pb, pol) : 0.f;
+    q.c1 = (has && !z0) ? r.a(pa) : 0.f;
+    q.c3 = !z0 ? r.b(pa) : 0.f;
+    q.c4 = (has && !edge) ? r.a(pb) : 0.f;
+    q.c2 = !edge ? r.b(pb) : 0.f;
   }
   return q;
 }
 
 // Preprocess of both items: points t + TPS j of the returned butterfly t in v.
-template <int L, bool MAPPED, bool FIRST, bool STAGED = false>
-__device__ __forceinline__ int inv_pre_x2(const Dct2dArgs& a, const InvRows& A, const InvRows& B, int k1, int kb,
+template <int L, bool MAPPED, bool FIRST, typename Reads>
+__device__ __forceinline__ int inv_pre_x2(const Dct2dArgs& a, const Reads& A, const Reads& B, int vkind, int k1, int kb,
                                           bool packed, int g, soa::C2* v) {
-  const bool rev = MAPPED && a.vkind == 1, swapc = MAPPED && a.vkind == 2;
-  const uint64_t pol = l2::evict_first();  // the input is streamed in
+  const bool rev = MAPPED && vkind == 1, swapc = MAPPED && vkind == 2;
   auto quads = [&](int k2, int km, bool edge, rowp::Quad& qa, rowp::Quad& qb) {
-    qa = inv_quad<L, MAPPED, STAGED, FIRST>(A, k2, km, edge, rev, swapc, pol);
-    qb = inv_quad<L, MAPPED, STAGED, false>(B, k2, km, edge, rev, swapc, pol);
+    qa = inv_quad<L, MAPPED, FIRST>(A, k2, km, edge, rev, swapc);
+    qb = inv_quad<L, MAPPED, false>(B, k2, km, edge, rev, swapc);
   };
   return rowp::inv_pre<L, FIRST>(quads, a.ib, __ldg(a.ia + k1), __ldg(a.ia + kb), __ldg(a.ia + a.n1 / 2), packed, g, v);
 }
@@ -892,14 +891,15 @@ __global__ void __launch_bounds__(RowX2Geom<L>::THREADS, RowX2Geom<L>::MINB_INV)
   float4* s = sxi + pi * R::LP;
   const int k1 = 2 * (blockIdx.x * R::NP + pi);
   const float* C = a.in + (long long)blockIdx.z * a.in_bstride;
-  const InvRows A = inv_rows_of(a, C, k1, L), B = inv_rows_of(a, C, k1 + 1, L);
+  const uint64_t pol = l2::evict_first();  // the input is streamed in
+  const RowReads<false> A{inv_rows_of(a, C, k1, L, a.vkind), pol}, B{inv_rows_of(a, C, k1 + 1, L, a.vkind), pol};
   const bool packed = (k1 == 0);
   soa::C2 v[16];
   int t;
   if (rowp::warp_has_first<R::TPS>(packed))
-    t = inv_pre_x2<L, MAPPED, true>(a, A, B, k1, k1 + 1, packed, g, v);
+    t = inv_pre_x2<L, MAPPED, true>(a, A, B, a.vkind, k1, k1 + 1, packed, g, v);
   else
-    t = inv_pre_x2<L, MAPPED, false>(a, A, B, k1, k1 + 1, false, g, v);
+    t = inv_pre_x2<L, MAPPED, false>(a, A, B, a.vkind, k1, k1 + 1, false, g, v);
   soa::first_stage<L, true>(v, s, t);
   rowp::stages_to_regs<L, 16, true, false>(s, g, pi, a.tw2x, v);
   float2* Zw = a.work + (long long)blockIdx.z * a.work_bstride;

@@ -70,6 +70,18 @@ struct Dct2dArgs {
   int nsm;            // host side only: multiprocessors of the device
 };
 
+// The three inverse transforms of a spectral Poisson solve (Section V-B,
+// Algorithm 4) as one batch over one spectrum: entry 0 the potential (DCT-II
+// inverse of a inv), 1 the field along axis 0 (IDXST_IDCT of a inv wu), 2 the
+// field along axis 1 (IDCT_IDXST of a inv wv).
+struct PoissonArgs {
+  const float* w;    // wu[n1], wv[n2]
+  const float* inv;  // 1 / (wu^2 + wv^2), n1 x n2, 0 at (0, 0)
+  float* out[3];
+};
+// The kind whose maps entry z folds in (gbdct_kind numbers).
+__host__ __device__ constexpr int poisson_vkind(int z) { return z == 0 ? 0 : z == 1 ? 3 : 2; }
+
 template <int L>
 __host__ __device__ constexpr int max_threads_for() { return L >= 16384 ? 1024 : 512; }
 

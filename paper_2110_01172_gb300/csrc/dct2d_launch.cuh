@@ -62,7 +62,17 @@ inline void fs2_split(int log2N1, int* A, int* B) {
 // column pass).
 cudaError_t run_tp(int log2N1, int log2N2, bool inverse, const Dct2dArgs& a, int batch, cudaStream_t s,
                    bool prepare);
-cudaError_t run_tp_cols(int lg1, bool inverse, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
+cudaError_t run_tp_cols_fwd(int lg1, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
+cudaError_t run_tp_cols_inv(int lg1, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
+cudaError_t run_tp_rows_fwd(int lg2, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
+cudaError_t run_tp_rows_inv(int lg2, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
+cudaError_t run_tp_cols_poisson(int lg1, const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare);
+cudaError_t run_tp_rows_poisson(int lg2, const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare);
+// The three inverses of a Poisson solve from the spectrum at a.in (the row pass
+// and the column pass once each, over a workspace of three entries).
+cudaError_t run_tp_poisson(int log2N1, int log2N2, const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s,
+                           bool prepare);
+constexpr int kTpPoissonMinLog2 = 6;  // a solve's sides also go down to 64
 constexpr int kTpMinLog2N1 = 7, kTpMaxLog2N1 = 13, kTpMinLog2N2 = 7, kTpMaxLog2N2 = 13;
 // Strip widths NP (column pairs per CTA) the two-pass column pass is built
 // for at half-length M: 64 to 512 threads (M/16 per pair), the strip's

@@ -25,7 +25,8 @@
 // Eq. (2d_idct_post).
 //
 // Workspace: N1 rows of N2/2 complex; rows [0, M) hold E (E'), rows [M, N1) O (O').
-// Supported: N1 in {128, ..., 8192}, N2 in {128, ..., 8192}.
+// Supported: N1 in {128, ..., 8192}, N2 in {128, ..., 8192}; the solves of
+// gbdct_poisson.cu also run sides of 64.
 #pragma once
 
 #include "dct2d_fs2_kernels.cuh"
@@ -54,7 +55,9 @@ struct TpColGeom {
   // faster than two at 128 registers (4096^2: 35.5 / 33.3 us vs 37.6 / 37.4),
   // the CTAs' strip loads overlapping the others' FFTs; else 128 registers
   static constexpr int MINB = THREADS == 256 ? 3 : (THREADS <= 512 ? 512 / THREADS : 1);
-  static constexpr bool VALID = THREADS >= 64 && THREADS <= 512 && SMEM <= 227 * 1024 - 256;
+  static constexpr bool VALID = THREADS >= (M == 32 ? 32 : 64) && THREADS <= 512 && SMEM <= 227 * 1024 - 256;
+  // widths the default rule can pick, which a Poisson solve runs
+  static constexpr bool POISSON = VALID && (THREADS <= 128 || NP == 2);
   // bulk tensor copy form: + 128-byte alignment slack, the mbarrier and a flag
   static constexpr size_t SMEM_TMA = SMEM + 256;
   static constexpr int HALF = M / 2;                    // rows of one reorder residue
@@ -71,8 +74,9 @@ __device__ __forceinline__ float4 soa_to_aos(soa::C2 y) { return make_float4(y.r
 // Forward (INV = false): reorder + E or O (blockIdx.y = parity of the
 // reordered row) -> workspace.  Inverse: E' or O' -> IDFT_M -> output rows
 // with the inverse reorder.
-template <int M, int NP, bool INV>
-__global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::MINB) k_tp_cols(Dct2dArgs a) {
+template <int M, int NP, bool INV, bool POIS>
+__global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::MINB)
+    k_tp_cols(Dct2dArgs a, PoissonArgs ps) {
   using G = TpColGeom<M, NP>;
   constexpr int TPS = G::TPS;
   extern __shared__ float4 stc[];
@@ -115,15 +119,18 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
       l2::st(W + (long long)k * hv, soa_to_aos(soa::unpack(s[G::NP * soa::pidx4(k)])), pol_keep);
     }
   } else {
-    float4* xo = reinterpret_cast<float4*>(a.out + (long long)blockIdx.z * a.out_bstride) + vcol;
+    const int vkind = POIS ? poisson_vkind(blockIdx.z) : a.vkind;
+    float* out = a.out + (long long)blockIdx.z * a.out_bstride;
+    if constexpr (POIS) out = blockIdx.z == 0 ? ps.out[0] : blockIdx.z == 1 ? ps.out[1] : ps.out[2];
+    float4* xo = reinterpret_cast<float4*>(out) + vcol;
 #pragma unroll 4
     for (int r = 0; r < 16; ++r) {
       const int m = g + TPS * r;
       const int row = reorder_src(2 * m + par, N1);
       float4 y = soa_to_aos(soa::unpack(s[G::NP * soa::pidx4(m)]));
-      if (a.vkind) {  // output signs: (-1)^(n1+n2) DST-II, (-1)^n2 IDCT_IDXST, (-1)^n1 IDXST_IDCT
-        const float sr = (a.vkind != 2 && (row & 1)) ? -1.f : 1.f;
-        const float sc = (a.vkind != 3) ? -sr : sr;
+      if (vkind) {  // output signs: (-1)^(n1+n2) DST-II, (-1)^n2 IDCT_IDXST, (-1)^n1 IDXST_IDCT
+        const float sr = (vkind != 2 && (row & 1)) ? -1.f : 1.f;
+        const float sc = (vkind != 3) ? -sr : sr;
         y = vsign(y, sr, sc);
       }
       l2::st(xo + (long long)row * hv, y, pol_stream);
@@ -151,9 +158,17 @@ __device__ __forceinline__ float4* align128(float4* p) {
   return reinterpret_cast<float4*>((a + 127) & ~uintptr_t(127));
 }
 
-template <int M, int NP, bool INV>
+// POIS: batch entry z of the workspace goes to output array z (its own map, one
+// array each), with that entry's kind.
+template <int N>
+struct ColMaps {
+  CUtensorMap x[N];  // input (forward) or output (inverse)
+  CUtensorMap w;     // workspace
+};
+
+template <int M, int NP, bool INV, bool POIS>
 __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::MINB)
-    k_tp_cols_tma(Dct2dArgs a, const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mw) {
+    k_tp_cols_tma(Dct2dArgs a, const __grid_constant__ ColMaps<POIS ? 3 : 1> maps) {
   using G = TpColGeom<M, NP>;
   constexpr int TPS = G::TPS, HALF = G::HALF, ZB = G::ZB;
   extern __shared__ float4 stt_raw[];
@@ -162,6 +177,10 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
   int* flag = reinterpret_cast<int*>(bar + 1);
   const int pi = threadIdx.x % NP, g = threadIdx.x / NP;
   const int par = blockIdx.y, b = blockIdx.z;
+  const CUtensorMap& mx = maps.x[POIS ? b : 0];
+  const CUtensorMap& mw = maps.w;
+  const int xb = POIS ? 0 : b;  // batch coordinate within the input or output map
+  const int vkind = POIS ? poisson_vkind(b) : a.vkind;
   const int x0 = blockIdx.x * NP * 4;  // first float column of the strip
   if (threadIdx.x == 0) {
     tma::bar_init(bar, 1);
@@ -173,8 +192,8 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
     const uint64_t pol = l2::evict_first();  // input streamed once / last use of the workspace
     if constexpr (!INV) {
       for (int z = 0; z < HALF; z += ZB) {
-        tma::load_4d(buf + z * NP, &mx, x0, 2 * par, z, b, bar, pol);
-        tma::load_4d(buf + (HALF + z) * NP, &mx, x0, 3 - 2 * par, z, b, bar, pol);
+        tma::load_4d(buf + z * NP, &mx, x0, 2 * par, z, xb, bar, pol);
+        tma::load_4d(buf + (HALF + z) * NP, &mx, x0, 3 - 2 * par, z, xb, bar, pol);
       }
     } else {
       for (int z = 0; z < M; z += ZB) tma::load_3d(buf + z * NP, &mw, x0, par * M + z, b, bar, pol);
@@ -213,12 +232,12 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
   __syncthreads();
   soa::stages<M, 16, INV, NP, INV ? 2 : 1>(s, g, a.tw1x);
   if constexpr (INV) {
-    if (a.vkind) {  // output signs: (-1)^(n1+n2) DST-II, (-1)^n2 IDCT_IDXST, (-1)^n1 IDXST_IDCT
+    if (vkind) {  // output signs: (-1)^(n1+n2) DST-II, (-1)^n2 IDCT_IDXST, (-1)^n1 IDXST_IDCT
 #pragma unroll 4
       for (int r = 0; r < 16; ++r) {
         const int pos = g + TPS * r;  // slots of the second half hold odd rows
-        const float sr = (a.vkind != 2 && pos >= HALF) ? -1.f : 1.f;
-        const float sc = (a.vkind != 3) ? -sr : sr;
+        const float sr = (vkind != 2 && pos >= HALF) ? -1.f : 1.f;
+        const float sc = (vkind != 3) ? -sr : sr;
         buf[NP * pos + pi] = vsign(buf[NP * pos + pi], sr, sc);
       }
     }
@@ -233,8 +252,8 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
     } else {
       const uint64_t pol = l2::evict_first();
       for (int z = 0; z < HALF; z += ZB) {
-        tma::store_4d(&mx, buf + z * NP, x0, 2 * par, z, b, pol);
-        tma::store_4d(&mx, buf + (HALF + z) * NP, x0, 3 - 2 * par, z, b, pol);
+        tma::store_4d(&mx, buf + z * NP, x0, 2 * par, z, xb, pol);
+        tma::store_4d(&mx, buf + (HALF + z) * NP, x0, 3 - 2 * par, z, xb, pol);
       }
     }
     tma::commit_group();
@@ -361,8 +380,56 @@ __device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a
 // buffer (17 L bytes) holds the 16 L bytes of the rows until the first FFT
 // stage overwrites it.  Device buffers only.
 
-template <int L, bool MAPPED, bool STAGED, bool NARROW>
-__global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>::MINB) k_tp_rows_inv(Dct2dArgs a) {
+// The scaled reads of a Poisson solve: RowReads' value times the eigenvalue
+// denominator and (entry 1) the row's wu or (entry 2) the column's wv.
+template <bool STAGED>
+struct PoissonReads {
+  RowReads<STAGED> r;
+  const float *ia, *ib;  // the denominators of the two rows
+  const float* wv;       // entry 2 only
+  float ua, ub;          // wu of the two rows (entry 1), else 1
+  __device__ __forceinline__ PoissonReads(const RowReads<STAGED>& reads, const InvRows& src, const float* spectrum,
+                                          const PoissonArgs& ps, int n1, int L, int z)
+      : r(reads), ia(src.ra ? ps.inv + (src.ra - spectrum) : nullptr), ib(ps.inv + (src.rb - spectrum)),
+        wv(z == 2 ? ps.w + n1 : nullptr), ua(1.f), ub(1.f) {
+    if (z == 1) {
+      if (src.ra) ua = __ldg(ps.w + (src.ra - spectrum) / L);
+      ub = __ldg(ps.w + (src.rb - spectrum) / L);
+    }
+  }
+  __device__ __forceinline__ bool has_a() const { return ia != nullptr; }
+  __device__ __forceinline__ float a(int c) const {
+    return r.a(c) * __ldg(ia + c) * (wv ? __ldg(wv + c) : ua);
+  }
+  __device__ __forceinline__ float b(int c) const {
+    return r.b(c) * __ldg(ib + c) * (wv ? __ldg(wv + c) : ub);
+  }
+};
+
+// Preprocess of a group from its rows' reads (POIS: scaled).
+template <int L, bool MAPPED, bool POIS, bool STAGED>
+__device__ __forceinline__ int tp_inv_pre(const Dct2dArgs& a, const PoissonArgs& ps, const RowReads<STAGED>& A,
+                                          const RowReads<STAGED>& B, const InvRows& srcA, const InvRows& srcB,
+                                          const float* C, int vkind, int c, int kb, bool first, int g, soa::C2* v) {
+  auto pre = [&](const auto& ra, const auto& rb) {
+    return rowp::warp_has_first<fft_tps(L)>(first)
+               ? inv_pre_x2<L, MAPPED, true>(a, ra, rb, vkind, c, kb, first, g, v)
+               : inv_pre_x2<L, MAPPED, false>(a, ra, rb, vkind, c, kb, false, g, v);
+  };
+  if constexpr (POIS) {
+    const int z = blockIdx.z;
+    return pre(PoissonReads<STAGED>(A, srcA, C, ps, a.n1, L, z), PoissonReads<STAGED>(B, srcB, C, ps, a.n1, L, z));
+  } else {
+    return pre(A, B);
+  }
+}
+
+// POIS: blockIdx.z counts the three inverses of a Poisson solve, which read the
+// one spectrum; its scaling is applied to the values as they are read (the
+// products rounded in the order a inv, then times wu or wv).
+template <int L, bool MAPPED, bool STAGED, bool NARROW, bool POIS>
+__global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>::MINB)
+    k_tp_rows_inv(Dct2dArgs a, PoissonArgs ps) {
   using R = TpRows<L, NARROW>;
   extern __shared__ float4 sxti[];
   const int pi = threadIdx.x / R::TPS, g = threadIdx.x % R::TPS;
@@ -371,8 +438,9 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
   const int c = blockIdx.x * R::NP + pi;
   const bool first = (c == 0);
   const int kb = tp_item_b(c, M);
-  const float* C = a.in + (long long)blockIdx.z * a.in_bstride;
-  const InvRows A = inv_rows_of(a, C, c, L), B = inv_rows_of(a, C, kb, L);
+  const float* C = a.in + (POIS ? 0 : (long long)blockIdx.z * a.in_bstride);
+  const int vkind = POIS ? poisson_vkind(blockIdx.z) : a.vkind;
+  const InvRows A = inv_rows_of(a, C, c, L, vkind), B = inv_rows_of(a, C, kb, L, vkind);
   soa::C2 v[16];
   int t;
   if constexpr (STAGED) {
@@ -406,18 +474,14 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
     __syncthreads();
     if (!*flag) return;
     tma::test_wait(bar, 0);  // completed: every thread observes the copied rows
-    const InvRows As{A.ra ? st : nullptr, st + L}, Bs{B.ra ? st + 2 * L : nullptr, st + 3 * L};
-    if (rowp::warp_has_first<R::TPS>(first))
-      t = inv_pre_x2<L, MAPPED, true, true>(a, As, Bs, c, kb, first, g, v);
-    else
-      t = inv_pre_x2<L, MAPPED, false, true>(a, As, Bs, c, kb, false, g, v);
+    const RowReads<true> As{{A.ra ? st : nullptr, st + L}, 0}, Bs{{B.ra ? st + 2 * L : nullptr, st + 3 * L}, 0};
+    t = tp_inv_pre<L, MAPPED, POIS>(a, ps, As, Bs, A, B, C, vkind, c, kb, first, g, v);
     rowp::group_sync<R::TPS>(pi);  // the first stage overwrites the staged rows
   } else {
     pdl::wait_prior_grid();
-    if (rowp::warp_has_first<R::TPS>(first))
-      t = inv_pre_x2<L, MAPPED, true>(a, A, B, c, kb, first, g, v);
-    else
-      t = inv_pre_x2<L, MAPPED, false>(a, A, B, c, kb, false, g, v);
+    const uint64_t pol = l2::evict_first();  // the input is streamed in
+    t = tp_inv_pre<L, MAPPED, POIS>(a, ps, RowReads<false>{A, pol}, RowReads<false>{B, pol}, A, B, C, vkind, c, kb,
+                                    first, g, v);
   }
   soa::first_stage<L, true>(v, s, t);
   rowp::stages_to_regs<L, 16, true, false>(s, g, pi, a.tw2x, v);

@@ -10,6 +10,7 @@
 #include "dct2d_launch.cuh"
 #include "dct_axis0.cuh"
 #include "gemm_path.cuh"
+#include "poisson_path.cuh"
 
 using gbdct::Dct2dArgs;
 
@@ -252,7 +253,7 @@ static gbdct_status run_plan(gbdct_plan_t p, bool inverse, int step, const void*
 }
 
 static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims, int64_t batch, int kind,
-                                int dtype, const char* force);
+                                int dtype, const char* force, bool poisson = false);
 
 static gbdct_status create_3d(gbdct_plan_t* out, const int64_t* dims, int64_t batch, int kind, int dtype,
                               const char* force) {
@@ -370,8 +371,10 @@ gbdct_status gbdct_plan_create_family(gbdct_plan_t* out, int ndim, const int64_t
 // force: a family name that must be used (UNSUPPORTED if it does not support
 // the shape), or NULL for the default choice (GBDCT_KERNEL_FAMILY may override
 // it when the named family supports the shape).
+// poisson: the plan of a fused Poisson solve, in the two-pass family only
+// (sides of 64 included).
 static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims, int64_t batch, int kind,
-                                int dtype, const char* force) {
+                                int dtype, const char* force, bool poisson) {
   if (!out || !dims || batch < 1) return GBDCT_ERR_INVALID_ARG;
   if (ndim < 1 || ndim > 3) return GBDCT_ERR_INVALID_ARG;
   for (int i = 0; i < ndim; ++i)
@@ -426,8 +429,10 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
                     p->lg2 >= gbdct::kPairMinLog2 && p->lg2 <= gbdct::kPairMaxLog2;
   const bool fs2 = p->lg1 >= gbdct::kFs2MinLog2N1 && p->lg1 <= gbdct::kFs2MaxLog2N1 &&
                    p->lg2 >= gbdct::kFs2MinLog2N2 && p->lg2 <= gbdct::kFs2MaxLog2N2;
-  const bool tp = p->lg1 >= gbdct::kTpMinLog2N1 && p->lg1 <= gbdct::kTpMaxLog2N1 &&
-                  p->lg2 >= gbdct::kTpMinLog2N2 && p->lg2 <= gbdct::kTpMaxLog2N2;
+  const int tp_min1 = poisson ? gbdct::kTpPoissonMinLog2 : gbdct::kTpMinLog2N1;
+  const int tp_min2 = poisson ? gbdct::kTpPoissonMinLog2 : gbdct::kTpMinLog2N2;
+  const bool tp = p->lg1 >= tp_min1 && p->lg1 <= gbdct::kTpMaxLog2N1 && p->lg2 >= tp_min2 &&
+                  p->lg2 <= gbdct::kTpMaxLog2N2;
   // a strip width the two-pass column pass is built for at this shape
   const bool tp_np_ok = tp && strip_np > 0 && gbdct::tp_strip_ok(n1 / 2, n2, strip_np);
   // Default: the two-pass family for N1 <= 4096, the four-step family where
@@ -454,6 +459,10 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
       return GBDCT_ERR_UNSUPPORTED;
     }
     p->family = chosen < 0 ? before : chosen;
+  }
+  if (poisson && (p->family != FAM_TP || strip_np)) {
+    delete p;
+    return GBDCT_ERR_UNSUPPORTED;
   }
   const bool two_pass = p->family == FAM_TP;
   // a two-pass plan also carries the four-step configuration: full transforms
@@ -574,6 +583,7 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   } else if (p->family == FAM_TP) {
     e = gbdct::run_tp(p->lg1, p->lg2, false, a, 1, 0, true);
     if (e == cudaSuccess && p->host_fs2) e = gbdct::run_fs2(p->lg1, p->lg2, false, a, 1, 0, true);
+    if (e == cudaSuccess && poisson) e = gbdct::run_tp_poisson(p->lg1, p->lg2, a, gbdct::PoissonArgs{}, 0, true);
   } else if (p->family == FAM_PAIR) {
     e = gbdct::run_fwd_cols2(p->lg1, a, 1, 1, 0, true);
     if (e == cudaSuccess) e = gbdct::run_inv_cols2(p->lg1, a, 1, 1, 0, true);
@@ -714,6 +724,43 @@ static gbdct_status exec_core(gbdct_plan_t p, const void* in, void* out, cudaStr
   }
   return cuda_status(e);
 }
+
+}  // extern "C"
+
+namespace gbdct {
+
+gbdct_status poisson_plan_create(gbdct_plan_t* out, const int64_t* dims) {
+  return create_impl(out, 2, dims, 3, GBDCT_DCT2, GBDCT_F32, nullptr, true);
+}
+
+gbdct_status poisson_plan_solve(gbdct_plan_t p, const void* rho, void* const* out, const float* w, const float* inv,
+                                cudaStream_t s) {
+  const void* io[4] = {rho, out[0], out[1], out[2]};
+  bool dev[4];
+  for (int i = 0; i < 4; ++i) {
+    if ((uintptr_t)io[i] & 15u) return GBDCT_ERR_INVALID_ARG;
+    const int k = pointer_kind(io[i], p->device, s);
+    if (k == PTR_NONE) return GBDCT_ERR_INVALID_ARG;
+    dev[i] = k == PTR_DEVICE;
+  }
+  Dct2dArgs a = p->args;
+  a.polls = p->wait_polls;
+  // forward into psi, which the inverse row pass reads and the column pass overwrites
+  a.in = static_cast<const float*>(rho);
+  a.out = static_cast<float*>(out[0]);
+  a.io_dev = dev[0] && dev[1];
+  cudaError_t e = !a.io_dev && p->host_fs2 ? run_fs2(p->lg1, p->lg2, false, a, 1, s, false)
+                                           : run_tp(p->lg1, p->lg2, false, a, 1, s, false);
+  if (e != cudaSuccess) return cuda_status(e);
+  PoissonArgs ps{w, inv, {static_cast<float*>(out[0]), static_cast<float*>(out[1]), static_cast<float*>(out[2])}};
+  a.in = a.out;
+  a.io_dev = dev[1] && dev[2] && dev[3];
+  return cuda_status(run_tp_poisson(p->lg1, p->lg2, a, ps, s, false));
+}
+
+}  // namespace gbdct
+
+extern "C" {
 
 gbdct_status gbdct_exec_forward(gbdct_plan_t plan, const void* in, void* out, void* stream) {
   return exec2d(plan, in, out, stream, false, -1);

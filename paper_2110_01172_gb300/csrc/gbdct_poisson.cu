@@ -4,8 +4,18 @@
 // field xi0 = IDXST_IDCT(a wu / (wu^2 + wv^2)), xi1 = IDCT_IDXST(a wv / (...)),
 // with wu = pi u / N1, wv = pi v / N2 and the DC term zeroed (the paper's
 // "scaled electric potential a1, a2"; the scaling is the grid-unit
-// eigenfrequency reading of the cosine basis).  The transforms are the
-// library's own plans; one kernel applies the three spectral scalings.
+// eigenfrequency reading of the cosine basis).
+//
+// Where the two-pass family applies (sides 64..4096, and 8192 x 64 / 128) a
+// solve is four launches: the forward's column and row pass, then one row pass
+// and one column pass over the three inverses as a batch, the spectral scalings
+// applied to the spectrum as the row pass reads it.  Small solves are bound by
+// launches and by too few CTAs per launch (512^2: 128 per inverse), large ones
+// by the array passes; separate transforms take nine launches (13 with a side
+// of 64, whose default family is not folded) and the scaling seven more passes
+// over the array.  GPU time per solve, separate -> fused: 64^2 48.5 -> 17.0 us,
+// 64 x 2048 62.5 -> 17.6, 512^2 32.7 -> 18.0, 1024^2 41.4 -> 25.3, 2048^2 92.7 -> 74.7.
+// Other shapes run the library's own plans around one scaling kernel.
 // The eigenvalue denominators 1 / (wu^2 + wv^2) are evaluated in FP64 once,
 // when the solver is created, and rounded once into an FP32 table that every
 // solve reads; wu and wv are FP64 values rounded once as well.
@@ -15,9 +25,11 @@
 #include <new>
 
 #include "../../include/gbdct.h"
+#include "poisson_path.cuh"
 
 struct gbdct_poisson_s {
   int n1, n2, device;
+  gbdct_plan_t fused;            // the fused solve, or null:
   gbdct_plan_t fwd, fld0, fld1;  // DCT2 (forward and potential inverse), IDXST_IDCT, IDCT_IDXST
   float* w;    // wu[N1], wv[N2]
   float* inv;  // 1 / (wu^2 + wv^2) per (u, v), 0 at (0, 0): N1 x N2
@@ -71,6 +83,7 @@ struct DeviceGuard {
 
 void destroy(gbdct_poisson_s* p) {
   if (!p) return;
+  gbdct_plan_destroy(p->fused);
   gbdct_plan_destroy(p->fwd);
   gbdct_plan_destroy(p->fld0);
   gbdct_plan_destroy(p->fld1);
@@ -88,9 +101,12 @@ gbdct_status gbdct_poisson_create(gbdct_poisson_t* out, int64_t n1, int64_t n2) 
   const int64_t dims[2] = {n1, n2};
   gbdct_poisson_s* p = new (std::nothrow) gbdct_poisson_s();
   if (!p) return GBDCT_ERR_OOM;
-  gbdct_status st = gbdct_plan_create(&p->fwd, 2, dims, GBDCT_DCT2, GBDCT_F32);
-  if (st == GBDCT_OK) st = gbdct_plan_create(&p->fld0, 2, dims, GBDCT_IDXST_IDCT, GBDCT_F32);
-  if (st == GBDCT_OK) st = gbdct_plan_create(&p->fld1, 2, dims, GBDCT_IDCT_IDXST, GBDCT_F32);
+  gbdct_status st = gbdct::poisson_plan_create(&p->fused, dims);
+  if (st == GBDCT_ERR_UNSUPPORTED) {
+    st = gbdct_plan_create(&p->fwd, 2, dims, GBDCT_DCT2, GBDCT_F32);
+    if (st == GBDCT_OK) st = gbdct_plan_create(&p->fld0, 2, dims, GBDCT_IDXST_IDCT, GBDCT_F32);
+    if (st == GBDCT_OK) st = gbdct_plan_create(&p->fld1, 2, dims, GBDCT_IDCT_IDXST, GBDCT_F32);
+  }
   if (st != GBDCT_OK) {
     destroy(p);
     return st;
@@ -121,6 +137,10 @@ gbdct_status gbdct_poisson_solve(gbdct_poisson_t p, const void* rho, void* psi, 
   if (psi == xi0 || psi == xi1 || xi0 == xi1) return GBDCT_ERR_INVALID_ARG;
   DeviceGuard guard(p->device);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  if (p->fused) {
+    void* const out[3] = {psi, xi0, xi1};
+    return gbdct::poisson_plan_solve(p->fused, rho, out, p->w, p->inv, s);
+  }
   gbdct_status st = gbdct_exec_forward(p->fwd, rho, psi, stream);
   if (st != GBDCT_OK) return st;
   const dim3 grid((p->n2 + 255) / 256, p->n1);
@@ -135,7 +155,8 @@ gbdct_status gbdct_poisson_solve(gbdct_poisson_t p, const void* rho, void* psi, 
 
 size_t gbdct_poisson_workspace_bytes(gbdct_poisson_t p) {
   if (!p) return 0;
-  return gbdct_plan_workspace_bytes(p->fwd) + gbdct_plan_workspace_bytes(p->fld0) + gbdct_plan_workspace_bytes(p->fld1) +
+  return gbdct_plan_workspace_bytes(p->fused) + gbdct_plan_workspace_bytes(p->fwd) +
+         gbdct_plan_workspace_bytes(p->fld0) + gbdct_plan_workspace_bytes(p->fld1) +
          (size_t)p->n1 * p->n2 * sizeof(float) /* denominators */ + (size_t)(p->n1 + p->n2) * sizeof(float);
 }
 

@@ -1,0 +1,38 @@
+// pass_tp_rows_fwd.cu - forward row pass of the two-pass family (radix-2 column
+// step folded into the loads).
+#include "tp_rows_launch.cuh"
+
+namespace gbdct {
+namespace {
+
+template <int L, bool NARROW, bool GENERAL>
+cudaError_t launch_k(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
+  using R = TpRows<L, NARROW>;
+  const auto k = k_tp_rows_fwd<L, NARROW, GENERAL>;
+  if (prepare) return tp_smem_limit(reinterpret_cast<const void*>(k), R::SMEM);
+  if ((a.n1 / 4) % R::NP) return cudaErrorInvalidValue;
+  return pdl::launch(k, dim3(a.n1 / 4 / R::NP, 1, batch), dim3(R::THREADS), R::SMEM, s, a);
+}
+
+template <int L>
+cudaError_t launch(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
+  if (prepare) {
+    cudaError_t e = launch_k<L, false, false>(a, batch, s, true);
+    if (e == cudaSuccess) e = launch_k<L, false, true>(a, batch, s, true);
+    if (e == cudaSuccess) e = launch_k<L, true, false>(a, batch, s, true);
+    if (e == cudaSuccess) e = launch_k<L, true, true>(a, batch, s, true);
+    return e;
+  }
+  const bool general = a.vkind == 1 || a.thresh > 0.f;
+  if (tp_rows_narrow<L>(a, batch))
+    return general ? launch_k<L, true, true>(a, batch, s, false) : launch_k<L, true, false>(a, batch, s, false);
+  return general ? launch_k<L, false, true>(a, batch, s, false) : launch_k<L, false, false>(a, batch, s, false);
+}
+
+}  // namespace
+
+cudaError_t run_tp_rows_fwd(int lg2, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
+  GBDCT_TP_ROWS_SWITCH(lg2, launch, a, batch, s, prepare);
+}
+
+}  // namespace gbdct

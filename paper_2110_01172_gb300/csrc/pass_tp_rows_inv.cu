@@ -1,0 +1,51 @@
+// pass_tp_rows_inv.cu - inverse row pass of the two-pass family (radix-2
+// column step folded into the stores).
+#include "tp_rows_launch.cuh"
+
+namespace gbdct {
+namespace {
+
+template <int L, bool NARROW, bool MAPPED, bool STAGED>
+cudaError_t launch_k(const Dct2dArgs& a, const PoissonArgs& ps, int batch, cudaStream_t s, bool prepare) {
+  using R = TpRows<L, NARROW>;
+  constexpr size_t SMEM = STAGED ? R::SMEM_STAGED : R::SMEM;
+  const auto k = k_tp_rows_inv<L, MAPPED, STAGED, NARROW, false>;
+  if (prepare) return tp_smem_limit(reinterpret_cast<const void*>(k), SMEM);
+  if ((a.n1 / 4) % R::NP) return cudaErrorInvalidValue;
+  return pdl::launch(k, dim3(a.n1 / 4 / R::NP, 1, batch), dim3(R::THREADS), SMEM, s, a, ps);
+}
+
+template <int L, bool NARROW>
+cudaError_t launch_n(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
+  const PoissonArgs none{};
+  if (prepare) {
+    cudaError_t e = launch_k<L, NARROW, false, false>(a, none, batch, s, true);
+    if (e == cudaSuccess) e = launch_k<L, NARROW, false, true>(a, none, batch, s, true);
+    if (e == cudaSuccess) e = launch_k<L, NARROW, true, false>(a, none, batch, s, true);
+    if (e == cudaSuccess) e = launch_k<L, NARROW, true, true>(a, none, batch, s, true);
+    return e;
+  }
+  // device input: the rows are staged by bulk copies; host-mapped input: read directly
+  if (a.vkind == 1 || a.vkind == 2)
+    return a.io_dev ? launch_k<L, NARROW, true, true>(a, none, batch, s, false)
+                    : launch_k<L, NARROW, true, false>(a, none, batch, s, false);
+  return a.io_dev ? launch_k<L, NARROW, false, true>(a, none, batch, s, false)
+                  : launch_k<L, NARROW, false, false>(a, none, batch, s, false);
+}
+
+template <int L>
+cudaError_t launch(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
+  if (prepare) {
+    const cudaError_t e = launch_n<L, false>(a, batch, s, true);
+    return e == cudaSuccess ? launch_n<L, true>(a, batch, s, true) : e;
+  }
+  return tp_rows_narrow<L>(a, batch) ? launch_n<L, true>(a, batch, s, false) : launch_n<L, false>(a, batch, s, false);
+}
+
+}  // namespace
+
+cudaError_t run_tp_rows_inv(int lg2, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
+  GBDCT_TP_ROWS_SWITCH(lg2, launch, a, batch, s, prepare);
+}
+
+}  // namespace gbdct

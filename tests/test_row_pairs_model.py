@@ -7,7 +7,7 @@ or in one warp, so that each pair of columns meets in registers exactly once.
 
 import pytest
 
-LENGTHS = [128, 256, 512, 1024, 2048, 4096, 8192]
+LENGTHS = [64, 128, 256, 512, 1024, 2048, 4096, 8192]
 
 
 def radix(L, ns):
