@@ -165,7 +165,10 @@ int gbdct_plan_launches_per_exec(gbdct_plan_t plan);
  * and N2 in 256..16384, three launches; pair: both sides in 16..8192; seq:
  * any supported size), and the environment variable
  * GBDCT_KERNEL_FAMILY=seq|pair|fs2|tp, read at plan creation, forces a family
- * when it supports the shape (for testing and comparison). */
+ * when it supports the shape (for testing and comparison).  Default plans of
+ * small shapes (both sides from 32, N1*N2 <= 16384; 128 x 128 for larger
+ * batches) run each transform in one launch and without a workspace, under
+ * their family's name. */
 const char* gbdct_plan_kernel_family(gbdct_plan_t plan);
 
 /* Reports (and clears) a failure recorded on the device by the plan's

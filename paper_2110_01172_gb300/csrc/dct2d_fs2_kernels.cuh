@@ -722,11 +722,12 @@ __device__ __forceinline__ void fwd_split_x2(const float2* __restrict__ za, cons
 }
 
 // Forward postprocess of both items (rowp::fwd_post) into the output rows k1,
-// N1-k1 (lane a; rows 0 and N1/2 of the packed item) and kb, N1-kb (lane b).
-// GENERAL: plans with the DST-II order or a magnitude threshold.
-template <int L, bool GENERAL, bool FIRST>
-__device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, float* y, int k1, int kb, bool packed,
-                                            int g) {
+// N1-k1 (lane a; rows 0 and N1/2 of the packed item) and kb, N1-kb (lane b) of
+// y, `stride` floats apart.  GENERAL: plans with the DST-II order or a magnitude
+// threshold.
+template <int L, bool GENERAL, bool FIRST, bool SMEM>
+__device__ __forceinline__ void fwd_post_rows(soa::C2* v, const Dct2dArgs& a, float* y, long long stride, int k1,
+                                              int kb, bool packed, int g) {
   const int N1 = a.n1;
   const float2 fa0 = __ldg(a.fa + k1), fa1 = __ldg(a.fa + kb);
   // 1/2 of the split folded into the a-twiddle (not for the packed item)
@@ -734,15 +735,23 @@ __device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, floa
   const float2 avi = make_float2(packed ? 0.f : 0.5f * fa0.y, 0.5f * fa1.y);
   const bool rev = GENERAL && a.vkind == 1;  // DST-II: output (k1, k2) goes to (N1-1-k1, N2-1-k2)
   const int kma = row_mirror(k1, N1), kmb = row_mirror(kb, N1);
-  rowp::FwdOut<L, GENERAL> out;
-  out.a0 = y + (long long)(rev ? N1 - 1 - k1 : k1) * L;
-  out.a1 = y + (long long)(rev ? N1 - 1 - kma : kma) * L;
-  out.b0 = y + (long long)(rev ? N1 - 1 - kb : kb) * L;
-  out.b1 = y + (long long)(rev ? N1 - 1 - kmb : kmb) * L;
+  rowp::FwdOut<L, GENERAL, SMEM> out;
+  out.a0 = y + (rev ? N1 - 1 - k1 : k1) * stride;
+  out.a1 = y + (rev ? N1 - 1 - kma : kma) * stride;
+  out.b0 = y + (rev ? N1 - 1 - kb : kb) * stride;
+  out.b1 = y + (rev ? N1 - 1 - kmb : kmb) * stride;
   out.pol = l2::evict_first();  // the output is streamed out
   out.eps = a.thresh;           // magnitude threshold of Section V-A, Eq. image-compression (0: off)
   out.rev = rev;
-  rowp::fwd_post<L, FIRST, GENERAL>(v, out, avr, avi, a.fb4, g, packed);
+  rowp::fwd_post<L, FIRST>(v, out, avr, avi, a.fb4, g, packed);
+}
+template <int L, bool GENERAL, bool SMEM>
+__device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, float* y, long long stride, int k1, int kb,
+                                            bool packed, int g) {
+  if (rowp::warp_has_first<fft_tps(L)>(packed))
+    fwd_post_rows<L, GENERAL, true, SMEM>(v, a, y, stride, k1, kb, packed, g);
+  else
+    fwd_post_rows<L, GENERAL, false, SMEM>(v, a, y, stride, k1, kb, false, g);
 }
 
 // Row FFT of both items from registers (v: points t + TPS j of the thread's
@@ -750,14 +759,10 @@ __device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, floa
 template <int L, bool GENERAL>
 __device__ __forceinline__ void fwd_fft_post_x2(soa::C2* v, float4* s, const Dct2dArgs& a, float* y, int k1, int kb,
                                                 bool packed, int t, int g, int group) {
-  constexpr int TPS = fft_tps(L);
   soa::first_stage<L, false>(v, s, t);
   rowp::stages_to_regs<L, 16, false, true>(s, g, group, a.tw2x, v);
   pdl::launch_dependents();
-  if (rowp::warp_has_first<TPS>(packed))
-    fwd_post_x2<L, GENERAL, true>(v, a, y, k1, kb, packed, g);
-  else
-    fwd_post_x2<L, GENERAL, false>(v, a, y, k1, kb, false, g);
+  fwd_post_x2<L, GENERAL, false>(v, a, y, L, k1, kb, packed, g);
 }
 
 template <int L, bool GENERAL>
@@ -791,6 +796,7 @@ struct InvRows {
   const float* rb;  // row of c3 / c2
 };
 
+// Input rows of item k (rows L floats apart).
 __device__ __forceinline__ InvRows inv_rows_of(const Dct2dArgs& a, const float* C, int k, int L, int vkind) {
   const int N1 = a.n1;
   const int kmir = row_mirror(k, N1);

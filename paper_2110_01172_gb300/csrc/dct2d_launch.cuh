@@ -83,6 +83,11 @@ inline bool tp_strip_ok(int M, int n2, int np) {
   return np >= 1 && threads >= 64 && threads <= 512 && smem <= 227 * 1024 - 256 && (n2 / 4) % np == 0;
 }
 
+// Whole small transforms in one launch: both sides from 32, N1 * N2 <= 16384.
+cudaError_t run_small_fwd(int log2N1, int log2N2, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
+cudaError_t run_small_inv(int log2N1, int log2N2, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
+constexpr int kSmallMinLog2 = 5, kSmallMaxLog2 = 14;
+
 constexpr int kPairMinLog2 = 4;
 constexpr int kPairMaxLog2 = 13;
 

@@ -288,18 +288,20 @@ struct TpRows {
 };
 
 // The thread's points of both items in v, straight from the group's four
-// workspace rows (w1, w2: the radix-2 twiddles on O[c] and O[kb]).
-template <int L, bool FIRST>
+// workspace rows (SMEM: in shared memory; w1, w2: the radix-2 twiddles on O[c]
+// and O[kb]).
+template <int L, bool FIRST, bool SMEM = false>
 __device__ __forceinline__ void tp_fwd_load(const float2* e1r, const float2* o1r, const float2* e2r, const float2* o2r,
                                             float2 w1, float2 w2, bool first, int t, soa::C2* v) {
   constexpr int TPS = fft_tps(L);
   constexpr int MASK = rowp::rev_lane_mask<TPS>();
   const uint64_t pol = l2::evict_first();  // last use of the workspace
+  auto ld = [&](const float2* r) { return SMEM ? *r : l2::ld_once(r, pol); };
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int p = t + TPS * j;
-    const float2 e1 = l2::ld_once(e1r + p, pol), e2 = l2::ld_once(e2r + p, pol);
-    const float2 o1 = cmul(l2::ld_once(o1r + p, pol), w1), o2 = cmul(l2::ld_once(o2r + p, pol), w2);
+    const float2 e1 = ld(e1r + p), e2 = ld(e2r + p);
+    const float2 o1 = cmul(ld(o1r + p), w1), o2 = cmul(ld(o2r + p), w2);
     const float2 P = cadd(e1, o1), Q = csub(e1, o1), Rr = cadd(e2, o2), S = csub(e2, o2);
     // (z_a, m_a, z_b, m_b) = (V[c], V[N1-c], V[M-c], V[M+c]); first group:
     // (V[0], V[M], V[M/2], V[3M/2])
@@ -346,14 +348,15 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
 //   E'[M-c] = V[M-c] + V[N1-c], O'[M-c] = w (V[N1-c] - V[M-c])
 // and for the first group E'[0], O'[0] from V[0] +- V[M], E'[M/2] = V[M/2] +
 // V[3M/2], O'[M/2] = i (V[M/2] - V[3M/2]).
-template <int L>
-__device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a, float2* Zw, int c, int kb, bool first,
-                                            int g) {
+// Rows of Zw are `stride` complex values apart (SMEM: in shared memory).
+template <int L, bool SMEM>
+__device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a, float2* Zw, long long stride, int c,
+                                            int kb, bool first, int g) {
   const int M = a.n1 / 2;
-  float2* e1r = Zw + (long long)c * (L / 2);
-  float2* o1r = Zw + (long long)(M + c) * (L / 2);
-  float2* e2r = Zw + (long long)kb * (L / 2);
-  float2* o2r = Zw + (long long)(M + kb) * (L / 2);
+  float2* e1r = Zw + c * stride;
+  float2* o1r = Zw + (M + c) * stride;
+  float2* e2r = Zw + kb * stride;
+  float2* o2r = Zw + (M + kb) * stride;
   const float2 cw = __ldg(a.r2w + c);
   const uint64_t pol = l2::evict_last();  // read again by the column pass
   rowp::inv_pairs<L>(v, g, [&](int base, int off, const soa::C2& u, const soa::C2& w) {
@@ -367,10 +370,16 @@ __device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a
     const float2 d2 = csub(zb0, x2);
     const float2 o1 = first ? d1 : cmulc(d1, cw);
     const float2 o2 = first ? make_float2(-d2.y, d2.x) : cmul(make_float2(-d2.x, -d2.y), cw);
-    l2::st(e1r + base + off, cadd(za0, x1), pol);
-    l2::st(o1r + base + off, o1, pol);
-    l2::st(e2r + base + off, cadd(zb0, x2), pol);
-    l2::st(o2r + base + off, o2, pol);
+    auto st = [&](float2* p, float2 z) {
+      if constexpr (SMEM)
+        *p = z;
+      else
+        l2::st(p, z, pol);
+    };
+    st(e1r + base + off, cadd(za0, x1));
+    st(o1r + base + off, o1);
+    st(e2r + base + off, cadd(zb0, x2));
+    st(o2r + base + off, o2);
   });
 }
 
@@ -488,9 +497,9 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
   pdl::launch_dependents();
   float2* Zw = a.work + (long long)blockIdx.z * a.work_bstride;
   if (rowp::warp_has_first<R::TPS>(first))
-    tp_inv_pair<L>(v, a, Zw, c, kb, first, g);
+    tp_inv_pair<L, false>(v, a, Zw, L / 2, c, kb, first, g);
   else
-    tp_inv_pair<L>(v, a, Zw, c, kb, false, g);
+    tp_inv_pair<L, false>(v, a, Zw, L / 2, c, kb, false, g);
 }
 
 }  // namespace gbdct

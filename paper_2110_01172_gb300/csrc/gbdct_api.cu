@@ -30,6 +30,7 @@ struct gbdct_plan_s {
   int family;          // kernel family (FAM_*)
   float2* fstw;        // four-step twiddles W_N1^{n1a k1b} (FAM_FS2)
   int* err;            // device error word (bounded waits that gave up)
+  bool one_launch;     // small default plan: the whole transform in one launch (dct2d_small.cuh)
   bool host_fs2;       // two-pass plan that runs full transforms on host-mapped buffers with the four-step kernels
   int nsm;             // multiprocessors of the plan's device
   float* tmp;          // variant kinds: staging array (batch * N1 * N2 floats)
@@ -59,9 +60,9 @@ namespace {
 //   FAM_SEQ  one sequence per thread group, any supported size
 enum { FAM_SEQ = 0, FAM_PAIR = 1, FAM_FS2 = 5, FAM_TP = 6 };
 
-// Families whose kernels fold the other kinds' index/sign maps into their
+// Plans whose kernels fold the other kinds' index/sign maps into their
 // loads and stores (no map kernels, no staging array).
-bool folds_maps(int family) { return family == FAM_FS2 || family == FAM_TP; }
+bool folds_maps(const gbdct_plan_s* p) { return p->family == FAM_FS2 || p->family == FAM_TP || p->one_launch; }
 
 // Radix-2 twiddles of the two-pass family: out[k] = W_N1^k, k in [0, N1/2], FP64.
 __global__ void k_gen_r2_twiddles(float2* out, int n1) {
@@ -464,13 +465,25 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
     delete p;
     return GBDCT_ERR_UNSUPPORTED;
   }
-  const bool two_pass = p->family == FAM_TP;
+  // Small shapes of a default plan (no family asked for) run in one launch
+  // whatever their family; a forced family keeps its own kernels.  Where the
+  // two-pass family applies (128 x 128) its many CTAs per transform are faster
+  // until there is a transform for half of the SMs (forward, two-pass vs one
+  // launch: batch 1 5.3 vs 6.4 us, 16 5.5 vs 6.4, 203 13.5 vs 10.8, 2048 103 vs 73);
+  // against the pair family one launch won at every batch.
+  if (cudaDeviceGetAttribute(&p->nsm, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
+    delete p;
+    return GBDCT_ERR_CUDA;
+  }
+  p->one_launch = !fname && !poisson && p->lg1 >= gbdct::kSmallMinLog2 && p->lg2 >= gbdct::kSmallMinLog2 &&
+                  p->lg1 + p->lg2 <= gbdct::kSmallMaxLog2 && (!tp || 2 * batch >= p->nsm);
+  const bool two_pass = p->family == FAM_TP || p->one_launch;  // tables of the two-pass kernels
   // a two-pass plan also carries the four-step configuration: full transforms
   // on host-mapped buffers run the four-step kernels, whose first and last
   // launches read and write whole 1 KB row segments (the two-pass column
   // pass's 32-byte row pieces cross the host link poorly), where the
   // four-step family supports the shape
-  p->host_fs2 = two_pass && fs2;
+  p->host_fs2 = two_pass && fs2 && !p->one_launch;
   const bool four_step = p->family == FAM_FS2 || p->host_fs2;
   const bool two_item_rows = four_step || two_pass;  // row passes on the SoA engine (float4 twiddles)
   p->pmax = 16;
@@ -508,10 +521,10 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   float2* r2w = two_pass ? ib + tb + tf + tx + 3 * tm : nullptr;
   p->err = reinterpret_cast<int*>(ib + tb + tf + tx + 3 * tm + tr);
 
-  p->work_bytes = (size_t)batch * (size_t)(n1 / 2) * (size_t)n2 * sizeof(float2);
-  e = cudaMalloc(&p->work, p->work_bytes);
+  p->work_bytes = p->one_launch ? 0 : (size_t)batch * (size_t)(n1 / 2) * (size_t)n2 * sizeof(float2);
+  if (p->work_bytes) e = cudaMalloc(&p->work, p->work_bytes);
   // staging array for the map kernels of the other kinds (fs2 folds the maps in)
-  if (e == cudaSuccess && kind != GBDCT_DCT2 && !folds_maps(p->family))
+  if (e == cudaSuccess && kind != GBDCT_DCT2 && !folds_maps(p))
     e = cudaMalloc(&p->tmp, (size_t)batch * (size_t)n1 * (size_t)n2 * sizeof(float));
   if (e != cudaSuccess) {
     free_plan(p);
@@ -542,7 +555,6 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   }
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemset(p->err, 0, 16);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->nsm, cudaDevAttrMultiProcessorCount, p->device);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     free_plan(p);
@@ -572,13 +584,16 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   a.fsA = fsA;
   a.fsB = fsB;
   a.tpNP = (two_pass && tp_np_ok) ? strip_np : 0;  // strip width of the column pass (0: default)
-  a.vkind = folds_maps(p->family) ? kind : 0;
+  a.vkind = folds_maps(p) ? kind : 0;
   a.nsm = p->nsm;
   p->b_cols = gbdct::choose_seq_per_cta(n1, n2 / 2);
   p->b_rows = gbdct::choose_seq_per_cta(n2, n1 / 2);
 
   // Raise the dynamic shared-memory limit of the kernels once.
-  if (p->family == FAM_FS2) {
+  if (p->one_launch) {
+    e = gbdct::run_small_fwd(p->lg1, p->lg2, a, 1, 0, true);
+    if (e == cudaSuccess) e = gbdct::run_small_inv(p->lg1, p->lg2, a, 1, 0, true);
+  } else if (p->family == FAM_FS2) {
     e = gbdct::run_fs2(p->lg1, p->lg2, false, a, 1, 0, true);
   } else if (p->family == FAM_TP) {
     e = gbdct::run_tp(p->lg1, p->lg2, false, a, 1, 0, true);
@@ -617,7 +632,7 @@ gbdct_status gbdct_plan_create(gbdct_plan_t* out, int ndim, const int64_t* dims,
 static gbdct_status exec_core(gbdct_plan_t p, const void* in, void* out, cudaStream_t s, bool inverse,
                               int step = -1, bool io_dev = false);
 static int core_launches(gbdct_plan_t p) {
-  return p->family == FAM_FS2 ? 3 : 2;
+  return p->one_launch ? 1 : p->family == FAM_FS2 ? 3 : 2;
 }
 
 static cudaError_t run_map(gbdct_plan_t p, const float* in, float* out, MapSpec m, cudaStream_t s) {
@@ -644,7 +659,7 @@ static gbdct_status exec2d(gbdct_plan_t p, const void* in, void* out, void* stre
                      : gbdct::gemm_exec(p->gemm, inverse, static_cast<const float*>(in), static_cast<float*>(out), s);
   if (p->kind == GBDCT_DCT2) return exec_core(p, in, out, s, inverse, step, io_dev);
   if (!inverse && (p->kind == GBDCT_IDCT_IDXST || p->kind == GBDCT_IDXST_IDCT)) return GBDCT_ERR_UNSUPPORTED;
-  if (folds_maps(p->family)) return exec_core(p, in, out, s, inverse, step, io_dev);  // maps folded in (vkind)
+  if (folds_maps(p)) return exec_core(p, in, out, s, inverse, step, io_dev);  // maps folded in (vkind)
   MapSpec pre{}, post{};
   if (p->kind == GBDCT_DST2) {
     if (!inverse) {
@@ -690,6 +705,9 @@ static gbdct_status exec_core(gbdct_plan_t p, const void* in, void* out, cudaStr
   const int batch = (int)p->batch;
   const bool s0 = step < 0 || step == 0, s1 = step < 0 || step == 1;
   cudaError_t e = cudaSuccess;
+  if (p->one_launch)
+    return cuda_status(inverse ? gbdct::run_small_inv(p->lg1, p->lg2, a, batch, s, false)
+                               : gbdct::run_small_fwd(p->lg1, p->lg2, a, batch, s, false));
   if (p->family == FAM_FS2) {
     return cuda_status(gbdct::run_fs2(p->lg1, p->lg2, inverse, a, batch, s, false));
   }
@@ -796,9 +814,10 @@ const char* gbdct_plan_step_name(gbdct_plan_t plan, int inverse, int step) {
                                 "row pass (split + row FFT + postprocess)"};
   static const char* kInv3[] = {"row pass (preprocess + row IFFT + pairing)", "column step C2' (DFT_A + twiddle)",
                                 "column step C1' (DFT_B + inverse reorder)"};
+  if (plan->one_launch) return "whole transform (one CTA each)";
   const bool three = core_launches(plan) == 3;
   int k = step;
-  if (plan->kind != GBDCT_DCT2 && !folds_maps(plan->family)) {
+  if (plan->kind != GBDCT_DCT2 && !folds_maps(plan)) {
     if (k == 0) return "index/sign map (pre)";
     if (k == gbdct_plan_launches_per_exec(plan) - 1) return "index/sign map (post)";
     k -= 1;
@@ -841,7 +860,7 @@ int gbdct_plan_launches_per_exec(gbdct_plan_t plan) {
   if (plan->precision == GBDCT_PREC_SPLIT_BF16) return 3;  // split kernel + two tensor-core products
   if (plan->ndim == 3) return gbdct_plan_launches_per_exec(plan->inner) + 1;
   const int core = core_launches(plan);
-  return (plan->kind == GBDCT_DCT2 || folds_maps(plan->family)) ? core : core + 2;
+  return (plan->kind == GBDCT_DCT2 || folds_maps(plan)) ? core : core + 2;
 }
 
 const char* gbdct_plan_kernel_family(gbdct_plan_t plan) {
@@ -856,7 +875,8 @@ const char* gbdct_plan_kernel_family(gbdct_plan_t plan) {
 
 gbdct_status gbdct_plan_set_threshold(gbdct_plan_t plan, float eps) {
   if (!plan || !(eps >= 0.f)) return GBDCT_ERR_INVALID_ARG;
-  if (plan->ndim != 2 || !folds_maps(plan->family) || plan->n2 > 8192) return GBDCT_ERR_UNSUPPORTED;
+  const bool supported = plan->family == FAM_FS2 || plan->family == FAM_TP;
+  if (plan->ndim != 2 || !supported || plan->n2 > 8192) return GBDCT_ERR_UNSUPPORTED;
   plan->args.thresh = eps;
   return GBDCT_OK;
 }

@@ -142,6 +142,20 @@ gbdct_status gbdct_plan_create_tuned(gbdct_plan_t* out, int ndim, const int64_t*
       family_out[family_cap - 1] = 0;
     }
   };
+  // A cached name that is the default plan's own means that plan, which for a
+  // small shape runs one launch (a plan of the named family would not).
+  const bool small = ndim == 2 && dims[0] > 0 && dims[1] > 0 && dims[0] <= 16384 && dims[0] * dims[1] <= 16384;
+  if (!cached.empty() && small) {
+    gbdct_plan_t p = nullptr;
+    if (gbdct_plan_create_batched(&p, ndim, dims, batch, kind, dtype) == GBDCT_OK) {
+      if (cached == gbdct_plan_kernel_family(p)) {
+        report(cached.c_str());
+        *out = p;
+        return GBDCT_OK;
+      }
+      gbdct_plan_destroy(p);
+    }
+  }
   if (!cached.empty() && gbdct_plan_create_family(out, ndim, dims, batch, kind, dtype, cached.c_str()) == GBDCT_OK) {
     report(cached.c_str());
     return GBDCT_OK;

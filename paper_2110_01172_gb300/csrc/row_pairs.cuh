@@ -190,7 +190,8 @@ __device__ __forceinline__ Outs combine(soa::C2 P, soa::C2 M, float2 avr, float2
 // (output (k1, k2) stored at (N1-1-k1, N2-1-k2)) and the magnitude threshold of
 // Section V-A (outputs below eps stored as zero; 0: off); otherwise the
 // DCT-II order and no threshold, with every column offset an immediate.
-template <int L, bool GENERAL>
+// SMEM: the rows are in shared memory.
+template <int L, bool GENERAL, bool SMEM = false>
 struct FwdOut {
   float *a0, *a1, *b0, *b1;  // rows k1 and kmir of lane a, of lane b
   uint64_t pol;
@@ -199,7 +200,10 @@ struct FwdOut {
 
   __device__ __forceinline__ void put(float* p, float v) const {
     if constexpr (GENERAL) v = fabsf(v) < eps ? 0.f : v;
-    l2::st(p, v, pol);
+    if constexpr (SMEM)
+      *p = v;
+    else
+      l2::st(p, v, pol);
   }
   // the outputs of columns c = base + off and L - c (off a compile-time constant)
   __device__ __forceinline__ void store(const Outs& o, int base, int off, bool mirror) const {
@@ -218,8 +222,8 @@ struct FwdOut {
 };
 
 // Postprocess of a group's two rows from the last stage's registers.
-template <int L, bool FIRST, bool GENERAL>
-__device__ __forceinline__ void fwd_post(soa::C2* v, const FwdOut<L, GENERAL>& out, float2 avr, float2 avi,
+template <int L, bool FIRST, typename Out>
+__device__ __forceinline__ void fwd_post(soa::C2* v, const Out& out, float2 avr, float2 avi,
                                          const float4* __restrict__ fb4, int g, bool packed) {
   using S = Last<L>;
   constexpr int NS = S::NS, R = S::R;
