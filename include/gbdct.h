@@ -229,10 +229,11 @@ gbdct_status gbdct_plan_create_tuned(gbdct_plan_t* out, int ndim, const int64_t*
 /*
  * Precision mode of a plan.  GBDCT_PREC_SPLIT_BF16 evaluates the separable
  * definition as dense products, X = C1 x C2^T forward and x = D1 X D2^T
- * inverse (C the DCT-II matrix, D its exact inverse), on the tensor cores by
- * a hand-written tcgen05 kernel: every operand is split into bf16 hi + lo
- * parts and each product is accumulated in FP32 (in tensor memory) as
- * hi*hi + hi*lo + lo*hi.  Its error is that of the split (about 5e-6 relative
+ * inverse (C the DCT-II matrix, D its exact inverse), by frequency parity at
+ * half size along each axis, on the tensor cores by a hand-written tcgen05
+ * kernel: every operand is split into bf16 hi + lo parts and each product is
+ * accumulated in FP32 (in tensor memory) as hi*hi + hi*lo + lo*hi + lo*lo.
+ * Its error is that of the split (about 5e-6 relative
  * in L2, stated per result), not the FP32 path's.  Supported for 2D GBDCT_DCT2
  * plans with both sides between 128 and 2048 (UNSUPPORTED otherwise); the
  * first switch allocates the matrices (FP64-generated, split once) and four

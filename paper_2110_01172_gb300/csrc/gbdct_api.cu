@@ -857,7 +857,7 @@ gbdct_status gbdct_plan_set_precision(gbdct_plan_t plan, int precision) {
 
 int gbdct_plan_launches_per_exec(gbdct_plan_t plan) {
   if (!plan) return 0;
-  if (plan->precision == GBDCT_PREC_SPLIT_BF16) return 3;  // split kernel + two tensor-core products
+  if (plan->precision == GBDCT_PREC_SPLIT_BF16) return 3;  // split + two tensor-core products (+ mirror sums, inverse)
   if (plan->ndim == 3) return gbdct_plan_launches_per_exec(plan->inner) + 1;
   const int core = core_launches(plan);
   return (plan->kind == GBDCT_DCT2 || folds_maps(plan)) ? core : core + 2;

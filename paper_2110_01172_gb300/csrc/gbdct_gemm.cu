@@ -16,16 +16,15 @@ struct GemmPath {
   int n1 = 0, n2 = 0, batch = 0, nsm = 0;
   int* err = nullptr;                          // the plan's device error word
   uint32_t polls = tc::kDefaultPolls;          // bound of every device-side wait
-  // row-major N x N matrices, split: C1h C1l D1h D1l (n1), C2h C2l D2h D2l (n2)
+  // Half-size matrices of one side, split: rows [forward p0, forward p1, inverse
+  // p0, inverse p1] of N/2 each, N/2 columns; hi then lo, side 1 then side 2
   __nv_bfloat16* mats = nullptr;
-  __nv_bfloat16 *xh = nullptr, *xl = nullptr;  // split input, [batch n1][n2]
-  __nv_bfloat16 *th = nullptr, *tl = nullptr;  // split intermediate, transposed: [batch n2][n1]
+  __nv_bfloat16 *xh = nullptr, *xl = nullptr;  // split input quadrants, [p2][batch][p1][n1/2][n2/2]
+  __nv_bfloat16 *th = nullptr, *tl = nullptr;  // split intermediate, [p1][batch][p2][n2/2][n1/2]
   size_t bytes = 0;
-  // tensor maps (box 64 x 128 for A operands; 64 x 128 and 64 x 64 for B operands)
-  CUtensorMap xa[2];           // x hi / lo as A of the first product
-  CUtensorMap ra[2][4];        // [BN 128 / 64][C2h, C2l, D2h, D2l] as B of the first product
-  CUtensorMap la[4];           // C1h, C1l, D1h, D1l as A of the second product
-  CUtensorMap tb[2][2];        // [BN 128 / 64][T hi, T lo] as B of the second product
+  // tensor maps, hi / lo (box 64 x 128 for A operands; 64 x 128 and 64 x 64 for B operands)
+  CUtensorMap xa[2], ta[2];        // input quadrants and intermediate as A
+  CUtensorMap m1[2][2], m2[2][2];  // [BN 128 / 64][hi / lo] matrices of side 1 and 2 as B
 };
 
 namespace {
@@ -33,29 +32,122 @@ namespace {
 // Matrix entry in FP64 from the integer-reduced angle m = k (2j+1) mod 4N.
 __device__ double cos_half(long long m, int n) { return cospi((double)(m % (4LL * n)) / (2.0 * n)); }
 
-// C (DCT-II, rows index the output) and D = (2/N) C^T diag(w) for one side n,
-// split into bf16 hi / lo.
-__global__ void k_gemm_mats(__nv_bfloat16* ch, __nv_bfloat16* cl, __nv_bfloat16* dh, __nv_bfloat16* dl, int n) {
+// The half-size matrices of side n (see GemmPath::mats): with j < n/2 the position,
+// k = 2i + p the frequency, forward row i, column j: cos(pi k (2j+1) / 2n);
+// inverse row j, column i: (2/n) w_k cos(pi k (2j+1) / 2n), w_0 = 1/2.
+__global__ void k_gemm_mats(__nv_bfloat16* hi, __nv_bfloat16* lo, int n) {
+  const int h = n / 2;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)n * n) return;
-  const int r = (int)(idx / n), c = (int)(idx % n);
-  const double cv = cos_half((long long)r * (2 * c + 1), n);                                 // C[r][c]
-  const double dv = (2.0 / n) * (c ? 1.0 : 0.5) * cos_half((long long)c * (2 * r + 1), n);  // D[r][c]
-  const __nv_bfloat16 chv = __float2bfloat16_rn((float)cv), dhv = __float2bfloat16_rn((float)dv);
-  ch[idx] = chv;
-  cl[idx] = __float2bfloat16_rn((float)(cv - (double)__bfloat162float(chv)));
-  dh[idx] = dhv;
-  dl[idx] = __float2bfloat16_rn((float)(dv - (double)__bfloat162float(dhv)));
+  if (idx >= 4LL * h * h) return;
+  const int c = (int)(idx % h), r = (int)(idx / h % h), m = (int)(idx / ((long long)h * h));
+  const bool inv = m >= 2;
+  const int k = 2 * (inv ? c : r) + (m & 1), j = inv ? r : c;
+  double v = cos_half((long long)k * (2 * j + 1), n);
+  if (inv) v *= (2.0 / n) * (k ? 1.0 : 0.5);
+  const __nv_bfloat16 hv = __float2bfloat16_rn((float)v);
+  hi[idx] = hv;
+  lo[idx] = __float2bfloat16_rn((float)(v - (double)__bfloat162float(hv)));
 }
 
-__global__ void k_split(const float* __restrict__ v, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                        long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float x = v[i];
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  hi[i] = h;
-  lo[i] = __float2bfloat16_rn(x - __bfloat162float(h));
+// Four values as bf16 hi and lo parts.
+__device__ __forceinline__ void put_split(__nv_bfloat16* hi, __nv_bfloat16* lo, long long i, const float (&v)[4]) {
+  __nv_bfloat16 h[4], l[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    h[j] = __float2bfloat16_rn(v[j]);
+    l[j] = __float2bfloat16_rn(v[j] - __bfloat162float(h[j]));
+  }
+  auto pack = [](const __nv_bfloat16* q) {
+    const __nv_bfloat162 a = __halves2bfloat162(q[0], q[1]), b = __halves2bfloat162(q[2], q[3]);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+  };
+  *reinterpret_cast<uint2*>(hi + i) = pack(h);
+  *reinterpret_cast<uint2*>(lo + i) = pack(l);
+}
+
+__device__ __forceinline__ float4 rev4(float4 v) { return make_float4(v.w, v.z, v.y, v.x); }
+
+// Sums and differences of four float4: s[p1][p2] = (a +- b) +- (c +- d), minus for p = 1
+// (p2 within a pair, p1 between the pairs).
+__device__ __forceinline__ void mirror_sums(float4 a, float4 b, float4 c, float4 d, float (&s)[2][2][4]) {
+  const float va[4] = {a.x, a.y, a.z, a.w}, vb[4] = {b.x, b.y, b.z, b.w};
+  const float vc[4] = {c.x, c.y, c.z, c.w}, vd[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float e0 = va[j] + vb[j], e1 = vc[j] + vd[j], o0 = va[j] - vb[j], o1 = vc[j] - vd[j];
+    s[0][0][j] = e0 + e1;
+    s[1][0][j] = e0 - e1;
+    s[0][1][j] = o0 + o1;
+    s[1][1][j] = o0 - o1;
+  }
+}
+
+// One thread: four columns j2 .. j2+3 of row i1 of every quadrant of one transform.
+struct Quads {
+  int i1, j2, b;
+  bool live;
+  __device__ __forceinline__ Quads(int n1, int n2, int batch) {
+    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int w = n2 / 8;  // groups of four columns in a quadrant's row
+    j2 = 4 * (int)(idx % w);
+    i1 = (int)(idx / w % (n1 / 2));
+    const long long bb = idx / w / (n1 / 2);
+    live = bb < batch;
+    b = live ? (int)bb : 0;
+  }
+};
+
+// The split input quadrants.  Forward: q[p1][p2] = mirror sums of the input over
+// both axes (x_j +- x_{N-1-j}); inverse: the spectrum's entries of parity (p1, p2).
+template <bool INV>
+__global__ void __launch_bounds__(256) k_split(const float* __restrict__ in, __nv_bfloat16* __restrict__ hi,
+                                               __nv_bfloat16* __restrict__ lo, int n1, int n2, int batch) {
+  const Quads t(n1, n2, batch);
+  pdl::wait_prior_grid();
+  pdl::launch_dependents();
+  if (!t.live) return;
+  const float* x = in + (long long)t.b * n1 * n2;
+  auto ld = [&](int r, int c) { return *reinterpret_cast<const float4*>(x + (long long)r * n2 + c); };
+  float q[2][2][4];
+  if constexpr (!INV) {
+    mirror_sums(ld(t.i1, t.j2), rev4(ld(t.i1, n2 - 4 - t.j2)), ld(n1 - 1 - t.i1, t.j2),
+                rev4(ld(n1 - 1 - t.i1, n2 - 4 - t.j2)), q);
+  } else {
+#pragma unroll
+    for (int p1 = 0; p1 < 2; ++p1) {
+      const float4 u = ld(2 * t.i1 + p1, 2 * t.j2), v = ld(2 * t.i1 + p1, 2 * t.j2 + 4);
+      q[p1][0][0] = u.x, q[p1][0][1] = u.z, q[p1][0][2] = v.x, q[p1][0][3] = v.z;
+      q[p1][1][0] = u.y, q[p1][1][1] = u.w, q[p1][1][2] = v.y, q[p1][1][3] = v.w;
+    }
+  }
+  const int h1 = n1 / 2, h2 = n2 / 2;
+#pragma unroll
+  for (int p2 = 0; p2 < 2; ++p2)
+#pragma unroll
+    for (int p1 = 0; p1 < 2; ++p1)
+      put_split(hi, lo, ((((long long)p2 * batch + t.b) * 2 + p1) * h1 + t.i1) * h2 + t.j2, q[p1][p2]);
+}
+
+// Inverse: the output from the quadrants y[b][p1][p2] of the second product, whose
+// entries of odd frequency parity change sign at the mirror position.
+__global__ void __launch_bounds__(256) k_join(const float* __restrict__ y, float* __restrict__ out, int n1, int n2,
+                                              int batch) {
+  const Quads t(n1, n2, batch);
+  pdl::wait_prior_grid();
+  pdl::launch_dependents();
+  if (!t.live) return;
+  const long long quad = (long long)(n1 / 2) * (n2 / 2);
+  const float* q = y + (long long)t.b * n1 * n2 + (long long)t.i1 * (n2 / 2) + t.j2;
+  auto ld = [&](int p1, int p2) { return *reinterpret_cast<const float4*>(q + (2 * p1 + p2) * quad); };
+  float s[2][2][4];  // [mirror of axis 0][mirror of axis 1]
+  mirror_sums(ld(0, 0), ld(0, 1), ld(1, 0), ld(1, 1), s);
+  float* o = out + (long long)t.b * n1 * n2;
+  auto f4 = [](const float (&v)[4]) { return make_float4(v[0], v[1], v[2], v[3]); };
+  const long long r0 = (long long)t.i1 * n2, r1 = (long long)(n1 - 1 - t.i1) * n2;
+  *reinterpret_cast<float4*>(o + r0 + t.j2) = f4(s[0][0]);
+  *reinterpret_cast<float4*>(o + r0 + n2 - 4 - t.j2) = rev4(f4(s[0][1]));
+  *reinterpret_cast<float4*>(o + r1 + t.j2) = f4(s[1][0]);
+  *reinterpret_cast<float4*>(o + r1 + n2 - 4 - t.j2) = rev4(f4(s[1][1]));
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() { return tma::encoder(); }
@@ -73,18 +165,21 @@ bool map2d(CUtensorMap* m, const void* base, long long rows, long long cols, int
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// One product: A (map pair a) times the side's matrices, rows x cols outputs for
+// each of the two parities in blockIdx.z.
 template <int BN>
-cudaError_t launch(const CUtensorMap& ah, const CUtensorMap& al, const CUtensorMap& bh, const CUtensorMap& bl,
-                   const tc::Epi& e, int rows, int cols, int kdim, int nz, uint32_t polls, int* err, cudaStream_t s) {
+cudaError_t launch(const CUtensorMap (&a)[2], const CUtensorMap (&b)[2][2], const tc::Epi& e, int rows, int cols,
+                   int kdim, uint32_t polls, int* err, cudaStream_t s) {
   using Cf = tc::Cfg<BN>;
-  const dim3 grid((unsigned)(cols / BN), (unsigned)(rows / tc::BM), (unsigned)nz);
-  tc::k_tc_dftgemm<BN><<<grid, 128, Cf::SMEM, s>>>(ah, al, bh, bl, e, kdim / tc::BK, polls, err);
-  return cudaGetLastError();
+  const CUtensorMap(&m)[2] = b[BN == 128 ? 0 : 1];
+  const dim3 grid((unsigned)(cols / BN), (unsigned)(rows / tc::BM), 2);
+  return pdl::launch(tc::k_tc_dftgemm<BN>, grid, dim3(128), (size_t)Cf::SMEM, s, a[0], a[1], m[0], m[1], e,
+                     kdim / tc::BK, polls, err);
 }
 
 // BN = 128 when that already gives at least one tile per SM, else 64.
-bool wide_tiles(long long rows, long long cols, int nz, int nsm) {
-  return (rows / tc::BM) * (cols / 128) * nz >= nsm;
+bool wide_tiles(long long rows, long long cols, int nsm) {
+  return cols % 128 == 0 && (rows / tc::BM) * (cols / 128) * 2 >= nsm;
 }
 
 }  // namespace
@@ -104,18 +199,19 @@ GemmPath* gemm_create(int n1, int n2, int batch, int* err, gbdct_status* st) {
   int dev = 0;
   cudaError_t ce = cudaGetDevice(&dev);
   if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&g->nsm, cudaDevAttrMultiProcessorCount, dev);
+  // elements of one side's matrices (hi or lo), and of the array
   const size_t m1 = (size_t)n1 * n1, m2 = (size_t)n2 * n2, e = (size_t)batch * n1 * n2;
-  if (ce == cudaSuccess) ce = cudaMalloc(&g->mats, (4 * m1 + 4 * m2) * sizeof(__nv_bfloat16));
+  if (ce == cudaSuccess) ce = cudaMalloc(&g->mats, 2 * (m1 + m2) * sizeof(__nv_bfloat16));
   if (ce == cudaSuccess) ce = cudaMalloc(&g->xh, 4 * e * sizeof(__nv_bfloat16));  // xh, xl, th, tl
-  g->bytes = (4 * m1 + 4 * m2) * sizeof(__nv_bfloat16) + 4 * e * sizeof(__nv_bfloat16);
+  g->bytes = 2 * (m1 + m2) * sizeof(__nv_bfloat16) + 4 * e * sizeof(__nv_bfloat16);
   if (ce == cudaSuccess) {
     g->xl = g->xh + e;
     g->th = g->xl + e;
     g->tl = g->th + e;
     __nv_bfloat16* m = g->mats;
-    k_gemm_mats<<<(unsigned)((m1 + 255) / 256), 256>>>(m, m + m1, m + 2 * m1, m + 3 * m1, n1);
-    __nv_bfloat16* q = m + 4 * m1;
-    k_gemm_mats<<<(unsigned)((m2 + 255) / 256), 256>>>(q, q + m2, q + 2 * m2, q + 3 * m2, n2);
+    k_gemm_mats<<<(unsigned)((m1 + 255) / 256), 256>>>(m, m + m1, n1);
+    __nv_bfloat16* q = m + 2 * m1;
+    k_gemm_mats<<<(unsigned)((m2 + 255) / 256), 256>>>(q, q + m2, n2);
     ce = cudaGetLastError();
     if (ce == cudaSuccess) ce = cudaDeviceSynchronize();
   }
@@ -126,16 +222,15 @@ GemmPath* gemm_create(int n1, int n2, int batch, int* err, gbdct_status* st) {
   bool maps = ce == cudaSuccess;
   if (maps) {
     const __nv_bfloat16* m = g->mats;
-    const __nv_bfloat16* q = m + 4 * m1;
-    const long long rows1 = (long long)batch * n1;
-    maps = map2d(&g->xa[0], g->xh, rows1, n2, tc::BM) && map2d(&g->xa[1], g->xl, rows1, n2, tc::BM);
-    for (int w = 0; w < 2 && maps; ++w) {
-      const int bn = w ? 64 : 128;
-      for (int i = 0; i < 4 && maps; ++i) maps = map2d(&g->ra[w][i], q + i * m2, n2, n2, bn);
-      maps = maps && map2d(&g->tb[w][0], g->th, (long long)batch * n2, n1, bn) &&
-             map2d(&g->tb[w][1], g->tl, (long long)batch * n2, n1, bn);
+    const __nv_bfloat16* q = m + 2 * m1;
+    const long long xr = 2LL * batch * n1, tr = 2LL * batch * n2;  // both parities stacked
+    for (int l = 0; l < 2 && maps; ++l) {
+      maps = map2d(&g->xa[l], l ? g->xl : g->xh, xr, n2 / 2, tc::BM) &&
+             map2d(&g->ta[l], l ? g->tl : g->th, tr, n1 / 2, tc::BM);
+      for (int w = 0; w < 2 && maps; ++w)
+        maps = map2d(&g->m1[w][l], m + l * m1, 2LL * n1, n1 / 2, w ? 64 : 128) &&
+               map2d(&g->m2[w][l], q + l * m2, 2LL * n2, n2 / 2, w ? 64 : 128);
     }
-    for (int i = 0; i < 4 && maps; ++i) maps = map2d(&g->la[i], m + i * m1, n1, n1, tc::BM);
   }
   if (ce != cudaSuccess || !maps) {
     gemm_destroy(g);
@@ -151,30 +246,27 @@ void gemm_set_wait_polls(GemmPath* g, uint32_t polls) {
 }
 
 gbdct_status gemm_exec(GemmPath* g, bool inverse, const float* in, float* out, cudaStream_t s) {
-  const int n1 = g->n1, n2 = g->n2;
-  const long long e = (long long)g->batch * n1 * n2;
-  const int r0 = inverse ? 2 : 0;  // forward: C1, C2; inverse: D1, D2
-  k_split<<<(unsigned)((e + 255) / 256), 256, 0, s>>>(in, g->xh, g->xl, e);
-  cudaError_t ce = cudaGetLastError();
-  // first product T = x R^T (rows: batch * n1), stored split and transposed
-  tc::Epi e1{tc::EPI_SPLIT_T, n1, n2, 0, 0, g->th, g->tl, nullptr};
-  const long long rows1 = (long long)g->batch * n1;
-  if (ce == cudaSuccess) {
-    const bool wide = wide_tiles(rows1, n2, 1, g->nsm);
-    ce = wide ? launch<128>(g->xa[0], g->xa[1], g->ra[0][r0], g->ra[0][r0 + 1], e1, (int)rows1, n2, n2, 1, g->polls,
-                            g->err, s)
-              : launch<64>(g->xa[0], g->xa[1], g->ra[1][r0], g->ra[1][r0 + 1], e1, (int)rows1, n2, n2, 1, g->polls,
-                           g->err, s);
-  }
-  // second product out_b = L T_b (rows n1 per batch entry)
-  tc::Epi e2{tc::EPI_F32, n1, n2, 0, n2, nullptr, nullptr, out};
-  if (ce == cudaSuccess) {
-    const bool wide = wide_tiles(n1, n2, g->batch, g->nsm);
-    ce = wide ? launch<128>(g->la[r0], g->la[r0 + 1], g->tb[0][0], g->tb[0][1], e2, n1, n2, n1, g->batch, g->polls,
-                            g->err, s)
-              : launch<64>(g->la[r0], g->la[r0 + 1], g->tb[1][0], g->tb[1][1], e2, n1, n2, n1, g->batch, g->polls,
-                           g->err, s);
-  }
+  const int n1 = g->n1, n2 = g->n2, h1 = n1 / 2, h2 = n2 / 2, batch = g->batch;
+  const long long threads = (long long)batch * h1 * (n2 / 8);
+  const dim3 blocks((unsigned)((threads + 255) / 256));
+  cudaError_t ce = inverse ? pdl::launch(k_split<true>, blocks, dim3(256), 0, s, in, g->xh, g->xl, n1, n2, batch)
+                           : pdl::launch(k_split<false>, blocks, dim3(256), 0, s, in, g->xh, g->xl, n1, n2, batch);
+  // first product, along axis 1 (rows (b, p1, i1), for each parity p2)
+  const tc::Epi e1{tc::EPI_SPLIT_T, n1, n2, batch, batch * n1, h2, inverse ? n2 : 0, g->th, g->tl, nullptr};
+  if (ce == cudaSuccess)
+    ce = wide_tiles((long long)batch * n1, h2, g->nsm)
+             ? launch<128>(g->xa, g->m2, e1, batch * n1, h2, h2, g->polls, g->err, s)
+             : launch<64>(g->xa, g->m2, e1, batch * n1, h2, h2, g->polls, g->err, s);
+  // second product, along axis 0 (rows (b, p2, j2), for each parity p1); the
+  // inverse's quadrants reuse the split input's memory
+  float* y = reinterpret_cast<float*>(g->xh);
+  const tc::Epi e2{inverse ? tc::EPI_QUADRANT : tc::EPI_DCT, n1, n2, batch, batch * n2, h1, inverse ? n1 : 0, nullptr,
+                   nullptr, inverse ? y : out};
+  if (ce == cudaSuccess)
+    ce = wide_tiles((long long)batch * n2, h1, g->nsm)
+             ? launch<128>(g->ta, g->m1, e2, batch * n2, h1, h1, g->polls, g->err, s)
+             : launch<64>(g->ta, g->m1, e2, batch * n2, h1, h1, g->polls, g->err, s);
+  if (ce == cudaSuccess && inverse) ce = pdl::launch(k_join, blocks, dim3(256), 0, s, static_cast<const float*>(y), out, n1, n2, batch);
   return ce == cudaSuccess ? GBDCT_OK : GBDCT_ERR_CUDA;
 }
 

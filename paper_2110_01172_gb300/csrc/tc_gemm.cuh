@@ -3,22 +3,22 @@
 //
 // One CTA computes one 128 x BN tile of D = A B^T for row-major ("K-major")
 // operands A (rows x K) and B (cols x K), each given as a bf16 pair hi + lo:
-//   D = Ah Bh^T + Ah Bl^T + Al Bh^T
-// (the lo lo term is dropped), all three products accumulated into the same
-// FP32 accumulator in tensor memory.  K advances in blocks of 64 elements: the
-// four operand tiles of a block (128 x 64 and BN x 64 bf16, 128-byte rows with
-// the 128-byte swizzle) arrive by tiled tensor loads into a ring of NST
+//   D = Ah Bh^T + Ah Bl^T + Al Bh^T + Al Bl^T,
+// all four products accumulated into the same FP32 accumulator in tensor
+// memory.  K advances in blocks of 64 elements: the four operand tiles of a
+// block (128 x 64 and BN x 64 bf16, 128-byte rows with the 128-byte swizzle) arrive by tiled tensor loads into a ring of NST
 // shared-memory stages; one thread issues the loads and the MMAs (K = 16 per
 // instruction) and releases a stage with tcgen05.commit when the MMAs that
 // read it are done.  The four warps then read the accumulator rows back with
 // tcgen05.ld (warp w owns lanes 32w .. 32w+31, lane = tile row) and apply the
 // epilogue:
-//   EPI_SPLIT_T   row r of the tile is (batch b, n1) = (r / N1, r % N1) of the
-//                 first product T = x M^T; it is stored transposed and split,
-//                 Th/Tl[b][col][n1], as the K-major operand of the second
-//                 product
-//   EPI_F32       row r is output row k1 of batch entry blockIdx.z; stored as
-//                 FP32, out[b][k1][col]
+//   EPI_SPLIT_T   first product: row (b, p1, i1) of A, column j2 of parity
+//                 p2 = blockIdx.z; stored split and transposed,
+//                 Th/Tl[p1][b][p2][j2][i1], as the K-major operand of the second
+//   EPI_DCT       second product of the forward: row (b, p2, j2), column j1 of
+//                 parity p1 = blockIdx.z -> out[b][2 j1 + p1][2 j2 + p2]
+//   EPI_QUADRANT  second product of the inverse: the same row and column
+//                 -> y[b][p1][p2][j1][j2] (the mirror sums follow)
 // Every mbarrier wait is bounded (poll limit); a wait that gives up records
 // the failure in the device error word, the issuing thread stops issuing,
 // waits (with the default limit) for the copies it issued and commits, so the
@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "launch_dep.cuh"
 #include "tma_util.cuh"
 
 namespace gbdct {
@@ -41,7 +42,7 @@ constexpr int BK = 64;                   // K per stage: one 128-byte swizzle ro
 constexpr uint32_t kDefaultPolls = tma::kDefaultPolls;
 using tma::bar_wait;
 using tma::su32;
-enum { EPI_SPLIT_T = 0, EPI_F32 = 1 };
+enum { EPI_SPLIT_T = 0, EPI_DCT = 1, EPI_QUADRANT = 2 };
 
 template <int BN>
 struct Cfg {
@@ -56,13 +57,13 @@ struct Cfg {
 };
 
 struct Epi {
-  int mode;                 // EPI_SPLIT_T or EPI_F32
-  int n1, n2;               // transform sides
-  int a_batch_rows;         // A row offset per blockIdx.z
-  int b_batch_rows;         // B row offset per blockIdx.z
+  int mode;                 // EPI_*
+  int n1, n2, batch;        // transform sides, transforms
+  int a_rows, b_rows;       // operand row offsets per blockIdx.z
+  int b_base;               // first operand row of B
   __nv_bfloat16* th;        // EPI_SPLIT_T outputs
   __nv_bfloat16* tl;
-  float* out;               // EPI_F32 output
+  float* out;               // EPI_DCT / EPI_QUADRANT output
 };
 
 // Shared-memory matrix descriptor of a K-major bf16 tile with the 128-byte
@@ -109,8 +110,9 @@ k_tc_dftgemm(const __grid_constant__ CUtensorMap mah, const __grid_constant__ CU
   int* fail = reinterpret_cast<int*>(tslot + 1);
   const int warp = threadIdx.x / 32;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int arow = e.a_batch_rows * (int)blockIdx.z + m0;
-  const int brow = e.b_batch_rows * (int)blockIdx.z + n0;
+  const int z = (int)blockIdx.z;
+  const int arow = e.a_rows * z + m0;
+  const int brow = e.b_base + e.b_rows * z + n0;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NST; ++i) {
@@ -130,6 +132,7 @@ k_tc_dftgemm(const __grid_constant__ CUtensorMap mah, const __grid_constant__ CU
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
+  pdl::wait_prior_grid();  // the operands and the outputs' last readers
 
   if (threadIdx.x == 0) {
     auto stage_ptr = [&](int s) { return sm + s * C::STAGE; };
@@ -167,6 +170,7 @@ k_tc_dftgemm(const __grid_constant__ CUtensorMap mah, const __grid_constant__ CU
         mma_bf16(tmem, sw128_desc(ah + off), sw128_desc(bh + off), C::IDESC, first);
         mma_bf16(tmem, sw128_desc(ah + off), sw128_desc(bl + off), C::IDESC, 1u);
         mma_bf16(tmem, sw128_desc(al + off), sw128_desc(bh + off), C::IDESC, 1u);
+        mma_bf16(tmem, sw128_desc(al + off), sw128_desc(bl + off), C::IDESC, 1u);
       }
       commit(empty + s);
       // refill the stage of block kb-1 once its MMAs are done
@@ -191,6 +195,7 @@ k_tc_dftgemm(const __grid_constant__ CUtensorMap mah, const __grid_constant__ CU
   const bool fin = bar_wait(done, 0, kDefaultPolls);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   __syncthreads();
+  pdl::launch_dependents();
   if (!fin && threadIdx.x == 0) atomicExch(err, 1);
   if (fin && !*fail) {
     const int r = warp * 32 + (threadIdx.x & 31);  // tile row = TMEM lane
@@ -205,22 +210,27 @@ k_tc_dftgemm(const __grid_constant__ CUtensorMap mah, const __grid_constant__ CU
             "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
           : "r"(ta));
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (e.mode == EPI_F32) {
-        float* o = e.out + ((long long)blockIdx.z * e.n1 + row) * e.n2 + n0 + c0;
-#pragma unroll
-        for (int i = 0; i < 16; i += 4)
-          *reinterpret_cast<float4*>(o + i) = make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]),
-                                                          __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
-      } else {
-        const int b = row / e.n1, n1 = row % e.n1;
+      if (e.mode == EPI_SPLIT_T) {
+        const int h1 = e.n1 / 2, h2 = e.n2 / 2;
+        const int i1 = row % h1, q = row / h1, b = q >> 1, p1 = q & 1;
+        const long long col = (((long long)p1 * e.batch + b) * 2 + z) * h2 + n0 + c0;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const float x = __uint_as_float(v[i]);
           const __nv_bfloat16 h = __float2bfloat16_rn(x);
-          const long long idx = ((long long)b * e.n2 + n0 + c0 + i) * e.n1 + n1;
+          const long long idx = (col + i) * h1 + i1;
           e.th[idx] = h;
           e.tl[idx] = __float2bfloat16_rn(x - __bfloat162float(h));
         }
+      } else {
+        const int h1 = e.n1 / 2, h2 = e.n2 / 2;
+        const int j2 = row % h2, q = row / h2, b = q >> 1, p2 = q & 1;
+        const bool dct = e.mode == EPI_DCT;
+        float* o = dct ? e.out + ((long long)b * e.n1 + 2 * (n0 + c0) + z) * e.n2 + 2 * j2 + p2
+                       : e.out + ((((long long)b * 2 + z) * 2 + p2) * h1 + n0 + c0) * h2 + j2;
+        const long long step = dct ? 2LL * e.n2 : h2;  // to the next column j1
+#pragma unroll
+        for (int i = 0; i < 16; ++i) o[i * step] = __uint_as_float(v[i]);
       }
     }
   }
