@@ -387,7 +387,15 @@ __device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a
 // shared buffer by contiguous bulk copies (one mbarrier per group, bounded
 // wait as in the column pass), so few registers hold loads in flight; the
 // buffer (17 L bytes) holds the 16 L bytes of the rows until the first FFT
-// stage overwrites it.  Device buffers only.
+// stage overwrites it.  Device buffers only.  Otherwise the preprocess loads
+// its points straight from global memory, every value once: faster for short
+// rows, whose groups would all wait for the slowest group's copies (inverse,
+// staged vs direct: 25 x 512^2 22.3 vs 20.6 us, 64 x 256^2 13.9 vs 13.5, 1024^2
+// 8.9 vs 8.6, 2048^2 17.5 vs 17.3, but 4096^2 62.3 vs 63.3).  A Poisson solve,
+// which also loads a denominator for every value, stages at every length (512^2
+// 19.8 vs 21.0 us).
+template <int L>
+constexpr bool tp_inv_staged() { return L >= 4096; }
 
 // The scaled reads of a Poisson solve: RowReads' value times the eigenvalue
 // denominator and (entry 1) the row's wu or (entry 2) the column's wv.

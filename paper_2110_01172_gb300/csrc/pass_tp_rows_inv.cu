@@ -15,22 +15,28 @@ cudaError_t launch_k(const Dct2dArgs& a, const PoissonArgs& ps, int batch, cudaS
   return pdl::launch(k, dim3(a.n1 / 4 / R::NP, 1, batch), dim3(R::THREADS), SMEM, s, a, ps);
 }
 
+template <int L, bool NARROW, bool MAPPED>
+cudaError_t launch_m(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
+  const PoissonArgs none{};
+  if constexpr (tp_inv_staged<L>()) {
+    if (prepare) {
+      const cudaError_t e = launch_k<L, NARROW, MAPPED, true>(a, none, batch, s, true);
+      if (e != cudaSuccess) return e;
+    } else if (a.io_dev) {
+      return launch_k<L, NARROW, MAPPED, true>(a, none, batch, s, false);
+    }
+  }
+  return launch_k<L, NARROW, MAPPED, false>(a, none, batch, s, prepare);
+}
+
 template <int L, bool NARROW>
 cudaError_t launch_n(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
-  const PoissonArgs none{};
   if (prepare) {
-    cudaError_t e = launch_k<L, NARROW, false, false>(a, none, batch, s, true);
-    if (e == cudaSuccess) e = launch_k<L, NARROW, false, true>(a, none, batch, s, true);
-    if (e == cudaSuccess) e = launch_k<L, NARROW, true, false>(a, none, batch, s, true);
-    if (e == cudaSuccess) e = launch_k<L, NARROW, true, true>(a, none, batch, s, true);
-    return e;
+    const cudaError_t e = launch_m<L, NARROW, false>(a, batch, s, true);
+    return e == cudaSuccess ? launch_m<L, NARROW, true>(a, batch, s, true) : e;
   }
-  // device input: the rows are staged by bulk copies; host-mapped input: read directly
-  if (a.vkind == 1 || a.vkind == 2)
-    return a.io_dev ? launch_k<L, NARROW, true, true>(a, none, batch, s, false)
-                    : launch_k<L, NARROW, true, false>(a, none, batch, s, false);
-  return a.io_dev ? launch_k<L, NARROW, false, true>(a, none, batch, s, false)
-                  : launch_k<L, NARROW, false, false>(a, none, batch, s, false);
+  return (a.vkind == 1 || a.vkind == 2) ? launch_m<L, NARROW, true>(a, batch, s, false)
+                                        : launch_m<L, NARROW, false>(a, batch, s, false);
 }
 
 template <int L>

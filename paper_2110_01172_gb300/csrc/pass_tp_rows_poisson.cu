@@ -15,18 +15,22 @@ cudaError_t launch_k(const Dct2dArgs& a, const PoissonArgs& ps, int batch, cudaS
   return pdl::launch(k, dim3(a.n1 / 4 / R::NP, 1, batch), dim3(R::THREADS), SMEM, s, a, ps);
 }
 
+template <int L, bool NARROW>
+cudaError_t launch_n(const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare) {
+  if (prepare) {
+    const cudaError_t e = launch_k<L, NARROW, true, false>(a, ps, 3, s, true);
+    return e == cudaSuccess ? launch_k<L, NARROW, true, true>(a, ps, 3, s, true) : e;
+  }
+  return a.io_dev ? launch_k<L, NARROW, true, true>(a, ps, 3, s, false) : launch_k<L, NARROW, true, false>(a, ps, 3, s, false);
+}
+
 template <int L>
 cudaError_t launch(const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare) {
   if (prepare) {
-    cudaError_t e = launch_k<L, false, true, false>(a, ps, 3, s, true);
-    if (e == cudaSuccess) e = launch_k<L, false, true, true>(a, ps, 3, s, true);
-    if (e == cudaSuccess) e = launch_k<L, true, true, false>(a, ps, 3, s, true);
-    if (e == cudaSuccess) e = launch_k<L, true, true, true>(a, ps, 3, s, true);
-    return e;
+    const cudaError_t e = launch_n<L, false>(a, ps, s, true);
+    return e == cudaSuccess ? launch_n<L, true>(a, ps, s, true) : e;
   }
-  if (tp_rows_narrow<L>(a, 3))
-    return a.io_dev ? launch_k<L, true, true, true>(a, ps, 3, s, false) : launch_k<L, true, true, false>(a, ps, 3, s, false);
-  return a.io_dev ? launch_k<L, false, true, true>(a, ps, 3, s, false) : launch_k<L, false, true, false>(a, ps, 3, s, false);
+  return tp_rows_narrow<L>(a, 3) ? launch_n<L, true>(a, ps, s, false) : launch_n<L, false>(a, ps, s, false);
 }
 
 }  // namespace
