@@ -125,16 +125,31 @@ def _check(status: int, what: str):
         raise GbdctError(status, what)
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
+_current_stream = None
 
 
 def _stream_handle(stream, device):
-    torch = _torch()
-    if stream is None:
-        stream = torch.cuda.current_stream(device)
-    return ctypes.c_void_p(stream.cuda_stream)
+    """Raw handle of `stream`, or of the device's current stream (asked for on
+    every call; the raw query skips building a Stream object, 1 us)."""
+    global _current_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _current_stream is None:
+        torch = _torch()
+        _current_stream = (getattr(torch._C, "_cuda_getCurrentRawStream", None)
+                           or (lambda index: torch.cuda.current_stream(index).cuda_stream))
+    return _current_stream(device.index)
 
 
 class Plan:
@@ -173,6 +188,7 @@ class Plan:
                 _check(lib.gbdct_plan_create_batched(*args), "gbdct_plan_create")
         self._h = handle
         self._lib = lib
+        self._want = ((self.batch,) if self.batch > 1 else ()) + self.shape
 
     @property
     def workspace_bytes(self) -> int:
@@ -199,7 +215,13 @@ class Plan:
         """x and out: CUDA float32 tensors, or page-locked CPU float32 tensors
         (read/written by the kernels over the host link, no staging copy)."""
         torch = _torch()
-        want = ((self.batch,) if self.batch > 1 else ()) + self.shape
+        want = self._want
+        f32 = torch.float32
+        if x.is_cuda and x.dtype is f32 and x.shape == want and x.is_contiguous():  # the usual call
+            if out is None:
+                return x, torch.empty_like(x)
+            if out.is_cuda and out.dtype is f32 and out.shape == want and out.is_contiguous():
+                return x, out
 
         def usable(t):
             return t.dtype == torch.float32 and (t.is_cuda or (t.device.type == "cpu" and t.is_pinned()))
@@ -218,15 +240,13 @@ class Plan:
 
     def forward(self, x, out=None, stream=None):
         x, out = self._prep(x, out)
-        _check(self._lib.gbdct_exec_forward(self._h, ctypes.c_void_p(x.data_ptr()),
-                                            ctypes.c_void_p(out.data_ptr()),
+        _check(self._lib.gbdct_exec_forward(self._h, x.data_ptr(), out.data_ptr(),
                                             _stream_handle(stream, self.device)), "gbdct_exec_forward")
         return out
 
     def inverse(self, x, out=None, stream=None):
         x, out = self._prep(x, out)
-        _check(self._lib.gbdct_exec_inverse(self._h, ctypes.c_void_p(x.data_ptr()),
-                                            ctypes.c_void_p(out.data_ptr()),
+        _check(self._lib.gbdct_exec_inverse(self._h, x.data_ptr(), out.data_ptr(),
                                             _stream_handle(stream, self.device)), "gbdct_exec_inverse")
         return out
 
@@ -339,9 +359,8 @@ class MultiPlan:
         if x.dtype != torch.float32 or not x.is_cuda or x.numel() != self.total or not x.is_contiguous():
             raise ValueError(f"expected a contiguous CUDA float32 buffer of {self.total} values")
         out = torch.empty_like(x) if out is None else out
-        _check(self._lib.gbdct_multi_exec(self._h, int(inverse), ctypes.c_void_p(x.data_ptr()),
-                                          ctypes.c_void_p(out.data_ptr()), _stream_handle(stream, self.device)),
-               "gbdct_multi_exec")
+        _check(self._lib.gbdct_multi_exec(self._h, int(inverse), x.data_ptr(), out.data_ptr(),
+                                          _stream_handle(stream, self.device)), "gbdct_multi_exec")
         return out
 
     def forward(self, x, out=None, stream=None):
@@ -389,10 +408,8 @@ class PoissonSolver:
         psi = torch.empty_like(rho) if psi is None else psi
         xi0 = torch.empty_like(rho) if xi0 is None else xi0
         xi1 = torch.empty_like(rho) if xi1 is None else xi1
-        _check(self._lib.gbdct_poisson_solve(self._h, ctypes.c_void_p(rho.data_ptr()),
-                                             ctypes.c_void_p(psi.data_ptr()), ctypes.c_void_p(xi0.data_ptr()),
-                                             ctypes.c_void_p(xi1.data_ptr()), _stream_handle(stream, rho.device)),
-               "gbdct_poisson_solve")
+        _check(self._lib.gbdct_poisson_solve(self._h, rho.data_ptr(), psi.data_ptr(), xi0.data_ptr(), xi1.data_ptr(),
+                                             _stream_handle(stream, rho.device)), "gbdct_poisson_solve")
         return psi, xi0, xi1
 
     def close(self):
@@ -410,72 +427,58 @@ class PoissonSolver:
 _plans: dict = {}
 
 
-def _cached_plan(shape, kind, batch, device):
-    key = (tuple(shape), kind, batch, device)
+def _cached_plan(kind, ndim, x):
+    """The plan of the one-call functions for x: an array of `ndim` axes, or (2D) a batch of them."""
+    key = (kind, ndim, x.shape, x.get_device())
     p = _plans.get(key)
     if p is None:
-        p = Plan(shape, kind, batch, device)
-        _plans[key] = p
+        if ndim == 3 and x.dim() != 3:
+            raise ValueError("expected a 3D tensor")
+        if ndim == 2 and x.dim() not in (2, 3):
+            raise ValueError("expected a 2D tensor or a batch of 2D tensors")
+        p = _plans[key] = Plan(tuple(x.shape[-ndim:]), kind, int(x.shape[0]) if x.dim() > ndim else 1, x.device)
     return p
-
-
-def _split(x):
-    if x.dim() == 2:
-        return tuple(x.shape), 1
-    if x.dim() == 3:
-        return tuple(x.shape[1:]), int(x.shape[0])
-    raise ValueError("expected a 2D tensor or a batch of 2D tensors")
 
 
 def dct2(x, out=None):
     """2D DCT-II (unnormalised) of a CUDA float32 (N1, N2) or (B, N1, N2) tensor."""
-    shape, batch = _split(x)
-    return _cached_plan(shape, "dct2", batch, x.device).forward(x, out)
+    return _cached_plan("dct2", 2, x).forward(x, out)
 
 
 def idct2(x, out=None):
     """Exact inverse of ``dct2`` (2/N-scaled DCT-III per axis)."""
-    shape, batch = _split(x)
-    return _cached_plan(shape, "dct2", batch, x.device).inverse(x, out)
+    return _cached_plan("dct2", 2, x).inverse(x, out)
 
 
 def dct3(x, out=None):
     """3D DCT-II (unnormalised, the 1D DCT-II along every axis) of a CUDA float32
     (N0, N1, N2) tensor."""
-    if x.dim() != 3:
-        raise ValueError("expected a 3D tensor")
-    return _cached_plan(tuple(x.shape), "dct2", 1, x.device).forward(x, out)
+    return _cached_plan("dct2", 3, x).forward(x, out)
 
 
 def idct3(x, out=None):
     """Exact inverse of ``dct3``."""
-    if x.dim() != 3:
-        raise ValueError("expected a 3D tensor")
-    return _cached_plan(tuple(x.shape), "dct2", 1, x.device).inverse(x, out)
+    return _cached_plan("dct2", 3, x).inverse(x, out)
 
 
 def dst2(x, out=None):
     """2D DST-II (unnormalised sine analogue of ``dct2``)."""
-    shape, batch = _split(x)
-    return _cached_plan(shape, "dst2", batch, x.device).forward(x, out)
+    return _cached_plan("dst2", 2, x).forward(x, out)
 
 
 def idst2(x, out=None):
     """Exact inverse of ``dst2``."""
-    shape, batch = _split(x)
-    return _cached_plan(shape, "dst2", batch, x.device).inverse(x, out)
+    return _cached_plan("dst2", 2, x).inverse(x, out)
 
 
 def idct_idxst(x, out=None):
     """IDCT along axis 0 and IDXST along axis 1 (2/N-scaled, like ``idct2``)."""
-    shape, batch = _split(x)
-    return _cached_plan(shape, "idct_idxst", batch, x.device).inverse(x, out)
+    return _cached_plan("idct_idxst", 2, x).inverse(x, out)
 
 
 def idxst_idct(x, out=None):
     """IDXST along axis 0 and IDCT along axis 1."""
-    shape, batch = _split(x)
-    return _cached_plan(shape, "idxst_idct", batch, x.device).inverse(x, out)
+    return _cached_plan("idxst_idct", 2, x).inverse(x, out)
 
 
 def dct2_noalloc(x, out=None, stream=None):

@@ -205,15 +205,18 @@ struct DeviceGuard {
 // True when kernels on `device` may dereference `ptr`: this device's memory,
 // managed memory, page-locked host memory mapped at the same address (read
 // and written over the host link by the kernels themselves), or any host
-// memory when the device can access pageable memory.  While `s` is capturing
+// memory when the device can access pageable memory.  While the stream captures
 // a graph the check is skipped (the pointers of a captured launch are the
 // caller's own device buffers, and the query is not needed there).
 // Returns 0 (not accessible), 1 (this device's memory) or 2 (accessible
 // otherwise); *is_dev tells the kernels whether bulk tensor copies may be used.
 enum { PTR_NONE = 0, PTR_DEVICE = 1, PTR_OTHER = 2 };
-int pointer_kind(const void* ptr, int device, cudaStream_t s) {
+bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone) return PTR_DEVICE;
+  return cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
+}
+int pointer_kind(const void* ptr, int device, bool in_capture) {
+  if (in_capture) return PTR_DEVICE;
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
     cudaGetLastError();
@@ -650,7 +653,8 @@ static gbdct_status exec2d(gbdct_plan_t p, const void* in, void* out, void* stre
   if (((uintptr_t)in & 15u) || ((uintptr_t)out & 15u)) return GBDCT_ERR_INVALID_ARG;
   DeviceGuard guard(p->device);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const int kin = pointer_kind(in, p->device, s), kout = pointer_kind(out, p->device, s);
+  const bool cap = capturing(s);
+  const int kin = pointer_kind(in, p->device, cap), kout = pointer_kind(out, p->device, cap);
   if (kin == PTR_NONE || kout == PTR_NONE) return GBDCT_ERR_INVALID_ARG;
   const bool io_dev = kin == PTR_DEVICE && kout == PTR_DEVICE;
   if (p->ndim == 3) return exec3d(p, in, out, s, inverse, step);
@@ -755,9 +759,10 @@ gbdct_status poisson_plan_solve(gbdct_plan_t p, const void* rho, void* const* ou
                                 cudaStream_t s) {
   const void* io[4] = {rho, out[0], out[1], out[2]};
   bool dev[4];
+  const bool cap = capturing(s);
   for (int i = 0; i < 4; ++i) {
     if ((uintptr_t)io[i] & 15u) return GBDCT_ERR_INVALID_ARG;
-    const int k = pointer_kind(io[i], p->device, s);
+    const int k = pointer_kind(io[i], p->device, cap);
     if (k == PTR_NONE) return GBDCT_ERR_INVALID_ARG;
     dev[i] = k == PTR_DEVICE;
   }
