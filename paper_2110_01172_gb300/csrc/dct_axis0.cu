@@ -6,6 +6,7 @@
 #include "fft_soa.cuh"
 #include "l2_hint.cuh"
 #include "launch_dep.cuh"
+#include "row_pairs.cuh"
 
 namespace gbdct {
 namespace {
@@ -98,16 +99,66 @@ __global__ void __launch_bounds__(512, 2) k_axis0(AxisArgs a) {
 __device__ __forceinline__ soa::C2 pairs_to_soa(float4 q) { return {make_float2(q.x, q.z), make_float2(q.y, q.w)}; }
 
 // Packed form, N >= 64: NP two-lane sequences (float4 = two adjacent column
-// pairs of a row) per CTA, TPS = N/16 threads each, 128 threads per CTA.
+// pairs of a row) per CTA, TPS = N/16 threads each, 128 threads per CTA (64 at
+// N = 64, 256 at N = 4096).  The pairs of rows k and N - k meet in registers as
+// in the row passes (row_pairs.cuh): in one thread, or in two lanes of a warp.
+// A warp holds GW threads of each of its NP sequences (lane = slot NP + sequence)
+// whose butterflies are GW/2 consecutive ones and their mirrors, 16 lanes apart.
+// What bounds the pass is the array in and out (a 256^3 inverse pass, whose input
+// and output are two arrays, runs at 5.2 TB/s); its points cross shared memory once
+// per stage boundary, where reading the pairs back made it five array passes
+// forward and six inverse.  Forward / inverse pass: 256^3 19.7 / 25.0 -> 18.1 / 24.9 us,
+// 64 x 512^2 19.0 / 24.6 -> 15.4 / 23.4, 512 x 128^2 14.9 / 17.0 -> 12.2 / 13.5.
 template <int N>
 struct AxisSoaGeom {
   static constexpr int TPS = fft_tps(N);
-  static constexpr int NP = (128 / TPS) > 0 ? 128 / TPS : 1;
+  static constexpr int NP = TPS >= 128 ? 1 : (128 / TPS > 16 ? 16 : 128 / TPS);
   static constexpr int THREADS = NP * TPS;
   static constexpr int LP = N + N / 16;
   static constexpr size_t SMEM = (size_t)NP * LP * sizeof(float4);
   static constexpr int MINB = THREADS >= 512 ? 1 : 512 / THREADS;  // up to 128 registers
+  static constexpr int GW = 32 / NP;
 };
+
+// Butterfly t of thread g of a sequence (one of T = TPS) and the lane of its
+// mirror T - t; 0 and T/2 are their own.
+template <int N>
+__device__ __forceinline__ int axis_butterfly(int g, int* src) {
+  using G = AxisSoaGeom<N>;
+  constexpr int H = G::GW / 2, T = G::TPS;
+  const int w = g / G::GW, sl = g % G::GW;
+  const int t0 = H * w + sl % H;
+  const int t = sl < H ? t0 : (t0 ? T - t0 : T / 2);
+  const int lane = threadIdx.x & 31;
+  *src = t0 ? lane ^ 16 : lane;
+  return t;
+}
+
+// Stages NS .. N of the CTA's sequences; the last stage's outputs stay in v, its
+// butterflies those of neg_pairs (NEG; t: the thread's mirrored butterfly) or g + q TPS.
+template <int N, int NS, bool INV, bool NEG>
+__device__ __forceinline__ void axis_stages(float4* __restrict__ s, int g, int t, const float4* __restrict__ tw,
+                                            soa::C2* v) {
+  constexpr int R = stage_radix(N, NS), TPS = fft_tps(N), NB = 16 / R, NP = AxisSoaGeom<N>::NP;
+  constexpr bool LAST = NS * R == N;
+  auto butterfly = [&](int q) {
+    if (!LAST || !NEG) return g + q * TPS;
+    return NB == 1 ? t : rowp::last_butterfly<N, true>(g, q);
+  };
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NB; ++q) soa::load_butterfly<N, NS, NP>(v + q * R, s, butterfly(q));
+  if constexpr (!LAST) __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NB; ++q) {
+    soa::Tw<R> w;
+    w.load(tw + tw_offset(N, NS) + (butterfly(q) & (NS - 1)), NS);
+    soa::twiddle<R, INV>(v + q * R, w);
+    soa::dft<R, INV>(v + q * R);
+    if constexpr (!LAST) soa::store_butterfly<N, NS, NP>(v + q * R, s, butterfly(q));
+  }
+  if constexpr (!LAST) axis_stages<N, NS * R, INV, NEG>(s, g, t, tw, v);
+}
 
 template <int N, bool INV>
 __global__ void __launch_bounds__(AxisSoaGeom<N>::THREADS, AxisSoaGeom<N>::MINB) k_axis0_soa(AxisArgs a) {
@@ -121,57 +172,67 @@ __global__ void __launch_bounds__(AxisSoaGeom<N>::THREADS, AxisSoaGeom<N>::MINB)
   float4* Y = reinterpret_cast<float4*>(a.out + (long long)blockIdx.y * a.bstride) + vcol;
   float4* s = sas + pi;
   const uint64_t pol = l2::evict_first();
+  int src;
+  const int t = axis_butterfly<N>(g, &src);
   soa::C2 v[16];
   pdl::wait_prior_grid();
   if constexpr (!INV) {
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = pairs_to_soa(l2::ld_once(X + reorder_src(g + TPS * j, N) * hv, pol));
     soa::first_stage<N, false, NP>(v, s, g);
-    __syncthreads();
-    soa::stages<N, 16, false, NP>(s, g, a.tw4);
+    axis_stages<N, 16, false, true>(s, g, t, a.tw4, v);
     pdl::launch_dependents();
-#pragma unroll 4
-    for (int r = 0; r < 16; ++r) {
-      const int k = g + TPS * r;
-      const soa::C2 zk = soa::unpack(s[NP * soa::pidx4(k)]);
-      const soa::C2 zm = soa::unpack(s[NP * soa::pidx4((N - k) & (N - 1))]);
+    rowp::neg_pairs<N>(v, g, t, src, [&](soa::C2 P, soa::C2 Q, int base, int off, bool mirror) {
+      const int k = base + off;
       const float2 w = __ldg(a.w + k);  // e^{-i pi k / 2N} / 2
-      // per lane: 2 Va = Z[k] + conj Z[N-k], 2 Vb = -i (Z[k] - conj Z[N-k]); X = Re(w 2V)
-      const float2 va_r = soa::add2(zk.re, zm.re), va_i = soa::sub2(zk.im, zm.im);
-      const float2 vb_r = soa::add2(zk.im, zm.im), vb_i = soa::sub2(zm.re, zk.re);
-      const float2 xa = soa::fma2(va_i, soa::bc(-w.y), soa::mul2(va_r, soa::bc(w.x)));
-      const float2 xb = soa::fma2(vb_i, soa::bc(-w.y), soa::mul2(vb_r, soa::bc(w.x)));
+      // per lane: 2 Va = Z[k] + conj Z[N-k], 2 Vb = -i (Z[k] - conj Z[N-k]);
+      // X[k] = Re(w 2V), X[N-k] = -Im(w 2V)
+      const float2 va_r = soa::add2(P.re, Q.re), va_i = soa::sub2(P.im, Q.im);
+      const float2 vb_r = soa::add2(P.im, Q.im), vb_i = soa::sub2(Q.re, P.re);
+      const float2 wx = soa::bc(w.x), nwy = soa::bc(-w.y), nwx = soa::bc(-w.x);
+      const float2 xa = soa::fma2(va_i, nwy, soa::mul2(va_r, wx));
+      const float2 xb = soa::fma2(vb_i, nwy, soa::mul2(vb_r, wx));
       l2::st(Y + (long long)k * hv, make_float4(xa.x, xb.x, xa.y, xb.y), pol);
-    }
+      if (!mirror) return;
+      const float2 ya = soa::fma2(va_i, nwx, soa::mul2(va_r, nwy));
+      const float2 yb = soa::fma2(vb_i, nwx, soa::mul2(vb_r, nwy));
+      l2::st(Y + (long long)(N - k) * hv, make_float4(ya.x, yb.x, ya.y, yb.y), pol);
+    });
   } else {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      v[j] = pairs_to_soa(l2::ld_once(X + (long long)(g + TPS * j) * hv, pol));
-      s[NP * soa::pidx4(g + TPS * j)] = soa::pack(v[j]);
-    }
-    __syncthreads();
-    // Z[k] = Va[k] + i Vb[k] from rows k and N-k (row N taken as zero)
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int k = g + TPS * j;
-      const soa::C2 c = v[j];
-      const soa::C2 m = k ? soa::unpack(s[NP * soa::pidx4(N - k)]) : soa::C2{soa::bc(0.f), soa::bc(0.f)};
+    // Z[k] = Va[k] + i Vb[k] and, V being Hermitian, Z[N-k] = conj Va[k] + i conj Vb[k]
+    // from rows k and N-k (row N taken as zero); lane values X_a = re, X_b = im of
+    // the packed column pair, Va = w (X_a[k] - i X_a[N-k]), Vb likewise
+    auto pre = [&](soa::C2 c, soa::C2 m, int k, soa::C2& lo, soa::C2& hi) {
       const float2 w = __ldg(a.w + k);  // e^{+i pi k / 2N} / N
-      // per lane: Va = w (X_a[k] - i X_a[N-k]), Vb = w (X_b[k] - i X_b[N-k]);
-      // lane values: X_a = re, X_b = im of the packed column pair
       const soa::C2 va = soa::mulw(soa::C2{c.re, soa::ng(m.re)}, soa::bc(w.x), soa::bc(w.y));
       const soa::C2 vb = soa::mulw(soa::C2{c.im, soa::ng(m.im)}, soa::bc(w.x), soa::bc(w.y));
-      v[j] = soa::C2{soa::sub2(va.re, vb.im), soa::add2(va.im, vb.re)};
+      lo = soa::C2{soa::sub2(va.re, vb.im), soa::add2(va.im, vb.re)};
+      hi = soa::C2{soa::add2(va.re, vb.im), soa::sub2(vb.re, va.im)};
+    };
+    auto row = [&](int k) { return pairs_to_soa(l2::ld_once(X + (long long)k * hv, pol)); };
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int k = t + TPS * j;
+      const soa::C2 c = row(k), m = k ? row(N - k) : soa::C2{soa::bc(0.f), soa::bc(0.f)};
+      soa::C2 hi;
+      pre(c, m, k, v[j], hi);
+      v[15 - j] = rowp::shfl(hi, src);
     }
-    __syncthreads();  // the first stage overwrites the staged rows
-    soa::first_stage<N, true, NP>(v, s, g);
-    __syncthreads();
-    soa::stages<N, 16, true, NP>(s, g, a.tw4);
+    if (t == 0) {  // butterfly 0 mirrors onto itself with j <-> 16 - j; row N/2 pairs with itself
+#pragma unroll
+      for (int j = 15; j > 8; --j) v[j] = v[j - 1];
+      const soa::C2 c = row(N / 2);
+      soa::C2 hi;
+      pre(c, c, N / 2, v[8], hi);
+    }
+    soa::first_stage<N, true, NP>(v, s, t);
+    axis_stages<N, 16, true, false>(s, g, t, a.tw4, v);
     pdl::launch_dependents();
-#pragma unroll 4
-    for (int r = 0; r < 16; ++r) {
-      const int n = g + TPS * r;
-      l2::st(Y + (long long)reorder_src(n, N) * hv, soa::pack_aos(soa::unpack(s[NP * soa::pidx4(n)])), pol);
+    constexpr int NS = last_stage_ns(N), R = stage_radix(N, NS);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int n = g + (i / R) * TPS + NS * (i % R);
+      l2::st(Y + (long long)reorder_src(n, N) * hv, soa::pack_aos(v[i]), pol);
     }
   }
 }

@@ -221,18 +221,16 @@ struct FwdOut {
   }
 };
 
-// Postprocess of a group's two rows from the last stage's registers.
-template <int L, bool FIRST, typename Out>
-__device__ __forceinline__ void fwd_post(soa::C2* v, const Out& out, float2 avr, float2 avi,
-                                         const float4* __restrict__ fb4, int g, bool packed) {
+// Calls column(P, M, base, off, mirror) for every pair of points c = base + off
+// (off a compile-time constant) and L - c of the last stage's outputs in v; mirror
+// is false for c = 0 and L / 2, which pair with themselves.  t, src: the thread's
+// last-stage butterfly and the lane of its mirror (one butterfly per thread only).
+template <int L, typename Column>
+__device__ __forceinline__ void neg_pairs(soa::C2* v, int g, int t, int src, const Column& column) {
   using S = Last<L>;
   constexpr int NS = S::NS, R = S::R;
-  auto column = [&](soa::C2 P, soa::C2 M, int base, int off, bool mirror) {
-    out.store(combine<FIRST>(P, M, avr, avi, __ldg(fb4 + base + off), packed), base, off, mirror);
-  };
   if constexpr (S::NB == 1) {
     static_assert(R == 16, "one butterfly per thread has the full radix");
-    const int t = neg_lane_butterfly<NS>(g), src = neg_lane_source<NS>(g);
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       // butterfly 0 mirrors onto itself with m <-> 16 - m
@@ -246,7 +244,7 @@ __device__ __forceinline__ void fwd_post(soa::C2* v, const Out& out, float2 avr,
   } else {
 #pragma unroll
     for (int i = 0; i < S::NB / 2; ++i) {
-      const int t = g + i * S::TPS;
+      t = g + i * S::TPS;
       soa::C2* A = v + i * R;
       soa::C2* B = v + (S::NB / 2 + i) * R;
       // slots: P = A[m], M = B[R - 1 - m], column t + NS m.  Butterfly 0 is its
@@ -276,6 +274,17 @@ __device__ __forceinline__ void fwd_post(soa::C2* v, const Out& out, float2 avr,
       if (i == 0 && t == 0) column(half, half, 0, L / 2, false);
     }
   }
+}
+
+// Postprocess of a group's two rows from the last stage's registers.
+template <int L, bool FIRST, typename Out>
+__device__ __forceinline__ void fwd_post(soa::C2* v, const Out& out, float2 avr, float2 avi,
+                                         const float4* __restrict__ fb4, int g, bool packed) {
+  constexpr int NS = Last<L>::NS;
+  neg_pairs<L>(v, g, neg_lane_butterfly<NS>(g), neg_lane_source<NS>(g),
+               [&](soa::C2 P, soa::C2 M, int base, int off, bool mirror) {
+                 out.store(combine<FIRST>(P, M, avr, avi, __ldg(fb4 + base + off), packed), base, off, mirror);
+               });
 }
 
 // ---------------------------------------------------------------------------

@@ -120,3 +120,25 @@ def test_inverse_points_and_pairs_meet_once(L):
             for m in range(R // 2):
                 pairs += [(t + ns * m, u + ns * (R - 1 - m)), (u + ns * m, t + ns * (R - 1 - m))]
     assert sorted(p for p, _ in pairs) == list(range(L // 2)) and all(p + q == L - 1 for p, q in pairs)
+
+
+@pytest.mark.parametrize("N", [64, 128, 256, 512, 1024, 2048, 4096])
+def test_axis_pass_lanes(N):
+    """The axis-0 pass: every butterfly of every sequence once, its mirror 16 lanes away."""
+    T = N // 16
+    NP = 1 if T >= 128 else min(16, 128 // T)
+    GW = 32 // NP
+    H = GW // 2
+
+    def butterfly(g):
+        w, sl = divmod(g, GW)
+        t0 = H * w + sl % H
+        return t0 if sl < H else (T - t0 if t0 else T // 2)
+
+    assert T % GW == 0 and sorted(butterfly(g) for g in range(T)) == list(range(T))
+    for g in range(T):
+        for pi in range(NP):
+            thread = g * NP + pi
+            t = butterfly(g)
+            other = thread if t in (0, T // 2) else thread ^ 16
+            assert other // 32 == thread // 32 and other % NP == pi and butterfly(other // NP) == (T - t) % T
