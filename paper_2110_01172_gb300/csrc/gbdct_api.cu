@@ -599,7 +599,8 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   } else if (p->family == FAM_FS2) {
     e = gbdct::run_fs2(p->lg1, p->lg2, false, a, 1, 0, true);
   } else if (p->family == FAM_TP) {
-    e = gbdct::run_tp(p->lg1, p->lg2, false, a, 1, 0, true);
+    // every batch size that calls run: the plan's, or one spectrum and its three inverses
+    e = gbdct::run_tp(p->lg1, p->lg2, false, a, poisson ? 1 : (int)batch, 0, true);
     if (e == cudaSuccess && p->host_fs2) e = gbdct::run_fs2(p->lg1, p->lg2, false, a, 1, 0, true);
     if (e == cudaSuccess && poisson) e = gbdct::run_tp_poisson(p->lg1, p->lg2, a, gbdct::PoissonArgs{}, 0, true);
   } else if (p->family == FAM_PAIR) {
@@ -882,6 +883,13 @@ gbdct_status gbdct_plan_set_threshold(gbdct_plan_t plan, float eps) {
   if (!plan || !(eps >= 0.f)) return GBDCT_ERR_INVALID_ARG;
   const bool supported = plan->family == FAM_FS2 || plan->family == FAM_TP;
   if (plan->ndim != 2 || !supported || plan->n2 > 8192) return GBDCT_ERR_UNSUPPORTED;
+  gbdct::Dct2dArgs a = plan->args;
+  a.thresh = eps;
+  DeviceGuard guard(plan->device);
+  cudaError_t e = cudaSuccess;  // the kernels of the other forward variant
+  if (plan->family == FAM_TP && !plan->one_launch)
+    e = gbdct::run_tp_rows_fwd(plan->lg2, a, (int)plan->batch, 0, true);
+  if (e != cudaSuccess) return cuda_status(e);
   plan->args.thresh = eps;
   return GBDCT_OK;
 }

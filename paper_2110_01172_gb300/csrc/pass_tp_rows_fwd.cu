@@ -14,19 +14,13 @@ cudaError_t launch_k(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare
   return pdl::launch(k, dim3(a.n1 / 4 / R::NP, 1, batch), dim3(R::THREADS), R::SMEM, s, a);
 }
 
+// `prepare` readies the variant that a call with the same arguments runs.
 template <int L>
 cudaError_t launch(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
-  if (prepare) {
-    cudaError_t e = launch_k<L, false, false>(a, batch, s, true);
-    if (e == cudaSuccess) e = launch_k<L, false, true>(a, batch, s, true);
-    if (e == cudaSuccess) e = launch_k<L, true, false>(a, batch, s, true);
-    if (e == cudaSuccess) e = launch_k<L, true, true>(a, batch, s, true);
-    return e;
-  }
   const bool general = a.vkind == 1 || a.thresh > 0.f;
   if (tp_rows_narrow<L>(a, batch))
-    return general ? launch_k<L, true, true>(a, batch, s, false) : launch_k<L, true, false>(a, batch, s, false);
-  return general ? launch_k<L, false, true>(a, batch, s, false) : launch_k<L, false, false>(a, batch, s, false);
+    return general ? launch_k<L, true, true>(a, batch, s, prepare) : launch_k<L, true, false>(a, batch, s, prepare);
+  return general ? launch_k<L, false, true>(a, batch, s, prepare) : launch_k<L, false, false>(a, batch, s, prepare);
 }
 
 }  // namespace

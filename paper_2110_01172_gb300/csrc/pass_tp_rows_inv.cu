@@ -31,21 +31,16 @@ cudaError_t launch_m(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare
 
 template <int L, bool NARROW>
 cudaError_t launch_n(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
-  if (prepare) {
-    const cudaError_t e = launch_m<L, NARROW, false>(a, batch, s, true);
-    return e == cudaSuccess ? launch_m<L, NARROW, true>(a, batch, s, true) : e;
-  }
-  return (a.vkind == 1 || a.vkind == 2) ? launch_m<L, NARROW, true>(a, batch, s, false)
-                                        : launch_m<L, NARROW, false>(a, batch, s, false);
+  return (a.vkind == 1 || a.vkind == 2) ? launch_m<L, NARROW, true>(a, batch, s, prepare)
+                                        : launch_m<L, NARROW, false>(a, batch, s, prepare);
 }
 
+// `prepare` readies the kernels that a call with the same arguments may run
+// (device and host-mapped buffers).
 template <int L>
 cudaError_t launch(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
-  if (prepare) {
-    const cudaError_t e = launch_n<L, false>(a, batch, s, true);
-    return e == cudaSuccess ? launch_n<L, true>(a, batch, s, true) : e;
-  }
-  return tp_rows_narrow<L>(a, batch) ? launch_n<L, true>(a, batch, s, false) : launch_n<L, false>(a, batch, s, false);
+  return tp_rows_narrow<L>(a, batch) ? launch_n<L, true>(a, batch, s, prepare)
+                                      : launch_n<L, false>(a, batch, s, prepare);
 }
 
 }  // namespace

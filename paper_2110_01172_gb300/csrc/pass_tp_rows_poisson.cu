@@ -26,11 +26,7 @@ cudaError_t launch_n(const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, 
 
 template <int L>
 cudaError_t launch(const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare) {
-  if (prepare) {
-    const cudaError_t e = launch_n<L, false>(a, ps, s, true);
-    return e == cudaSuccess ? launch_n<L, true>(a, ps, s, true) : e;
-  }
-  return tp_rows_narrow<L>(a, 3) ? launch_n<L, true>(a, ps, s, false) : launch_n<L, false>(a, ps, s, false);
+  return tp_rows_narrow<L>(a, 3) ? launch_n<L, true>(a, ps, s, prepare) : launch_n<L, false>(a, ps, s, prepare);
 }
 
 }  // namespace

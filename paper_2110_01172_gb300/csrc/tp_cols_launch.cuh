@@ -39,6 +39,7 @@ template <int M, int NP, bool INV, bool POIS>
 cudaError_t col_launch_k(const Dct2dArgs& a, const PoissonArgs& ps, int batch, cudaStream_t s, bool prepare) {
   using G = TpColGeom<M, NP>;
   if (prepare) {
+    if (G::SMEM_TMA <= 48 * 1024) return cudaSuccess;  // within the default limit
     cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_tp_cols<M, NP, INV, POIS>),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
     if (e == cudaSuccess)
@@ -95,14 +96,7 @@ cudaError_t col_np(const Dct2dArgs& a, const PoissonArgs& ps, int batch, cudaStr
     }
     return cudaErrorInvalidValue;
   };
-  if (!prepare) return width(strip_np<M>(a, batch));
-  // every width the default or the grid rule can pick
-  for (int np = (a.tpNP ? a.tpNP : tp_default_np(M)); np >= 1; np /= 2) {
-    const cudaError_t e = width(np);
-    if (e != cudaSuccess && e != cudaErrorInvalidValue) return e;
-    if (a.tpNP) break;
-  }
-  return cudaSuccess;
+  return width(strip_np<M>(a, batch));  // prepare: the width that a call with this batch runs
 }
 
 // N1 = 2 M.

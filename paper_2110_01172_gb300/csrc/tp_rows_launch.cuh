@@ -14,7 +14,9 @@ bool tp_rows_narrow(const Dct2dArgs& a, int batch) {
   return wide_ctas < 2LL * (a.nsm > 0 ? a.nsm : 1) && (a.n1 / 4) % TpRows<L, true>::NP == 0;
 }
 
+// Raises a kernel's dynamic shared-memory limit where it needs more than the default.
 inline cudaError_t tp_smem_limit(const void* kernel, size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
