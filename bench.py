@@ -143,8 +143,9 @@ def measured_peaks():
 # Files that define the timed kernels of the default family (the ncu traffic in
 # TRAFFIC is valid only while these are unchanged).
 KERNEL_SOURCES = ("dct2d_tp_kernels.cuh", "dct2d_fs2_kernels.cuh", "dct2d_kernels.cuh", "dct2d_launch.cuh",
-                  "fft_core.cuh", "fft_soa.cuh", "l2_hint.cuh", "tma_util.cuh", "launch_dep.cuh",
-                  "pass_tp_cols.cu", "pass_tp_rows.cu")
+                  "fft_core.cuh", "fft_soa.cuh", "l2_hint.cuh", "tma_util.cuh", "launch_dep.cuh", "row_pairs.cuh",
+                  "tp_cols_launch.cuh", "tp_rows_launch.cuh", "pass_tp.cu", "pass_tp_cols_fwd.cu",
+                  "pass_tp_cols_inv.cu", "pass_tp_rows_fwd.cu", "pass_tp_rows_inv.cu")
 
 
 def sources_digest() -> str:
