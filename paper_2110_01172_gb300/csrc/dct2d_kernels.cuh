@@ -68,6 +68,9 @@ struct Dct2dArgs {
   uint32_t polls;     // bound of device-side waits in polls (0: the default)
   int io_dev;         // host side only: input and output are device memory (bulk tensor copies allowed)
   int nsm;            // host side only: multiprocessors of the device
+  long long l2;       // host side only: bytes of L2
+  int stream_work;    // two-pass workspace written evict-first (batches of plans larger than L2)
+  int ahead;          // row groups ahead whose rows a CTA sends for into L2 (0: none; fs2 forward rows)
 };
 
 // The three inverse transforms of a spectral Poisson solve (Section V-B,

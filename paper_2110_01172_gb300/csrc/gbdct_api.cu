@@ -10,6 +10,7 @@
 #include "dct2d_launch.cuh"
 #include "dct_axis0.cuh"
 #include "gemm_path.cuh"
+#include "multi_path.cuh"
 #include "poisson_path.cuh"
 
 using gbdct::Dct2dArgs;
@@ -564,6 +565,8 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
     return cuda_status(e);
   }
 
+  int l2_bytes = 0;
+  cudaDeviceGetAttribute(&l2_bytes, cudaDevAttrL2CacheSize, p->device);
   Dct2dArgs& a = p->args;
   a.n1 = n1;
   a.n2 = n2;
@@ -589,6 +592,7 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   a.tpNP = (two_pass && tp_np_ok) ? strip_np : 0;  // strip width of the column pass (0: default)
   a.vkind = folds_maps(p) ? kind : 0;
   a.nsm = p->nsm;
+  a.l2 = l2_bytes;
   p->b_cols = gbdct::choose_seq_per_cta(n1, n2 / 2);
   p->b_rows = gbdct::choose_seq_per_cta(n2, n1 / 2);
 
@@ -751,6 +755,8 @@ static gbdct_status exec_core(gbdct_plan_t p, const void* in, void* out, cudaStr
 }  // extern "C"
 
 namespace gbdct {
+
+void plan_stream_work(gbdct_plan_t p) { p->args.stream_work = 1; }
 
 gbdct_status poisson_plan_create(gbdct_plan_t* out, const int64_t* dims) {
   return create_impl(out, 2, dims, 3, GBDCT_DCT2, GBDCT_F32, nullptr, true);

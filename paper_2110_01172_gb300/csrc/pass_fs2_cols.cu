@@ -14,8 +14,7 @@ cudaError_t col_launch(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepa
     return cudaFuncSetAttribute(reinterpret_cast<const void*>(k_fs2_colv<N1, A, KIND>),
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
   }
-  k_fs2_colv<N1, A, KIND><<<dim3(nslab, a.n2 / 2 / C::COLS, batch), C::THREADS, C::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return pdl::launch(k_fs2_colv<N1, A, KIND>, dim3(nslab, a.n2 / 2 / C::COLS, batch), dim3(C::THREADS), C::SMEM, s, a);
 }
 
 template <int N1, int A>

@@ -25,15 +25,14 @@ cudaError_t row_launch(bool inverse, const Dct2dArgs& a, int batch, cudaStream_t
       return e;
     }
     const dim3 grid(a.n1 / 4 / R::NP, 1, batch);
+    const dim3 block(R::THREADS);
     if (inverse && (a.vkind == 1 || a.vkind == 2))
-      k_fs2_rows_inv_x2<L, true><<<grid, R::THREADS, R::SMEM, s>>>(a);
-    else if (inverse)
-      k_fs2_rows_inv_x2<L, false><<<grid, R::THREADS, R::SMEM, s>>>(a);
-    else if (a.vkind == 1 || a.thresh > 0.f)
-      k_fs2_rows_fwd_x2<L, true><<<grid, R::THREADS, R::SMEM, s>>>(a);
-    else
-      k_fs2_rows_fwd_x2<L, false><<<grid, R::THREADS, R::SMEM, s>>>(a);
-    return cudaGetLastError();
+      return pdl::launch(k_fs2_rows_inv_x2<L, true>, grid, block, R::SMEM, s, a);
+    if (inverse) return pdl::launch(k_fs2_rows_inv_x2<L, false>, grid, block, R::SMEM, s, a);
+    Dct2dArgs b = a;
+    b.ahead = L == 8192 && (long long)batch * a.n1 * a.n2 * 4 > a.l2 ? a.nsm : 0;
+    if (a.vkind == 1 || a.thresh > 0.f) return pdl::launch(k_fs2_rows_fwd_x2<L, true>, grid, block, R::SMEM, s, b);
+    return pdl::launch(k_fs2_rows_fwd_x2<L, false>, grid, block, R::SMEM, s, b);
   } else {
     using R = RowGeom<L>;
     if (prepare) {

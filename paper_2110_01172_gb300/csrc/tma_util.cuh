@@ -101,6 +101,11 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
       : "memory");
 }
 
+// Sends for `bytes` (a multiple of 16, 16-byte aligned) into L2 without waiting.
+__device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 // Tiled tensor stores from shared memory (bulk-group completion).
 __device__ __forceinline__ void store_3d(const CUtensorMap* map, const void* src, int x, int y, int z, uint64_t pol) {
   asm volatile(
