@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
   soa::stages<M, 16, INV, G::NP>(s, g, a.tw1x);
   pdl::launch_dependents();
   if constexpr (!INV) {
-    const uint64_t pol_keep = l2::evict_last();  // read again by the row pass
+    const uint64_t pol_keep = l2::work_policy(a.stream_work);  // read again by the row pass
 #pragma unroll 4
     for (int r = 0; r < 16; ++r) {
       const int k = g + TPS * r;
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
   pdl::launch_dependents();
   if (threadIdx.x == 0) {
     if constexpr (!INV) {
-      const uint64_t pol = l2::evict_last();  // read again by the row pass
+      const uint64_t pol = l2::work_policy(a.stream_work);  // read again by the row pass
       for (int z = 0; z < M; z += ZB) tma::store_3d(&mw, buf + z * NP, x0, par * M + z, b, pol);
     } else {
       const uint64_t pol = l2::evict_first();
@@ -358,7 +358,7 @@ __device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a
   float2* e2r = Zw + kb * stride;
   float2* o2r = Zw + (M + kb) * stride;
   const float2 cw = __ldg(a.r2w + c);
-  const uint64_t pol = l2::evict_last();  // read again by the column pass
+  const uint64_t pol = l2::work_policy(a.stream_work);  // read again by the column pass
   rowp::inv_pairs<L>(v, g, [&](int base, int off, const soa::C2& u, const soa::C2& w) {
     const float2 zb0 = make_float2(u.re.y - w.im.y, u.im.y + w.re.y);  // V[kb]
     const float2 zb1 = make_float2(u.re.y + w.im.y, w.re.y - u.im.y);  // V[mirror of kb]

@@ -29,6 +29,10 @@ __device__ __forceinline__ uint64_t evict_last() {
   return p;
 }
 
+// The intermediate array's stores: evict last, or first where the launches of
+// several plans share L2 (Dct2dArgs::stream_work).
+__device__ __forceinline__ uint64_t work_policy(bool stream) { return stream ? evict_first() : evict_last(); }
+
 __device__ __forceinline__ float ld(const float* a, uint64_t pol) {
   float v;
   asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(pol));
