@@ -167,8 +167,8 @@ int gbdct_plan_launches_per_exec(gbdct_plan_t plan);
  * GBDCT_KERNEL_FAMILY=seq|pair|fs2|tp, read at plan creation, forces a family
  * when it supports the shape (for testing and comparison).  Default plans of
  * small shapes (both sides from 32, N1*N2 <= 16384; 128 x 128 for larger
- * batches) run each transform in one launch and without a workspace, under
- * their family's name. */
+ * batches) run each transform in one launch and without a workspace, and larger
+ * ones with a side of 64 the two-pass launches, under their family's name. */
 const char* gbdct_plan_kernel_family(gbdct_plan_t plan);
 
 /* Reports (and clears) a failure recorded on the device by the plan's

@@ -143,9 +143,11 @@ gbdct_status gbdct_plan_create_tuned(gbdct_plan_t* out, int ndim, const int64_t*
       family_out[family_cap - 1] = 0;
     }
   };
-  // A cached name that is the default plan's own means that plan, which for a
-  // small shape runs one launch (a plan of the named family would not).
-  const bool small = ndim == 2 && dims[0] > 0 && dims[1] > 0 && dims[0] <= 16384 && dims[0] * dims[1] <= 16384;
+  // A cached name that is the default plan's own means that plan: with at most
+  // 16384 values or a side of 64 it runs other kernels than a plan that asks for
+  // the named family.
+  const bool small = ndim == 2 && dims[0] > 0 && dims[1] > 0 && dims[0] <= 16384 && dims[1] <= 16384 &&
+                     (dims[0] * dims[1] <= 16384 || dims[0] == 64 || dims[1] == 64);
   if (!cached.empty() && small) {
     gbdct_plan_t p = nullptr;
     if (gbdct_plan_create_batched(&p, ndim, dims, batch, kind, dtype) == GBDCT_OK) {
