@@ -283,7 +283,8 @@ struct TpRows {
   static constexpr int THREADS = NP * TPS;
   static constexpr int LP = L + L / 16;
   static constexpr size_t SMEM = (size_t)NP * LP * sizeof(float4);
-  static constexpr size_t SMEM_STAGED = SMEM + (size_t)NP * 8 + 16;
+  static constexpr size_t SMEM_STAGED = SMEM + (((size_t)NP * 8 + 16 + 15) & ~size_t(15));
+  static constexpr size_t SMEM_DEN = SMEM_STAGED + (size_t)NP * 16 * L;  // + a Poisson solve's denominators
   static constexpr int MINB = THREADS >= 512 ? 1 : 512 / THREADS;  // up to 128 registers
 };
 
@@ -393,52 +394,74 @@ __device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a
 // staged vs direct: 25 x 512^2 22.3 vs 20.6 us, 64 x 256^2 13.9 vs 13.5, 1024^2
 // 8.9 vs 8.6, 2048^2 17.5 vs 17.3, but 4096^2 62.3 vs 63.3).  A Poisson solve,
 // which also loads a denominator for every value, stages at every length (512^2
-// 19.8 vs 21.0 us).
+// 19.8 vs 21.0 us per call).
 template <int L>
 constexpr bool tp_inv_staged() { return L >= 4096; }
 
-// The scaled reads of a Poisson solve: RowReads' value times the eigenvalue
-// denominator and (entry 1) the row's wu or (entry 2) the column's wv.
-template <bool STAGED>
+// The scaled reads of entry Z of a Poisson solve: RowReads' value times the
+// eigenvalue denominator and (entry 1) the row's wu or (entry 2) the column's wv.
+// DEN: the denominators' rows are in shared memory, `den` floats behind the
+// values' rows.
+template <bool STAGED, bool DEN, int Z>
 struct PoissonReads {
   RowReads<STAGED> r;
   const float *ia, *ib;  // the denominators of the two rows
-  const float* wv;       // entry 2 only
-  float ua, ub;          // wu of the two rows (entry 1), else 1
+  const float* wv;       // entry 2
+  float ua, ub;          // entry 1: wu of the two rows
   __device__ __forceinline__ PoissonReads(const RowReads<STAGED>& reads, const InvRows& src, const float* spectrum,
-                                          const PoissonArgs& ps, int n1, int L, int z)
+                                          const PoissonArgs& ps, int n1, int L, int den)
       : r(reads), ia(src.ra ? ps.inv + (src.ra - spectrum) : nullptr), ib(ps.inv + (src.rb - spectrum)),
-        wv(z == 2 ? ps.w + n1 : nullptr), ua(1.f), ub(1.f) {
-    if (z == 1) {
+        wv(ps.w + n1), ua(1.f), ub(1.f) {
+    if constexpr (Z == 1) {
       if (src.ra) ua = __ldg(ps.w + (src.ra - spectrum) / L);
       ub = __ldg(ps.w + (src.rb - spectrum) / L);
     }
+    if constexpr (DEN) {
+      ia = src.ra ? reads.r.ra + den : nullptr;
+      ib = reads.r.rb + den;
+    }
   }
   __device__ __forceinline__ bool has_a() const { return ia != nullptr; }
-  __device__ __forceinline__ float a(int c) const {
-    return r.a(c) * __ldg(ia + c) * (wv ? __ldg(wv + c) : ua);
+  __device__ __forceinline__ float scaled(float v, const float* i, int c, float u) const {
+    v *= DEN ? i[c] : __ldg(i + c);
+    if constexpr (Z == 1) v *= u;
+    if constexpr (Z == 2) v *= __ldg(wv + c);
+    return v;
   }
-  __device__ __forceinline__ float b(int c) const {
-    return r.b(c) * __ldg(ib + c) * (wv ? __ldg(wv + c) : ub);
-  }
+  __device__ __forceinline__ float a(int c) const { return scaled(r.a(c), ia, c, ua); }
+  __device__ __forceinline__ float b(int c) const { return scaled(r.b(c), ib, c, ub); }
 };
 
-// Preprocess of a group from its rows' reads (POIS: scaled).
-template <int L, bool MAPPED, bool POIS, bool STAGED>
-__device__ __forceinline__ int tp_inv_pre(const Dct2dArgs& a, const PoissonArgs& ps, const RowReads<STAGED>& A,
-                                          const RowReads<STAGED>& B, const InvRows& srcA, const InvRows& srcB,
-                                          const float* C, int vkind, int c, int kb, bool first, int g, soa::C2* v) {
-  auto pre = [&](const auto& ra, const auto& rb) {
-    return rowp::warp_has_first<fft_tps(L)>(first)
-               ? inv_pre_x2<L, MAPPED, true>(a, ra, rb, vkind, c, kb, first, g, v)
-               : inv_pre_x2<L, MAPPED, false>(a, ra, rb, vkind, c, kb, false, g, v);
+// Whether a Poisson solve's staged rows take the denominators' rows with them:
+// in narrow CTAs, whose solves are bound by latency (the copies leave while the
+// forward transform finishes; with each entry's kind and factors as constants,
+// GPU time of a solve 256^2 18.5 -> 15.7 us, 512^2 18.3 -> 16.9, 1024^2 25.7 ->
+// 24.0); wide ones would be left with one CTA per SM.
+template <int L, bool NARROW>
+constexpr bool tp_den_staged() { return NARROW && L <= 2048; }
+
+// Preprocess of a group from its rows' reads.
+template <int L, bool MAPPED, typename Reads>
+__device__ __forceinline__ int tp_inv_pre(const Dct2dArgs& a, const Reads& A, const Reads& B, int vkind, int c, int kb,
+                                          bool first, int g, soa::C2* v) {
+  return rowp::warp_has_first<fft_tps(L)>(first) ? inv_pre_x2<L, MAPPED, true>(a, A, B, vkind, c, kb, first, g, v)
+                                                 : inv_pre_x2<L, MAPPED, false>(a, A, B, vkind, c, kb, false, g, v);
+}
+
+// The same for a Poisson solve: its entries' kinds and factors as constants.
+template <int L, bool STAGED, bool DEN>
+__device__ __forceinline__ int tp_poisson_pre(const Dct2dArgs& a, const PoissonArgs& ps, const RowReads<STAGED>& A,
+                                              const RowReads<STAGED>& B, const InvRows& srcA, const InvRows& srcB,
+                                              const float* C, int den, int c, int kb, bool first, int g, soa::C2* v) {
+  auto pre = [&](auto zc) {
+    constexpr int Z = decltype(zc)::value;
+    return tp_inv_pre<L, Z == 2>(a, PoissonReads<STAGED, DEN, Z>(A, srcA, C, ps, a.n1, L, den),
+                                 PoissonReads<STAGED, DEN, Z>(B, srcB, C, ps, a.n1, L, den), poisson_vkind(Z), c, kb,
+                                 first, g, v);
   };
-  if constexpr (POIS) {
-    const int z = blockIdx.z;
-    return pre(PoissonReads<STAGED>(A, srcA, C, ps, a.n1, L, z), PoissonReads<STAGED>(B, srcB, C, ps, a.n1, L, z));
-  } else {
-    return pre(A, B);
-  }
+  return blockIdx.z == 0   ? pre(std::integral_constant<int, 0>{})
+         : blockIdx.z == 1 ? pre(std::integral_constant<int, 1>{})
+                           : pre(std::integral_constant<int, 2>{});
 }
 
 // POIS: blockIdx.z counts the three inverses of a Poisson solve, which read the
@@ -464,19 +487,34 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
     uint64_t* bar = reinterpret_cast<uint64_t*>(sxti + R::NP * R::LP) + pi;
     int* flag = reinterpret_cast<int*>(reinterpret_cast<uint64_t*>(sxti + R::NP * R::LP) + R::NP);
     float* st = reinterpret_cast<float*>(s);
+    constexpr bool DEN = POIS && tp_den_staged<L, NARROW>();
+    // the denominators' rows, behind the barriers and the flag
+    float* dst = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(sxti) + R::SMEM_STAGED) + pi * 4 * L;
     if (threadIdx.x == 0) *flag = 1;
     if (g == 0) {
       tma::bar_init(bar, 1);
       tma::fence_barrier_init();
     }
-    pdl::wait_prior_grid();
+    if constexpr (!DEN) pdl::wait_prior_grid();
     __syncthreads();
+    const float* src[4] = {A.ra, A.rb, B.ra, B.rb};  // rb rows are never null
     if (g == 0) {
-      const float* src[4] = {A.ra, A.rb, B.ra, B.rb};  // rb rows are never null
       uint32_t bytes = 0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) bytes += src[i] ? L * (uint32_t)sizeof(float) : 0u;
+      for (int i = 0; i < 4; ++i) bytes += src[i] ? (DEN ? 2 : 1) * L * (uint32_t)sizeof(float) : 0u;
       tma::bar_expect_tx(bar, bytes);
+    }
+    if constexpr (DEN) {
+      // a table of the solver: sent for while the forward transform finishes
+      if (g == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (src[i])
+            tma::bulk_load(dst + i * L, ps.inv + (src[i] - C), L * (uint32_t)sizeof(float), bar, l2::evict_last());
+      }
+      pdl::wait_prior_grid();
+    }
+    if (g == 0) {
       const uint64_t pol = l2::evict_first();  // the input is streamed in
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -492,13 +530,19 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
     if (!*flag) return;
     tma::test_wait(bar, 0);  // completed: every thread observes the copied rows
     const RowReads<true> As{{A.ra ? st : nullptr, st + L}, 0}, Bs{{B.ra ? st + 2 * L : nullptr, st + 3 * L}, 0};
-    t = tp_inv_pre<L, MAPPED, POIS>(a, ps, As, Bs, A, B, C, vkind, c, kb, first, g, v);
+    if constexpr (POIS)
+      t = tp_poisson_pre<L, true, DEN>(a, ps, As, Bs, A, B, C, (int)(dst - st), c, kb, first, g, v);
+    else
+      t = tp_inv_pre<L, MAPPED>(a, As, Bs, vkind, c, kb, first, g, v);
     rowp::group_sync<R::TPS>(pi);  // the first stage overwrites the staged rows
   } else {
     pdl::wait_prior_grid();
     const uint64_t pol = l2::evict_first();  // the input is streamed in
-    t = tp_inv_pre<L, MAPPED, POIS>(a, ps, RowReads<false>{A, pol}, RowReads<false>{B, pol}, A, B, C, vkind, c, kb,
-                                    first, g, v);
+    const RowReads<false> Ag{A, pol}, Bg{B, pol};
+    if constexpr (POIS)
+      t = tp_poisson_pre<L, false, false>(a, ps, Ag, Bg, A, B, C, 0, c, kb, first, g, v);
+    else
+      t = tp_inv_pre<L, MAPPED>(a, Ag, Bg, vkind, c, kb, first, g, v);
   }
   soa::first_stage<L, true>(v, s, t);
   rowp::stages_to_regs<L, 16, true, false>(s, g, pi, a.tw2x, v);

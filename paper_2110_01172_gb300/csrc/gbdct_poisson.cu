@@ -13,8 +13,8 @@
 // launches and by too few CTAs per launch (512^2: 128 per inverse), large ones
 // by the array passes; separate transforms take nine launches (13 with a side
 // of 64, whose default family is not folded) and the scaling seven more passes
-// over the array.  GPU time per solve, separate -> fused: 64^2 48.5 -> 17.0 us,
-// 64 x 2048 62.5 -> 17.6, 512^2 32.7 -> 18.0, 1024^2 41.4 -> 25.3, 2048^2 92.7 -> 74.7.
+// over the array.  GPU time per solve, separate -> fused: 64^2 48.5 -> 15.8 us,
+// 64 x 2048 62.5 -> 16.1, 512^2 32.7 -> 16.9, 1024^2 41.4 -> 24.0, 2048^2 92.7 -> 74.1.
 // Other shapes run the library's own plans around one scaling kernel.
 // The eigenvalue denominators 1 / (wu^2 + wv^2) are evaluated in FP64 once,
 // when the solver is created, and rounded once into an FP32 table that every

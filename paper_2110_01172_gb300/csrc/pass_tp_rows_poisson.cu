@@ -8,7 +8,7 @@ namespace {
 template <int L, bool NARROW, bool MAPPED, bool STAGED>
 cudaError_t launch_k(const Dct2dArgs& a, const PoissonArgs& ps, int batch, cudaStream_t s, bool prepare) {
   using R = TpRows<L, NARROW>;
-  constexpr size_t SMEM = STAGED ? R::SMEM_STAGED : R::SMEM;
+  constexpr size_t SMEM = !STAGED ? R::SMEM : tp_den_staged<L, NARROW>() ? R::SMEM_DEN : R::SMEM_STAGED;
   const auto k = k_tp_rows_inv<L, MAPPED, STAGED, NARROW, true>;
   if (prepare) return tp_smem_limit(reinterpret_cast<const void*>(k), SMEM);
   if ((a.n1 / 4) % R::NP) return cudaErrorInvalidValue;
