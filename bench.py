@@ -50,10 +50,10 @@ FALLBACK_HBM_GBS = 6800.0
 # launches, so the workspace stays in L2 as it does here).  Valid only for the
 # kernel sources with this digest; otherwise reported as null.
 TRAFFIC = {
-    "sources_sha256": "c65eb368e1eeb8a80a7c5d1a9a03d361187dc9ab315b758b1b4701972b81dc6d",
+    "sources_sha256": "5fb873179485872c29c9a19aab0e2b700e5d23236e86beb6e7f6d406c5b9849b",
     "family": "tp",
-    "forward_bytes": 162805504,
-    "inverse_bytes": 153853184,
+    "forward_bytes": 157930240,
+    "inverse_bytes": 151274496,
 }
 
 
