@@ -545,7 +545,8 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
     return cuda_status(e);
   }
 
-  if (tot1 > 0) k_gen_stage_twiddles<<<(tot1 + 255) / 256, 256>>>(tw1, n1, p->pmax, tot1);
+  // length-N1 stage twiddles: the pair and seq kernels only
+  if (tot1 > 0 && !two_item_rows) k_gen_stage_twiddles<<<(tot1 + 255) / 256, 256>>>(tw1, n1, p->pmax, tot1);
   if (tot2 > 0) k_gen_stage_twiddles<<<(tot2 + 255) / 256, 256>>>(tw2, n2, p->pmax, tot2);
   const int nt = (n1 / 2 + 1 > n2) ? (n1 / 2 + 1) : n2;
   k_gen_dct_tables<<<(nt + 255) / 256, 256>>>(fa, fb, ia, ib, n1, n2);

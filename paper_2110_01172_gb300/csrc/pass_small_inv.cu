@@ -12,6 +12,7 @@ cudaError_t launch(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) 
   } else {
     using G = SmallGeom<LG1, LG2>;
     const auto k = k_small<LG1, LG2, true>;
+    if (prepare && G::SMEM <= 48 * 1024) return cudaSuccess;  // within the default limit
     if (prepare)
       return cudaFuncSetAttribute(reinterpret_cast<const void*>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)G::SMEM);
