@@ -9,10 +9,10 @@
  * mirror image: the four-reads/two-writes twiddle preprocess (Eq. 2d_idct_pre),
  * a complex-to-real 2D FFT and the inverse reorder (Eq. 2d_idct_post).  The
  * reorder and the twiddle stages are fused into the first and last FFT passes,
- * so a 2D transform is two or three kernel launches (by kernel family; three
- * for the default four-step family) around one L2-resident intermediate.  The
- * same plans cover batches, 3D (Section III-D), the DST-II / IDXST kinds of
- * Section V-B, uneven-size batches, the spectral Poisson solve of Algorithm 4
+ * so a 2D transform is one to three kernel launches (one for small transforms,
+ * two by default, three for the four-step family), with the intermediate kept in
+ * L2.  The same plans cover batches, 3D (Section III-D), the DST-II / IDXST kinds
+ * of Section V-B, uneven-size batches, the spectral Poisson solve of Algorithm 4
  * and a split-BF16 tensor-core precision mode.
  *
  * Conventions (all arrays are dense, row-major, last axis contiguous):
