@@ -165,14 +165,19 @@ bool map2d(CUtensorMap* m, const void* base, long long rows, long long cols, int
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// One product: A (map pair a) times the side's matrices, rows x cols outputs for
-// each of the two parities in blockIdx.z.
+// The largest grid that a plan can ask for: 65535 transforms, sides of kGemmMaxSide.
+static_assert(tc::tile_grid(65535LL * kGemmMaxSide, kGemmMaxSide / 2, 64) <= 0x7fffffffLL, "tiles fit the grid's x axis");
+
+// One product: A (map pair a) times the side's matrices, rows x cols outputs (cols /
+// BN a power of two) for each of the two parities in blockIdx.z.
 template <int BN>
-cudaError_t launch(const CUtensorMap (&a)[2], const CUtensorMap (&b)[2][2], const tc::Epi& e, int rows, int cols,
-                   int kdim, uint32_t polls, int* err, cudaStream_t s) {
+cudaError_t launch(const CUtensorMap (&a)[2], const CUtensorMap (&b)[2][2], tc::Epi e, int rows, int cols, int kdim,
+                   uint32_t polls, int* err, cudaStream_t s) {
   using Cf = tc::Cfg<BN>;
   const CUtensorMap(&m)[2] = b[BN == 128 ? 0 : 1];
-  const dim3 grid((unsigned)(cols / BN), (unsigned)(rows / tc::BM), 2);
+  e.lg_cols = 0;
+  while ((BN << e.lg_cols) < cols) ++e.lg_cols;
+  const dim3 grid((unsigned)tc::tile_grid(rows, cols, BN), 1, 2);
   return pdl::launch(tc::k_tc_dftgemm<BN>, grid, dim3(128), (size_t)Cf::SMEM, s, a[0], a[1], m[0], m[1], e,
                      kdim / tc::BK, polls, err);
 }
@@ -252,7 +257,7 @@ gbdct_status gemm_exec(GemmPath* g, bool inverse, const float* in, float* out, c
   cudaError_t ce = inverse ? pdl::launch(k_split<true>, blocks, dim3(256), 0, s, in, g->xh, g->xl, n1, n2, batch)
                            : pdl::launch(k_split<false>, blocks, dim3(256), 0, s, in, g->xh, g->xl, n1, n2, batch);
   // first product, along axis 1 (rows (b, p1, i1), for each parity p2)
-  const tc::Epi e1{tc::EPI_SPLIT_T, n1, n2, batch, batch * n1, h2, inverse ? n2 : 0, g->th, g->tl, nullptr};
+  const tc::Epi e1{tc::EPI_SPLIT_T, n1, n2, batch, batch * n1, h2, inverse ? n2 : 0, 0, g->th, g->tl, nullptr};
   if (ce == cudaSuccess)
     ce = wide_tiles((long long)batch * n1, h2, g->nsm)
              ? launch<128>(g->xa, g->m2, e1, batch * n1, h2, h2, g->polls, g->err, s)
@@ -260,7 +265,7 @@ gbdct_status gemm_exec(GemmPath* g, bool inverse, const float* in, float* out, c
   // second product, along axis 0 (rows (b, p2, j2), for each parity p1); the
   // inverse's quadrants reuse the split input's memory
   float* y = reinterpret_cast<float*>(g->xh);
-  const tc::Epi e2{inverse ? tc::EPI_QUADRANT : tc::EPI_DCT, n1, n2, batch, batch * n2, h1, inverse ? n1 : 0, nullptr,
+  const tc::Epi e2{inverse ? tc::EPI_QUADRANT : tc::EPI_DCT, n1, n2, batch, batch * n2, h1, inverse ? n1 : 0, 0, nullptr,
                    nullptr, inverse ? y : out};
   if (ce == cudaSuccess)
     ce = wide_tiles((long long)batch * n2, h1, g->nsm)

@@ -61,10 +61,15 @@ struct Epi {
   int n1, n2, batch;        // transform sides, transforms
   int a_rows, b_rows;       // operand row offsets per blockIdx.z
   int b_base;               // first operand row of B
+  int lg_cols;              // log2 of the column tiles
   __nv_bfloat16* th;        // EPI_SPLIT_T outputs
   __nv_bfloat16* tl;
   float* out;               // EPI_DCT / EPI_QUADRANT output
 };
+
+// Tiles of one parity.  All of them are in the grid's x axis: batch * N2 / 128 row
+// tiles exceed the 65535 of y and z from a batch of 4096 transforms of 128 x 2048 on.
+constexpr long long tile_grid(long long rows, long long cols, int bn) { return rows / BM * (cols / bn); }
 
 // Shared-memory matrix descriptor of a K-major bf16 tile with the 128-byte
 // swizzle: 8-row groups of 128-byte rows, 1024 bytes apart.
@@ -109,7 +114,8 @@ k_tc_dftgemm(const __grid_constant__ CUtensorMap mah, const __grid_constant__ CU
   uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
   int* fail = reinterpret_cast<int*>(tslot + 1);
   const int warp = threadIdx.x / 32;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  // blockIdx.x: column tiles fastest, then row tiles (tile_grid)
+  const int m0 = (int)(blockIdx.x >> e.lg_cols) * BM, n0 = (int)(blockIdx.x & ((1u << e.lg_cols) - 1)) * BN;
   const int z = (int)blockIdx.z;
   const int arow = e.a_rows * z + m0;
   const int brow = e.b_base + e.b_rows * z + n0;
