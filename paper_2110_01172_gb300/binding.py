@@ -425,6 +425,49 @@ class PoissonSolver:
 
 
 _plans: dict = {}
+_plans_lock = threading.Lock()
+
+
+class _StreamOrder:
+    """Orders the calls that share one cached plan, whose workspace holds the
+    intermediate array of one call: a call on another stream than the last one's
+    waits, on the device, for that stream.
+
+    The event is recorded when the stream changes, not after every call: between two
+    calls on one stream it would keep their launches from overlapping.  Only a stream
+    that PyTorch does not own (its id is its handle) may be gone by then, so there it
+    follows each call.  A call under capture is ordered where its graph is replayed.
+    """
+
+    def __init__(self, device):
+        self.lock = threading.Lock()
+        self.device = device
+        self.handle = self.stream = self.event = None   # of the last call; the event follows it
+        self.foreign = False
+
+    def switch(self, handle):
+        """Before a call on the current stream, `handle`, after one on another stream."""
+        torch = _torch()
+        with torch.cuda.device(self.device):
+            if torch.cuda.is_current_stream_capturing():
+                return
+            stream = torch.cuda.current_stream()
+            if self.stream is not None:
+                if self.foreign or self.record():
+                    stream.wait_event(self.event)
+            self.handle, self.stream = handle, stream
+            self.foreign = handle != 0 and stream.stream_id == handle
+            if self.event is None:
+                self.event = torch.cuda.Event()
+
+    def record(self):
+        """The event behind the last call's stream (not on one that another thread captures)."""
+        torch = _torch()
+        with torch.cuda.stream(self.stream):
+            if torch.cuda.is_current_stream_capturing():
+                return False
+            self.event.record()
+            return True
 
 
 def _cached_plan(kind, ndim, x):
@@ -436,49 +479,80 @@ def _cached_plan(kind, ndim, x):
             raise ValueError("expected a 3D tensor")
         if ndim == 2 and x.dim() not in (2, 3):
             raise ValueError("expected a 2D tensor or a batch of 2D tensors")
-        p = _plans[key] = Plan(tuple(x.shape[-ndim:]), kind, int(x.shape[0]) if x.dim() > ndim else 1, x.device)
+        with _plans_lock:
+            p = _plans.get(key)
+            if p is None:
+                p = Plan(tuple(x.shape[-ndim:]), kind, int(x.shape[0]) if x.dim() > ndim else 1, x.device)
+                p.order = _StreamOrder(p.device) if p.workspace_bytes else None
+                _plans[key] = p
     return p
 
 
+def _one_call(kind, ndim, inverse, x, out):
+    """The current stream's transform of x by the cached plan."""
+    p = _cached_plan(kind, ndim, x)
+    order = p.order
+    if order is None:  # nothing that two calls would share
+        return p.inverse(x, out) if inverse else p.forward(x, out)
+    with order.lock:
+        handle = _stream_handle(None, p.device)
+        if handle != order.handle:
+            order.switch(handle)
+        x, out = p._prep(x, out)
+        run = p._lib.gbdct_exec_inverse if inverse else p._lib.gbdct_exec_forward
+        status = run(p._h, x.data_ptr(), out.data_ptr(), handle)
+        if status != OK:
+            raise GbdctError(status, "gbdct_exec_inverse" if inverse else "gbdct_exec_forward")
+        if order.foreign:
+            order.record()
+    return out
+
+
 def dct2(x, out=None):
-    """2D DCT-II (unnormalised) of a CUDA float32 (N1, N2) or (B, N1, N2) tensor."""
-    return _cached_plan("dct2", 2, x).forward(x, out)
+    """2D DCT-II (unnormalised) of a CUDA float32 (N1, N2) or (B, N1, N2) tensor.
+
+    The one-call functions run on the current stream with a plan kept for the shape.
+    Calls on different streams and threads take turns on the device where the plan
+    has a workspace; replays of a graph that captured such a call are the caller's
+    to order with other calls of the shape.
+    """
+    return _one_call("dct2", 2, False, x, out)
 
 
 def idct2(x, out=None):
     """Exact inverse of ``dct2`` (2/N-scaled DCT-III per axis)."""
-    return _cached_plan("dct2", 2, x).inverse(x, out)
+    return _one_call("dct2", 2, True, x, out)
 
 
 def dct3(x, out=None):
     """3D DCT-II (unnormalised, the 1D DCT-II along every axis) of a CUDA float32
     (N0, N1, N2) tensor."""
-    return _cached_plan("dct2", 3, x).forward(x, out)
+    return _one_call("dct2", 3, False, x, out)
 
 
 def idct3(x, out=None):
     """Exact inverse of ``dct3``."""
-    return _cached_plan("dct2", 3, x).inverse(x, out)
+    return _one_call("dct2", 3, True, x, out)
 
 
 def dst2(x, out=None):
     """2D DST-II (unnormalised sine analogue of ``dct2``)."""
-    return _cached_plan("dst2", 2, x).forward(x, out)
+    return _one_call("dst2", 2, False, x, out)
 
 
 def idst2(x, out=None):
     """Exact inverse of ``dst2``."""
-    return _cached_plan("dst2", 2, x).inverse(x, out)
+    return _one_call("dst2", 2, True, x, out)
 
 
 def idct_idxst(x, out=None):
     """IDCT along axis 0 and IDXST along axis 1 (2/N-scaled, like ``idct2``)."""
-    return _cached_plan("idct_idxst", 2, x).inverse(x, out)
+    return _one_call("idct_idxst", 2, True, x, out)
 
 
 def idxst_idct(x, out=None):
     """IDXST along axis 0 and IDCT along axis 1."""
-    return _cached_plan("idxst_idct", 2, x).inverse(x, out)
+    return _one_call("idxst_idct", 2, True, x, out)
 
 
 def dct2_noalloc(x, out=None, stream=None):
