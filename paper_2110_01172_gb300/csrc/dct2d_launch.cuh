@@ -107,11 +107,13 @@ cudaError_t launch_pair(void (*kern)(Dct2dArgs), const Dct2dArgs& a, int npairs,
 template <int L>
 cudaError_t launch_pass(void (*kern)(Dct2dArgs), const Dct2dArgs& a, dim3 grid, cudaStream_t s,
                         bool prepare) {
-  const size_t smem = seq_smem_bytes(L, a.seq_per_cta);
   if (prepare) {
-    return cudaFuncSetAttribute(reinterpret_cast<const void*>(kern),
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the most that any plan asks of this kernel: the limit belongs to the kernel, and
+    // a plan with fewer sequences per CTA must not lower it for the others
+    return cudaFuncSetAttribute(reinterpret_cast<const void*>(kern), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)seq_smem_bytes(L, choose_seq_per_cta(L, 1 << (kMaxLog2 - 1))));
   }
+  const size_t smem = seq_smem_bytes(L, a.seq_per_cta);
   kern<<<grid, seq_threads(L, a.seq_per_cta), smem, s>>>(a);
   return cudaGetLastError();
 }
