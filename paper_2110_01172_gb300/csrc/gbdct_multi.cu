@@ -143,12 +143,10 @@ gbdct_status gbdct_plan_create_tuned(gbdct_plan_t* out, int ndim, const int64_t*
       family_out[family_cap - 1] = 0;
     }
   };
-  // A cached name that is the default plan's own means that plan: with at most
-  // 16384 values or a side of 64 it runs other kernels than a plan that asks for
-  // the named family.
-  const bool small = ndim == 2 && dims[0] > 0 && dims[1] > 0 && dims[0] <= 16384 && dims[1] <= 16384 &&
-                     (dims[0] * dims[1] <= 16384 || dims[0] == 64 || dims[1] == 64);
-  if (!cached.empty() && small) {
+  // A cached name that is the default plan's own means that plan, which may run other
+  // kernels than a plan that asks for the name (small transforms and sides of 64, also
+  // as the slices of a volume).  A name with a parameter ("tp/4") is never a default's.
+  if (!cached.empty() && cached.find('/') == std::string::npos) {
     gbdct_plan_t p = nullptr;
     if (gbdct_plan_create_batched(&p, ndim, dims, batch, kind, dtype) == GBDCT_OK) {
       if (cached == gbdct_plan_kernel_family(p)) {
@@ -181,10 +179,13 @@ gbdct_status gbdct_plan_create_tuned(gbdct_plan_t* out, int ndim, const int64_t*
     gbdct_plan_destroy(best);
     return cuda_err(e);
   }
-  std::string best_fam = gbdct_plan_kernel_family(best);
+  // The default plan goes by its family's name, so a plan that asks for that name is
+  // not a candidate of its own.
+  const std::string default_fam = gbdct_plan_kernel_family(best);
+  std::string best_fam = default_fam;
   double best_us = time_plan(best, kind, a, b, s);
   for (const char* fam : kFamilies) {
-    if (best_fam == fam) continue;
+    if (default_fam == fam) continue;
     gbdct_plan_t p = nullptr;
     if (gbdct_plan_create_family(&p, ndim, dims, batch, kind, dtype, fam) != GBDCT_OK) continue;
     const double us = time_plan(p, kind, a, b, s);
