@@ -137,8 +137,8 @@ gbdct_status gbdct_exec_forward(gbdct_plan_t plan, const void* in, void* out, vo
 gbdct_status gbdct_exec_inverse(gbdct_plan_t plan, const void* in, void* out, void* stream);
 
 /*
- * Diagnostic: runs launch `step` (0 <= step < gbdct_plan_launches_per_exec) of
- * the forward (inverse = 0) or inverse (inverse = 1) sequence alone, reading
+ * Diagnostic: runs launch `step` (0 <= step < gbdct_plan_launches) of the
+ * forward (inverse = 0) or inverse (inverse = 1) sequence alone, reading
  * and writing the same buffers the full call would.  Used to time each kernel
  * of a transform on its own stream; the result of a single step is an
  * intermediate, not a transform.  Errors: INVALID_ARG (NULL plan, step out of
@@ -155,7 +155,12 @@ const char* gbdct_plan_step_name(gbdct_plan_t plan, int inverse, int step);
  * counted. */
 size_t gbdct_plan_workspace_bytes(gbdct_plan_t plan);
 
-/* Number of kernel launches one exec call issues (0 for a NULL plan). */
+/* Number of kernel launches one forward (inverse = 0) or inverse (1) call issues
+ * (0 for a NULL plan). */
+int gbdct_plan_launches(gbdct_plan_t plan, int inverse);
+
+/* The launches of a forward call.  An inverse call issues as many, except in the
+ * split-BF16 mode, where it issues one more (gbdct_plan_launches). */
 int gbdct_plan_launches_per_exec(gbdct_plan_t plan);
 
 /* Name of the kernel family the plan runs ("seq", "pair", "fs2" or "tp"; ""

@@ -71,6 +71,7 @@ def load(path: str | None = None, build_if_missing: bool = True) -> ctypes.CDLL:
             "gbdct_exec_forward": (ctypes.c_int, [plan_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
             "gbdct_exec_inverse": (ctypes.c_int, [plan_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
             "gbdct_plan_workspace_bytes": (ctypes.c_size_t, [plan_p]),
+            "gbdct_plan_launches": (ctypes.c_int, [plan_p, ctypes.c_int]),
             "gbdct_plan_launches_per_exec": (ctypes.c_int, [plan_p]),
             "gbdct_plan_kernel_family": (ctypes.c_char_p, [plan_p]),
             "gbdct_plan_check_device_error": (ctypes.c_int, [plan_p]),
@@ -207,8 +208,13 @@ class Plan:
     def family(self) -> str:
         return self._lib.gbdct_plan_kernel_family(self._h).decode()
 
+    def launches(self, inverse: bool) -> int:
+        """Kernel launches of one forward or inverse call."""
+        return int(self._lib.gbdct_plan_launches(self._h, int(bool(inverse))))
+
     @property
     def launches_per_exec(self) -> int:
+        """Kernel launches of one forward call (an inverse one differs in the split-BF16 mode only)."""
         return int(self._lib.gbdct_plan_launches_per_exec(self._h))
 
     def _prep(self, x, out):

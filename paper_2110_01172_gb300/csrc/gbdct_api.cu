@@ -812,7 +812,7 @@ gbdct_status gbdct_exec_inverse(gbdct_plan_t plan, const void* in, void* out, vo
 }
 
 gbdct_status gbdct_exec_step(gbdct_plan_t plan, int inverse, int step, const void* in, void* out, void* stream) {
-  if (!plan || step < 0 || step >= gbdct_plan_launches_per_exec(plan)) return GBDCT_ERR_INVALID_ARG;
+  if (!plan || step < 0 || step >= gbdct_plan_launches(plan, inverse)) return GBDCT_ERR_INVALID_ARG;
   return exec2d(plan, in, out, stream, inverse != 0, step);
 }
 
@@ -878,13 +878,15 @@ gbdct_status gbdct_plan_set_precision(gbdct_plan_t plan, int precision) {
   return GBDCT_OK;
 }
 
-int gbdct_plan_launches_per_exec(gbdct_plan_t plan) {
+int gbdct_plan_launches(gbdct_plan_t plan, int inverse) {
   if (!plan) return 0;
-  if (plan->precision == GBDCT_PREC_SPLIT_BF16) return 3;  // split + two tensor-core products (+ mirror sums, inverse)
-  if (plan->ndim == 3) return gbdct_plan_launches_per_exec(plan->inner) + 1;
+  if (plan->precision == GBDCT_PREC_SPLIT_BF16) return inverse ? 4 : 3;  // split, two products (, mirror sums)
+  if (plan->ndim == 3) return gbdct_plan_launches(plan->inner, inverse) + 1;
   const int core = core_launches(plan);
   return (plan->kind == GBDCT_DCT2 || folds_maps(plan)) ? core : core + 2;
 }
+
+int gbdct_plan_launches_per_exec(gbdct_plan_t plan) { return gbdct_plan_launches(plan, 0); }
 
 const char* gbdct_plan_kernel_family(gbdct_plan_t plan) {
   if (!plan) return "";
