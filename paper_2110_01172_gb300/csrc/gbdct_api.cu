@@ -817,9 +817,9 @@ gbdct_status gbdct_exec_step(gbdct_plan_t plan, int inverse, int step, const voi
 }
 
 const char* gbdct_plan_step_name(gbdct_plan_t plan, int inverse, int step) {
-  if (!plan || step < 0 || step >= gbdct_plan_launches_per_exec(plan)) return "";
+  if (!plan || step < 0 || step >= gbdct_plan_launches(plan, inverse)) return "";
   if (plan->ndim == 3) {
-    const int ni = gbdct_plan_launches_per_exec(plan->inner);
+    const int ni = gbdct_plan_launches(plan->inner, inverse);
     if (!inverse) return step < ni ? gbdct_plan_step_name(plan->inner, 0, step)
                                    : "axis-0 pass (reorder + column FFT + split + twiddle)";
     return step == 0 ? "axis-0 pass (twiddle + column IFFT + inverse reorder)"
@@ -837,12 +837,17 @@ const char* gbdct_plan_step_name(gbdct_plan_t plan, int inverse, int step) {
                                 "row pass (split + row FFT + postprocess)"};
   static const char* kInv3[] = {"row pass (preprocess + row IFFT + pairing)", "column step C2' (DFT_A + twiddle)",
                                 "column step C1' (DFT_B + inverse reorder)"};
+  static const char* kFwdSplit[] = {"input split (mirror sums of both axes)", "product along axis 1 (by parity)",
+                                    "product along axis 0 (by parity)"};
+  static const char* kInvSplit[] = {"input split (entries by parity)", "product along axis 1 (by parity)",
+                                    "product along axis 0 (by parity)", "output (mirror sums of both axes)"};
+  if (plan->precision == GBDCT_PREC_SPLIT_BF16) return inverse ? kInvSplit[step] : kFwdSplit[step];
   if (plan->one_launch) return "whole transform (one CTA each)";
   const bool three = core_launches(plan) == 3;
   int k = step;
   if (plan->kind != GBDCT_DCT2 && !folds_maps(plan)) {
     if (k == 0) return "index/sign map (pre)";
-    if (k == gbdct_plan_launches_per_exec(plan) - 1) return "index/sign map (post)";
+    if (k == gbdct_plan_launches(plan, inverse) - 1) return "index/sign map (post)";
     k -= 1;
   }
   if (three) return inverse ? kInv3[k] : kFwd3[k];

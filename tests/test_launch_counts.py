@@ -1,4 +1,5 @@
-"""gbdct_plan_launches against the kernel nodes of a captured call (needs a GB300)."""
+"""gbdct_plan_launches against the kernel nodes of a captured call, and the names
+of a plan's launches (needs a GB300)."""
 
 import ctypes
 
@@ -43,4 +44,6 @@ def test_launches_of_a_call(shape, kind, batch, family, split):
         run = plan.inverse if inverse else plan.forward
         count = captured_nodes(lambda s: run(x, out, stream=s), x, out)
         assert plan.launches(inverse) == count
+        names = [plan.step_name(inverse, k) for k in range(count)]
+        assert all(names) and plan.step_name(inverse, count) == ""
     assert plan.launches_per_exec == plan.launches(False)
