@@ -730,7 +730,7 @@ __device__ __forceinline__ void fwd_split_x2(const float2* __restrict__ za, cons
 // N1-k1 (lane a; rows 0 and N1/2 of the packed item) and kb, N1-kb (lane b) of
 // y, `stride` floats apart.  GENERAL: plans with the DST-II order or a magnitude
 // threshold.
-template <int L, bool GENERAL, bool FIRST, bool SMEM>
+template <int L, bool GENERAL, bool FIRST, bool SMEM, bool EXACT>
 __device__ __forceinline__ void fwd_post_rows(soa::C2* v, const Dct2dArgs& a, float* y, long long stride, int k1,
                                               int kb, bool packed, int g) {
   const int N1 = a.n1;
@@ -748,26 +748,26 @@ __device__ __forceinline__ void fwd_post_rows(soa::C2* v, const Dct2dArgs& a, fl
   out.pol = l2::evict_first();  // the output is streamed out
   out.eps = a.thresh;           // magnitude threshold of Section V-A, Eq. image-compression (0: off)
   out.rev = rev;
-  rowp::fwd_post<L, FIRST>(v, out, avr, avi, a.fb4, g, packed);
+  rowp::fwd_post<L, FIRST, EXACT>(v, out, avr, avi, a.fb4, g, packed);
 }
-template <int L, bool GENERAL, bool SMEM>
+template <int L, bool GENERAL, bool SMEM, bool EXACT>
 __device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, float* y, long long stride, int k1, int kb,
                                             bool packed, int g) {
   if (rowp::warp_has_first<fft_tps(L)>(packed))
-    fwd_post_rows<L, GENERAL, true, SMEM>(v, a, y, stride, k1, kb, packed, g);
+    fwd_post_rows<L, GENERAL, true, SMEM, EXACT>(v, a, y, stride, k1, kb, packed, g);
   else
-    fwd_post_rows<L, GENERAL, false, SMEM>(v, a, y, stride, k1, kb, false, g);
+    fwd_post_rows<L, GENERAL, false, SMEM, EXACT>(v, a, y, stride, k1, kb, false, g);
 }
 
 // Row FFT of both items from registers (v: points t + TPS j of the thread's
 // first-stage butterfly t) and the postprocess.
-template <int L, bool GENERAL>
+template <int L, bool GENERAL, bool EXACT>
 __device__ __forceinline__ void fwd_fft_post_x2(soa::C2* v, float4* s, const Dct2dArgs& a, float* y, int k1, int kb,
                                                 bool packed, int t, int g, int group) {
   soa::first_stage<L, false>(v, s, t);
-  rowp::stages_to_regs<L, 16, false, true>(s, g, group, a.tw2x, v);
+  rowp::stages_to_regs<L, 16, false, true, EXACT>(s, g, group, a.tw2x, v);
   pdl::launch_dependents();
-  fwd_post_x2<L, GENERAL, false>(v, a, y, L, k1, kb, packed, g);
+  fwd_post_x2<L, GENERAL, false, EXACT>(v, a, y, L, k1, kb, packed, g);
 }
 
 template <int L, bool GENERAL>
@@ -800,7 +800,7 @@ __global__ void __launch_bounds__(RowX2Geom<L>::THREADS, RowX2Geom<L>::MINB) k_f
     fwd_split_x2<L>(za, ma, zb, mb, t, packed, v);
   else
     fwd_split_x2<L>(za, ma, zb, mb, t, false, v);
-  fwd_fft_post_x2<L, GENERAL>(v, s, a, a.out + (long long)blockIdx.z * a.out_bstride, k1, k1 + 1, packed, t, g, pi);
+  fwd_fft_post_x2<L, GENERAL, false>(v, s, a, a.out + (long long)blockIdx.z * a.out_bstride, k1, k1 + 1, packed, t, g, pi);
 }
 
 // Inverse four-read preprocess (Eq. 2d_idct_pre, conjugated twiddle, 1/(N1 N2)
@@ -871,7 +871,7 @@ __device__ __forceinline__ rowp::Quad inv_quad(const Reads& r, int k2, int km, b
 }
 
 // Preprocess of both items: points t + TPS j of the returned butterfly t in v.
-template <int L, bool MAPPED, bool FIRST, typename Reads>
+template <int L, bool MAPPED, bool FIRST, bool EXACT, typename Reads>
 __device__ __forceinline__ int inv_pre_x2(const Dct2dArgs& a, const Reads& A, const Reads& B, int vkind, int k1, int kb,
                                           bool packed, int g, soa::C2* v) {
   const bool rev = MAPPED && vkind == 1, swapc = MAPPED && vkind == 2;
@@ -879,7 +879,8 @@ __device__ __forceinline__ int inv_pre_x2(const Dct2dArgs& a, const Reads& A, co
     qa = inv_quad<L, MAPPED, FIRST>(A, k2, km, edge, rev, swapc);
     qb = inv_quad<L, MAPPED, false>(B, k2, km, edge, rev, swapc);
   };
-  return rowp::inv_pre<L, FIRST>(quads, a.ib, __ldg(a.ia + k1), __ldg(a.ia + kb), __ldg(a.ia + a.n1 / 2), packed, g, v);
+  return rowp::inv_pre<L, FIRST, EXACT>(quads, a.ib, a.ib4, __ldg(a.ia + k1), __ldg(a.ia + kb),
+                                        __ldg(a.ia + a.n1 / 2), packed, g, v);
 }
 
 // Inverse pairing of both items: row IFFT u in s -> workspace rows k1 and its
@@ -921,11 +922,11 @@ __global__ void __launch_bounds__(RowX2Geom<L>::THREADS, RowX2Geom<L>::MINB_INV)
   soa::C2 v[16];
   int t;
   if (rowp::warp_has_first<R::TPS>(packed))
-    t = inv_pre_x2<L, MAPPED, true>(a, A, B, a.vkind, k1, k1 + 1, packed, g, v);
+    t = inv_pre_x2<L, MAPPED, true, false>(a, A, B, a.vkind, k1, k1 + 1, packed, g, v);
   else
-    t = inv_pre_x2<L, MAPPED, false>(a, A, B, a.vkind, k1, k1 + 1, false, g, v);
+    t = inv_pre_x2<L, MAPPED, false, false>(a, A, B, a.vkind, k1, k1 + 1, false, g, v);
   soa::first_stage<L, true>(v, s, t);
-  rowp::stages_to_regs<L, 16, true, false>(s, g, pi, a.tw2x, v);
+  rowp::stages_to_regs<L, 16, true, false, false>(s, g, pi, a.tw2x, v);
   pdl::launch_dependents();
   float2* Zw = a.work + (long long)blockIdx.z * a.work_bstride;
   if (rowp::warp_has_first<R::TPS>(packed))

@@ -50,9 +50,10 @@ struct Dct2dArgs {
   const float2* tw2;  // stage twiddles for length N2
   const float2* fa;   // a_k1, k1 in [0, N1/2]
   const float2* fb;   // b_k2 / 2, k2 in [0, N2)
-  const float4* fb4;  // b_k2 / 2 as (br, br, bi, bi) (two-item row passes)
+  const float4* fb4;  // b_k2 / 2 as (br, br, bi, bi) (two-item row passes); exact: (br, bi, rests of br, bi)
   const float2* ia;   // conj(a_k1) / (N1 N2), k1 in [0, N1/2]
   const float2* ib;   // conj(b_k2), k2 in [0, N2)
+  const float4* ib4;  // the same with the rests that its rounding left (exact)
   int seq_per_cta;    // B
   const float2* fstw; // four-step twiddles W_N1^{n1a k1b} (four-step family only)
   int* err;           // device error word: set to 1 by a bounded wait that gave up
@@ -64,14 +65,30 @@ struct Dct2dArgs {
   float thresh;       // forward outputs with |X| < thresh stored as zero (0: off; two-item row passes)
   const float4* tw1x; // stage twiddles for length N1/2 as (wr, wr, wi, wi) (two-pass column passes)
   const float2* r2w;  // W_N1^k = exp(-2 pi i k / N1), k in [0, N1/2] (two-pass family's radix-2 step)
+  const float2* r2r;  // the rests that its rounding left (exact)
   int tpNP;           // strip width of the two-pass column pass in column pairs (0: the default)
   uint32_t polls;     // bound of device-side waits in polls (0: the default)
   int io_dev;         // host side only: input and output are device memory (bulk tensor copies allowed)
   int nsm;            // host side only: multiprocessors of the device
   long long l2;       // host side only: bytes of L2
   int stream_work;    // two-pass workspace written evict-first (batches of plans larger than L2)
+  int exact;          // host side only: every stage twiddle from the table, b_k2 with its rest (row_pairs.cuh)
   int ahead;          // row groups ahead whose rows a CTA sends for into L2 (0: none; fs2 forward rows)
 };
+
+// Shapes whose default kernels are exact (Dct2dArgs::exact): those with a side below
+// 128, which one launch or the two-pass kernels took over from the two-sequence
+// kernels.  The two-lane engine forms odd twiddle powers as products, and the
+// two-pass form multiplies by one twiddle more along axis 0; in transforms this
+// short both show in the result.  Exact kernels read every power from the table and
+// carry what the rounding of b_k2 and of the radix-2 twiddles left.  Forward error
+// against 64 bits (relative L2, 1e-7), two-sequence / products / exact: 64^2 1.32 /
+// 1.38 / 1.31, 32 x 256 1.39 / 1.48 / 1.37, 512 x 64 1.48 / 1.60 / 1.46, 64 x 2048
+// 1.57 / 1.71 / 1.57; a Poisson solve's potential 512 x 64 1.48 / 1.77 / 1.58.  Time,
+// products -> exact: 203 x 64^2 forward / inverse 5.4 / 6.5 -> 5.9 / 6.8 us (two-sequence
+// 12.7 / 15.8), 2048 x 64 7.4 / 8.2 -> 7.8 / 8.4 (14.5 / 16.9).  Larger sides keep the
+// products: they read 4 of 15 twiddles (exact at 4096^2: forward + inverse 12 % slower).
+constexpr bool side_exact(int lg1, int lg2) { return lg1 < 7 || lg2 < 7; }
 
 // The three inverse transforms of a spectral Poisson solve (Section V-B,
 // Algorithm 4) as one batch over one spectrum: entry 0 the potential (DCT-II

@@ -66,8 +66,10 @@ cudaError_t run_tp_cols_fwd(int lg1, const Dct2dArgs& a, int batch, cudaStream_t
 cudaError_t run_tp_cols_inv(int lg1, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
 cudaError_t run_tp_rows_fwd(int lg2, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
 cudaError_t run_tp_rows_inv(int lg2, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
+cudaError_t run_tp_rows_inv_exact(int lg2, const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare);
 cudaError_t run_tp_cols_poisson(int lg1, const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare);
 cudaError_t run_tp_rows_poisson(int lg2, const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare);
+cudaError_t run_tp_rows_poisson_exact(int lg2, const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare);
 // The three inverses of a Poisson solve from the spectrum at a.in (the row pass
 // and the column pass once each, over a workspace of three entries).
 cudaError_t run_tp_poisson(int log2N1, int log2N2, const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s,

@@ -39,6 +39,9 @@ struct SmallGeom {
   static constexpr int BUF = max2(max2(2 * ST * LPM, N1 * WS), max2(N1 * XS, (N1 / 4) * (L + L / 16)));
   static constexpr size_t SMEM = (size_t)NT * BUF * sizeof(float4);
   static constexpr int MINB = 512 / THREADS;    // up to 128 registers
+  static constexpr bool EXACT = side_exact(LG1, LG2);
+  // the radix-2 twiddles' rest: at N1 = 64 alone the other measures do not make up for the step
+  static constexpr bool REST = EXACT && LG1 == 6;
   static_assert(LG1 >= 5 && LG2 >= 5 && LG1 + LG2 <= 14, "sides from 32, at most 16384 values");
 };
 
@@ -51,7 +54,7 @@ __device__ __forceinline__ int small_col_out(int g, int i) {
   if constexpr (M == 16) return i;
   else return g + (i / R) * TPM + 16 * (i % R);
 }
-template <int M, int ST, bool INV>
+template <int M, int ST, bool INV, bool EXACT>
 __device__ __forceinline__ void small_col_fft(soa::C2* v, float4* __restrict__ s, int g,
                                               const float4* __restrict__ tw) {
   if constexpr (M == 16) {
@@ -65,8 +68,9 @@ __device__ __forceinline__ void small_col_fft(soa::C2* v, float4* __restrict__ s
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       soa::Tw<R> w;
-      w.load(tw + tw_offset(M, 16) + g + q * TPM, 16);
-      soa::twiddle<R, INV>(v + q * R, w);
+      const float4* twp = tw + tw_offset(M, 16) + g + q * TPM;
+      w.load(twp, 16);
+      soa::twiddle<R, INV, EXACT>(v + q * R, w, twp, 16);
       soa::dft<R, INV>(v + q * R);
     }
   }
@@ -107,7 +111,7 @@ __global__ void __launch_bounds__(SmallGeom<LG1, LG2>::THREADS, SmallGeom<LG1, L
       }
       v[j] = aos_to_soa(q);
     }
-    small_col_fft<M, ST, false>(v, cs, g, a.tw1x);
+    small_col_fft<M, ST, false, G::EXACT>(v, cs, g, a.tw1x);
     __syncthreads();  // the workspace rows overlay the points
 #pragma unroll
     for (int i = 0; i < 16; ++i) s[(par * M + small_col_out<M>(g, i)) * G::WS + pi] = soa::pack_aos(v[i]);
@@ -115,20 +119,18 @@ __global__ void __launch_bounds__(SmallGeom<LG1, LG2>::THREADS, SmallGeom<LG1, L
     const float2* Zw = reinterpret_cast<const float2*>(s);
     const float2 *e1r = Zw + c * (2 * G::WS), *o1r = Zw + (M + c) * (2 * G::WS);
     const float2 *e2r = Zw + kb * (2 * G::WS), *o2r = Zw + (M + kb) * (2 * G::WS);
-    const float2 w = __ldg(a.r2w + c);
-    const float2 w1 = first ? make_float2(1.f, 0.f) : w;
-    const float2 w2 = first ? __ldg(a.r2w + M / 2) : conjf2(w);
+    const R2<false, G::REST> w(a, c, first);
     const int t = rowp::rev_lane_butterfly<TPL>(gr);
     if (rowp::warp_has_first<TPL>(first))
-      tp_fwd_load<L, true, true>(e1r, o1r, e2r, o2r, w1, w2, first, t, v);
+      tp_fwd_load<L, true, true, G::REST>(e1r, o1r, e2r, o2r, w, first, t, v);
     else
-      tp_fwd_load<L, false, true>(e1r, o1r, e2r, o2r, w1, w2, false, t, v);
+      tp_fwd_load<L, false, true, G::REST>(e1r, o1r, e2r, o2r, w, false, t, v);
     __syncthreads();
     soa::first_stage<L, false>(v, rs, t);
-    rowp::stages_to_regs<L, 16, false, true>(rs, gr, c, a.tw2x, v);
+    rowp::stages_to_regs<L, 16, false, true, G::EXACT>(rs, gr, c, a.tw2x, v);
     pdl::launch_dependents();
     __syncthreads();
-    fwd_post_x2<L, true, true>(v, a, reinterpret_cast<float*>(s), 4 * G::XS, c, kb, first, gr);
+    fwd_post_x2<L, true, true, G::EXACT>(v, a, reinterpret_cast<float*>(s), 4 * G::XS, c, kb, first, gr);
     __syncthreads();
     if (live) {
 #pragma unroll
@@ -148,23 +150,23 @@ __global__ void __launch_bounds__(SmallGeom<LG1, LG2>::THREADS, SmallGeom<LG1, L
     const RowReads<true> A{inv_rows_of(a, C, c, 4 * G::XS, a.vkind), 0}, B{inv_rows_of(a, C, kb, 4 * G::XS, a.vkind), 0};
     int t;
     if (rowp::warp_has_first<TPL>(first))
-      t = inv_pre_x2<L, true, true>(a, A, B, a.vkind, c, kb, first, gr, v);
+      t = inv_pre_x2<L, true, true, G::EXACT>(a, A, B, a.vkind, c, kb, first, gr, v);
     else
-      t = inv_pre_x2<L, true, false>(a, A, B, a.vkind, c, kb, false, gr, v);
+      t = inv_pre_x2<L, true, false, G::EXACT>(a, A, B, a.vkind, c, kb, false, gr, v);
     __syncthreads();
     soa::first_stage<L, true>(v, rs, t);
-    rowp::stages_to_regs<L, 16, true, false>(rs, gr, c, a.tw2x, v);
+    rowp::stages_to_regs<L, 16, true, false, G::EXACT>(rs, gr, c, a.tw2x, v);
     __syncthreads();
     float2* Zw = reinterpret_cast<float2*>(s);
     if (rowp::warp_has_first<TPL>(first))
-      tp_inv_pair<L, true>(v, a, Zw, 2 * G::WS, c, kb, first, gr);
+      tp_inv_pair<L, true, G::REST>(v, a, Zw, 2 * G::WS, c, kb, first, gr);
     else
-      tp_inv_pair<L, true>(v, a, Zw, 2 * G::WS, c, kb, false, gr);
+      tp_inv_pair<L, true, G::REST>(v, a, Zw, 2 * G::WS, c, kb, false, gr);
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = aos_to_soa(s[(par * M + g + TPM * j) * G::WS + pi]);
     __syncthreads();
-    small_col_fft<M, ST, true>(v, cs, g, a.tw1x);
+    small_col_fft<M, ST, true, G::EXACT>(v, cs, g, a.tw1x);
     pdl::launch_dependents();
     if (live) {
 #pragma unroll

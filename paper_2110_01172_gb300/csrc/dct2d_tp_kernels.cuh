@@ -74,7 +74,7 @@ __device__ __forceinline__ float4 soa_to_aos(soa::C2 y) { return make_float4(y.r
 // Forward (INV = false): reorder + E or O (blockIdx.y = parity of the
 // reordered row) -> workspace.  Inverse: E' or O' -> IDFT_M -> output rows
 // with the inverse reorder.
-template <int M, int NP, bool INV, bool POIS>
+template <int M, int NP, bool INV, bool POIS, bool EXACT>
 __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::MINB)
     k_tp_cols(Dct2dArgs a, PoissonArgs ps) {
   using G = TpColGeom<M, NP>;
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
   }
   soa::first_stage<M, INV, G::NP>(v, s, g);
   __syncthreads();
-  soa::stages<M, 16, INV, G::NP>(s, g, a.tw1x);
+  soa::stages<M, 16, INV, G::NP, 0, EXACT>(s, g, a.tw1x);
   pdl::launch_dependents();
   if constexpr (!INV) {
     const uint64_t pol_keep = l2::work_policy(a.stream_work);  // read again by the row pass
@@ -166,7 +166,7 @@ struct ColMaps {
   CUtensorMap w;     // workspace
 };
 
-template <int M, int NP, bool INV, bool POIS>
+template <int M, int NP, bool INV, bool POIS, bool EXACT>
 __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::MINB)
     k_tp_cols_tma(Dct2dArgs a, const __grid_constant__ ColMaps<POIS ? 3 : 1> maps) {
   using G = TpColGeom<M, NP>;
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(TpColGeom<M, NP>::THREADS, TpColGeom<M, NP>::M
   float4* s = buf + pi;
   soa::first_stage<M, INV, NP>(v, s, g);
   __syncthreads();
-  soa::stages<M, 16, INV, NP, INV ? 2 : 1>(s, g, a.tw1x);
+  soa::stages<M, 16, INV, NP, INV ? 2 : 1, EXACT>(s, g, a.tw1x);
   if constexpr (INV) {
     if (vkind) {  // output signs: (-1)^(n1+n2) DST-II, (-1)^n2 IDCT_IDXST, (-1)^n1 IDXST_IDCT
 #pragma unroll 4
@@ -288,12 +288,53 @@ struct TpRows {
   static constexpr int MINB = THREADS >= 512 ? 1 : 512 / THREADS;  // up to 128 registers
 };
 
+// The radix-2 twiddles of a group: forward W_N1^c on O[c] and W_N1^-c on O[kb] (first
+// group: 1 and W_N1^{M/2}), inverse W_N1^-c and -W_N1^c on the differences (1 and i).
+// REST: with the rests that the table's rounding left, both products in one packed
+// multiplication.
+template <bool INV, bool REST>
+struct R2 {
+  float2 w1, w2;       // without rests: the two twiddles (inverse: w1 for both)
+  soa::C2 w, r;        // with rests: lane by lane
+  bool first;
+
+  __device__ __forceinline__ R2(const Dct2dArgs& a, int c, bool f) : first(f) {
+    const int k = !INV && f ? a.n1 / 4 : c;
+    const float2 t = __ldg(a.r2w + k);
+    if constexpr (!REST) {
+      w1 = !INV && f ? make_float2(1.f, 0.f) : t;
+      w2 = f ? t : conjf2(t);
+    } else {
+      const float2 u = __ldg(a.r2r + k);
+      if constexpr (!INV) {
+        w = f ? soa::C2{make_float2(1.f, t.x), make_float2(0.f, t.y)} : soa::C2{soa::bc(t.x), make_float2(t.y, -t.y)};
+        r = f ? soa::C2{make_float2(0.f, u.x), make_float2(0.f, u.y)} : soa::C2{soa::bc(u.x), make_float2(u.y, -u.y)};
+      } else {
+        w = f ? soa::C2{make_float2(1.f, 0.f), make_float2(0.f, 1.f)} : soa::C2{make_float2(t.x, -t.x), soa::bc(-t.y)};
+        r = f ? soa::C2{soa::bc(0.f), soa::bc(0.f)} : soa::C2{make_float2(u.x, -u.x), soa::bc(-u.y)};
+      }
+    }
+  }
+  __device__ __forceinline__ void mul(float2& a, float2& b) const {
+    if constexpr (REST) {
+      const soa::C2 o = soa::mulw(soa::C2{make_float2(a.x, b.x), make_float2(a.y, b.y)}, w.re, w.im, r.re, r.im);
+      a = make_float2(o.re.x, o.im.x);
+      b = make_float2(o.re.y, o.im.y);
+    } else if constexpr (!INV) {
+      a = cmul(a, w1);
+      b = cmul(b, w2);
+    } else {
+      a = first ? a : cmulc(a, w1);
+      b = first ? make_float2(-b.y, b.x) : cmul(make_float2(-b.x, -b.y), w1);
+    }
+  }
+};
+
 // The thread's points of both items in v, straight from the group's four
-// workspace rows (SMEM: in shared memory; w1, w2: the radix-2 twiddles on O[c]
-// and O[kb]).
-template <int L, bool FIRST, bool SMEM = false>
+// workspace rows (SMEM: in shared memory).
+template <int L, bool FIRST, bool SMEM, bool REST>
 __device__ __forceinline__ void tp_fwd_load(const float2* e1r, const float2* o1r, const float2* e2r, const float2* o2r,
-                                            float2 w1, float2 w2, bool first, int t, soa::C2* v) {
+                                            const R2<false, REST>& w, bool first, int t, soa::C2* v) {
   constexpr int TPS = fft_tps(L);
   constexpr int MASK = rowp::rev_lane_mask<TPS>();
   const uint64_t pol = l2::evict_first();  // last use of the workspace
@@ -302,7 +343,8 @@ __device__ __forceinline__ void tp_fwd_load(const float2* e1r, const float2* o1r
   for (int j = 0; j < 8; ++j) {
     const int p = t + TPS * j;
     const float2 e1 = ld(e1r + p), e2 = ld(e2r + p);
-    const float2 o1 = cmul(ld(o1r + p), w1), o2 = cmul(ld(o2r + p), w2);
+    float2 o1 = ld(o1r + p), o2 = ld(o2r + p);
+    w.mul(o1, o2);
     const float2 P = cadd(e1, o1), Q = csub(e1, o1), Rr = cadd(e2, o2), S = csub(e2, o2);
     // (z_a, m_a, z_b, m_b) = (V[c], V[N1-c], V[M-c], V[M+c]); first group:
     // (V[0], V[M], V[M/2], V[3M/2])
@@ -313,7 +355,7 @@ __device__ __forceinline__ void tp_fwd_load(const float2* e1r, const float2* o1r
 }
 
 // GENERAL: plans with the DST-II order or a magnitude threshold (row_pairs.cuh).
-template <int L, bool NARROW, bool GENERAL>
+template <int L, bool NARROW, bool GENERAL, bool EXACT>
 __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>::MINB) k_tp_rows_fwd(Dct2dArgs a) {
   using R = TpRows<L, NARROW>;
   constexpr int TPS = R::TPS;
@@ -329,18 +371,15 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
   const float2* o1r = Zw + (long long)(M + c) * (L / 2);
   const float2* e2r = Zw + (long long)kb * (L / 2);
   const float2* o2r = Zw + (long long)(M + kb) * (L / 2);
-  // radix-2 twiddles on O[c] and O[kb]: W_N1^c and W_N1^{-c}, or 1 and W_N1^{M/2}
-  const float2 w = __ldg(a.r2w + c);
-  const float2 w1 = first ? make_float2(1.f, 0.f) : w;
-  const float2 w2 = first ? __ldg(a.r2w + M / 2) : conjf2(w);
+  const R2<false, EXACT> w(a, c, first);
   const int t = rowp::rev_lane_butterfly<TPS>(g);
   pdl::wait_prior_grid();
   soa::C2 v[16];
   if (rowp::warp_has_first<TPS>(first))
-    tp_fwd_load<L, true>(e1r, o1r, e2r, o2r, w1, w2, first, t, v);
+    tp_fwd_load<L, true, false, EXACT>(e1r, o1r, e2r, o2r, w, first, t, v);
   else
-    tp_fwd_load<L, false>(e1r, o1r, e2r, o2r, w1, w2, false, t, v);
-  fwd_fft_post_x2<L, GENERAL>(v, s, a, a.out + (long long)blockIdx.z * a.out_bstride, c, kb, first, t, g, pi);
+    tp_fwd_load<L, false, false, EXACT>(e1r, o1r, e2r, o2r, w, false, t, v);
+  fwd_fft_post_x2<L, GENERAL, EXACT>(v, s, a, a.out + (long long)blockIdx.z * a.out_bstride, c, kb, first, t, g, pi);
 }
 
 // Inverse pairing of both items into E' / O' rows: from the row IFFT u in v,
@@ -350,7 +389,7 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
 // and for the first group E'[0], O'[0] from V[0] +- V[M], E'[M/2] = V[M/2] +
 // V[3M/2], O'[M/2] = i (V[M/2] - V[3M/2]).
 // Rows of Zw are `stride` complex values apart (SMEM: in shared memory).
-template <int L, bool SMEM>
+template <int L, bool SMEM, bool REST>
 __device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a, float2* Zw, long long stride, int c,
                                             int kb, bool first, int g) {
   const int M = a.n1 / 2;
@@ -358,7 +397,7 @@ __device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a
   float2* o1r = Zw + (M + c) * stride;
   float2* e2r = Zw + kb * stride;
   float2* o2r = Zw + (M + kb) * stride;
-  const float2 cw = __ldg(a.r2w + c);
+  const R2<true, REST> cw(a, c, first);
   const uint64_t pol = l2::work_policy(a.stream_work);  // read again by the column pass
   rowp::inv_pairs<L>(v, g, [&](int base, int off, const soa::C2& u, const soa::C2& w) {
     const float2 zb0 = make_float2(u.re.y - w.im.y, u.im.y + w.re.y);  // V[kb]
@@ -367,10 +406,8 @@ __device__ __forceinline__ void tp_inv_pair(const soa::C2* v, const Dct2dArgs& a
     const float2 za1 = first ? make_float2(u.im.x, w.im.x) : make_float2(u.re.x + w.im.x, w.re.x - u.im.x);
     const float2 x1 = first ? za1 : zb1;  // V[c + M]
     const float2 x2 = first ? zb1 : za1;  // V[kb + M]
-    const float2 d1 = csub(za0, x1);
-    const float2 d2 = csub(zb0, x2);
-    const float2 o1 = first ? d1 : cmulc(d1, cw);
-    const float2 o2 = first ? make_float2(-d2.y, d2.x) : cmul(make_float2(-d2.x, -d2.y), cw);
+    float2 o1 = csub(za0, x1), o2 = csub(zb0, x2);
+    cw.mul(o1, o2);
     auto st = [&](float2* p, float2 z) {
       if constexpr (SMEM)
         *p = z;
@@ -441,21 +478,22 @@ template <int L, bool NARROW>
 constexpr bool tp_den_staged() { return NARROW && L <= 2048; }
 
 // Preprocess of a group from its rows' reads.
-template <int L, bool MAPPED, typename Reads>
+template <int L, bool MAPPED, bool EXACT, typename Reads>
 __device__ __forceinline__ int tp_inv_pre(const Dct2dArgs& a, const Reads& A, const Reads& B, int vkind, int c, int kb,
                                           bool first, int g, soa::C2* v) {
-  return rowp::warp_has_first<fft_tps(L)>(first) ? inv_pre_x2<L, MAPPED, true>(a, A, B, vkind, c, kb, first, g, v)
-                                                 : inv_pre_x2<L, MAPPED, false>(a, A, B, vkind, c, kb, false, g, v);
+  return rowp::warp_has_first<fft_tps(L)>(first)
+             ? inv_pre_x2<L, MAPPED, true, EXACT>(a, A, B, vkind, c, kb, first, g, v)
+             : inv_pre_x2<L, MAPPED, false, EXACT>(a, A, B, vkind, c, kb, false, g, v);
 }
 
 // The same for a Poisson solve: its entries' kinds and factors as constants.
-template <int L, bool STAGED, bool DEN>
+template <int L, bool STAGED, bool DEN, bool EXACT>
 __device__ __forceinline__ int tp_poisson_pre(const Dct2dArgs& a, const PoissonArgs& ps, const RowReads<STAGED>& A,
                                               const RowReads<STAGED>& B, const InvRows& srcA, const InvRows& srcB,
                                               const float* C, int den, int c, int kb, bool first, int g, soa::C2* v) {
   auto pre = [&](auto zc) {
     constexpr int Z = decltype(zc)::value;
-    return tp_inv_pre<L, Z == 2>(a, PoissonReads<STAGED, DEN, Z>(A, srcA, C, ps, a.n1, L, den),
+    return tp_inv_pre<L, Z == 2, EXACT>(a, PoissonReads<STAGED, DEN, Z>(A, srcA, C, ps, a.n1, L, den),
                                  PoissonReads<STAGED, DEN, Z>(B, srcB, C, ps, a.n1, L, den), poisson_vkind(Z), c, kb,
                                  first, g, v);
   };
@@ -467,7 +505,7 @@ __device__ __forceinline__ int tp_poisson_pre(const Dct2dArgs& a, const PoissonA
 // POIS: blockIdx.z counts the three inverses of a Poisson solve, which read the
 // one spectrum; its scaling is applied to the values as they are read (the
 // products rounded in the order a inv, then times wu or wv).
-template <int L, bool MAPPED, bool STAGED, bool NARROW, bool POIS>
+template <int L, bool MAPPED, bool STAGED, bool NARROW, bool POIS, bool EXACT>
 __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>::MINB)
     k_tp_rows_inv(Dct2dArgs a, PoissonArgs ps) {
   using R = TpRows<L, NARROW>;
@@ -531,27 +569,27 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
     tma::test_wait(bar, 0);  // completed: every thread observes the copied rows
     const RowReads<true> As{{A.ra ? st : nullptr, st + L}, 0}, Bs{{B.ra ? st + 2 * L : nullptr, st + 3 * L}, 0};
     if constexpr (POIS)
-      t = tp_poisson_pre<L, true, DEN>(a, ps, As, Bs, A, B, C, (int)(dst - st), c, kb, first, g, v);
+      t = tp_poisson_pre<L, true, DEN, EXACT>(a, ps, As, Bs, A, B, C, (int)(dst - st), c, kb, first, g, v);
     else
-      t = tp_inv_pre<L, MAPPED>(a, As, Bs, vkind, c, kb, first, g, v);
+      t = tp_inv_pre<L, MAPPED, EXACT>(a, As, Bs, vkind, c, kb, first, g, v);
     rowp::group_sync<R::TPS>(pi);  // the first stage overwrites the staged rows
   } else {
     pdl::wait_prior_grid();
     const uint64_t pol = l2::evict_first();  // the input is streamed in
     const RowReads<false> Ag{A, pol}, Bg{B, pol};
     if constexpr (POIS)
-      t = tp_poisson_pre<L, false, false>(a, ps, Ag, Bg, A, B, C, 0, c, kb, first, g, v);
+      t = tp_poisson_pre<L, false, false, EXACT>(a, ps, Ag, Bg, A, B, C, 0, c, kb, first, g, v);
     else
-      t = tp_inv_pre<L, MAPPED>(a, Ag, Bg, vkind, c, kb, first, g, v);
+      t = tp_inv_pre<L, MAPPED, EXACT>(a, Ag, Bg, vkind, c, kb, first, g, v);
   }
   soa::first_stage<L, true>(v, s, t);
-  rowp::stages_to_regs<L, 16, true, false>(s, g, pi, a.tw2x, v);
+  rowp::stages_to_regs<L, 16, true, false, EXACT>(s, g, pi, a.tw2x, v);
   pdl::launch_dependents();
   float2* Zw = a.work + (long long)blockIdx.z * a.work_bstride;
   if (rowp::warp_has_first<R::TPS>(first))
-    tp_inv_pair<L, false>(v, a, Zw, L / 2, c, kb, first, g);
+    tp_inv_pair<L, false, EXACT>(v, a, Zw, L / 2, c, kb, first, g);
   else
-    tp_inv_pair<L, false>(v, a, Zw, L / 2, c, kb, false, g);
+    tp_inv_pair<L, false, EXACT>(v, a, Zw, L / 2, c, kb, false, g);
 }
 
 }  // namespace gbdct

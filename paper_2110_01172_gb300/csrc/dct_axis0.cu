@@ -152,8 +152,9 @@ __device__ __forceinline__ void axis_stages(float4* __restrict__ s, int g, int t
 #pragma unroll
   for (int q = 0; q < NB; ++q) {
     soa::Tw<R> w;
-    w.load(tw + tw_offset(N, NS) + (butterfly(q) & (NS - 1)), NS);
-    soa::twiddle<R, INV>(v + q * R, w);
+    const float4* twp = tw + tw_offset(N, NS) + (butterfly(q) & (NS - 1));
+    w.load(twp, NS);
+    soa::twiddle<R, INV>(v + q * R, w, twp, NS);
     soa::dft<R, INV>(v + q * R);
     if constexpr (!LAST) soa::store_butterfly<N, NS, NP>(v + q * R, s, butterfly(q));
   }

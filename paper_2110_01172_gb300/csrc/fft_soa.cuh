@@ -40,6 +40,11 @@ __device__ __forceinline__ C2 sub(C2 a, C2 b) { return {sub2(a.re, b.re), sub2(a
 __device__ __forceinline__ C2 mulw(C2 a, float2 wr, float2 wi) {
   return {fma2(a.im, ng(wi), mul2(a.re, wr)), fma2(a.im, wr, mul2(a.re, wi))};
 }
+// a * (wr + i wi) with w's rounding made good: (rr, ri) is the rest that it left
+__device__ __forceinline__ C2 mulw(C2 a, float2 wr, float2 wi, float2 rr, float2 ri) {
+  return {fma2(a.im, ng(wi), fma2(a.re, wr, fma2(a.im, ng(ri), mul2(a.re, rr)))),
+          fma2(a.im, wr, fma2(a.re, wi, fma2(a.im, rr, mul2(a.re, ri))))};
+}
 // a * conj(wr + i wi)
 __device__ __forceinline__ C2 mulwc(C2 a, float2 wr, float2 wi) {
   return {fma2(a.im, wi, mul2(a.re, wr)), fma2(a.re, ng(wi), mul2(a.im, wr))};
@@ -169,7 +174,9 @@ __device__ __forceinline__ C2 apply(C2 u, C2 w) {
 // Stage twiddles of one butterfly: the power-of-two powers of w (w, w^2, w^4,
 // w^8 for R = 16), entry (j-1)*NS of twp being w^j.  The other powers are
 // products of at most three of them (a few ulp from the exactly rounded
-// values), which keeps the table reads (and registers) low.
+// values), which keeps the table reads (and registers) low.  EXACT reads them from
+// the table too: for shapes whose transforms are short enough that the products'
+// error shows in the result (row_pairs.cuh).
 template <int R>
 struct Tw {
   static constexpr int N = R == 16 ? 4 : R == 8 ? 3 : R == 4 ? 2 : 1;
@@ -180,10 +187,20 @@ struct Tw {
   }
 };
 
-// u[j] *= w^j (conjugated for the inverse), j = 1 .. R-1.
-template <int R, bool INV>
-__device__ __forceinline__ void twiddle(C2* u, const Tw<R>& t) {
+// u[j] *= w^j (conjugated for the inverse), j = 1 .. R-1; twp, NS: t's own.
+template <int R, bool INV, bool EXACT = false>
+__device__ __forceinline__ void twiddle(C2* u, const Tw<R>& t, const float4* __restrict__ twp, int NS) {
   static_assert(R == 2 || R == 4 || R == 8 || R == 16, "stage radices");
+  if constexpr (EXACT) {
+#pragma unroll
+    for (int j = 1; j < R; ++j)
+      u[j] = apply<INV>(u[j], j == 1   ? t.w[0]
+                              : j == 2 ? t.w[R >= 4 ? 1 : 0]
+                              : j == 4 ? t.w[R >= 8 ? 2 : 0]
+                              : j == 8 ? t.w[R >= 16 ? 3 : 0]
+                                       : ldw(twp + (j - 1) * NS));
+    return;
+  }
   const C2 w1 = t.w[0];
   u[1] = apply<INV>(u[1], w1);
   if constexpr (R >= 4) {
@@ -260,7 +277,7 @@ __device__ __forceinline__ void store_butterfly(const C2* u, float4* __restrict_
 // Stages NS .. L through shared memory (natural order in and out); every
 // thread of the CTA calls this (it contains __syncthreads).  The last stage
 // writes its outputs in the form OUT.
-template <int L, int NS, bool INV, int ST = 1, int OUT = 0>
+template <int L, int NS, bool INV, int ST = 1, int OUT = 0, bool EXACT = false>
 __device__ __forceinline__ void stages(float4* __restrict__ s, int g, const float4* __restrict__ tw) {
   if constexpr (NS < L) {
     constexpr int R = stage_radix(L, NS);
@@ -276,8 +293,9 @@ __device__ __forceinline__ void stages(float4* __restrict__ s, int g, const floa
       const int t = g + q * TPS;
       C2* u = v + q * R;
       Tw<R> w;
-      w.load(tw + tw_offset(L, NS) + (t & (NS - 1)), NS);
-      twiddle<R, INV>(u, w);
+      const float4* twp = tw + tw_offset(L, NS) + (t & (NS - 1));
+      w.load(twp, NS);
+      twiddle<R, INV, EXACT>(u, w, twp, NS);
       dft<R, INV>(u);
       if constexpr (NS * R < L || OUT == 0) {
         store_butterfly<L, NS, ST>(u, s, t);
@@ -294,7 +312,7 @@ __device__ __forceinline__ void stages(float4* __restrict__ s, int g, const floa
       }
     }
     __syncthreads();
-    stages<L, NS * R, INV, ST, OUT>(s, g, tw);
+    stages<L, NS * R, INV, ST, OUT, EXACT>(s, g, tw);
   }
 }
 

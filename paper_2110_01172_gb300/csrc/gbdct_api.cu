@@ -70,13 +70,16 @@ bool folds_maps(const gbdct_plan_s* p) {
 // Plans that run the two-pass launches.
 bool runs_tp(const gbdct_plan_s* p) { return (p->family == FAM_TP || p->tp64) && !p->one_launch; }
 
-// Radix-2 twiddles of the two-pass family: out[k] = W_N1^k, k in [0, N1/2], FP64.
-__global__ void k_gen_r2_twiddles(float2* out, int n1) {
+// Radix-2 twiddles of the two-pass family: out[k] = W_N1^k, k in [0, N1/2], FP64; rest:
+// what their rounding left (may be null).
+__global__ void k_gen_r2_twiddles(float2* out, float2* rest, int n1) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k > n1 / 2) return;
   double sn, cs;
   sincospi(-2.0 * (double)k / (double)n1, &sn, &cs);
-  out[k] = make_float2((float)cs, (float)sn);
+  const float c = (float)cs, s = (float)sn;
+  out[k] = make_float2(c, s);
+  if (rest) rest[k] = make_float2((float)(cs - (double)c), (float)(sn - (double)s));
 }
 
 bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
@@ -140,6 +143,18 @@ __global__ void k_gen_dct_tables(float2* fa, float2* fb, float2* ia, float2* ib,
     fb[idx] = make_float2((float)(0.5 * cs), (float)(-0.5 * sn));
     ib[idx] = make_float2((float)cs, (float)sn);
   }
+}
+
+// The b tables of exact plans: fb4[k] = b_k / 2 and ib4[k] = conj(b_k), each as the
+// FP32 value and the FP32 rest that its rounding left.
+__global__ void k_gen_exact_b(float4* fb4, float4* ib4, int n2) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n2) return;
+  double sn, cs;
+  sincospi((double)k / (2.0 * (double)n2), &sn, &cs);
+  const float c = (float)cs, s = (float)sn, cr = (float)(cs - (double)c), sr = (float)(sn - (double)s);
+  fb4[k] = make_float4(0.5f * c, -0.5f * s, 0.5f * cr, -0.5f * sr);
+  ib4[k] = make_float4(c, s, cr, sr);
 }
 
 // Axis-0 tables of the 3D transform (FP64, k in [0, N)):
@@ -491,6 +506,8 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   // 512 11.5 -> 6.0 us, 2048 x 64 14.8 -> 7.4, 128 x (64 x 2048) 69 -> 50, 8192 x 64 23 -> 15).
   p->tp64 = !fname && !poisson && !p->one_launch && p->family == FAM_PAIR && p->lg1 >= gbdct::kTpPoissonMinLog2 &&
             p->lg1 <= gbdct::kTpMaxLog2N1 && p->lg2 >= gbdct::kTpPoissonMinLog2 && p->lg2 <= gbdct::kTpMaxLog2N2;
+  const bool exact = p->one_launch ? gbdct::side_exact(p->lg1, p->lg2)
+                                   : p->tp64 || (poisson && gbdct::side_exact(p->lg1, p->lg2));
   const bool two_pass = p->family == FAM_TP || p->tp64 || p->one_launch;  // tables of the two-pass kernels
   // a two-pass plan also carries the four-step configuration: full transforms
   // on host-mapped buffers run the four-step kernels, whose first and last
@@ -509,12 +526,13 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   const size_t ta = round_up(n1 / 2 + 1, 2);
   const size_t tb = round_up(n2, 2);
   const size_t tf = four_step ? round_up(n1, 2) : 0;
-  const size_t tx = two_item_rows ? 2 * t2 + 2 * tb : 0;  // float4 copies of the N2 stage twiddles and of b / 2
+  // float4 copies of the N2 stage twiddles and of b / 2; exact: conj(b) with its rest
+  const size_t tx = two_item_rows ? 2 * t2 + (exact ? 4 : 2) * tb : 0;
   // two-pass family: stage twiddles of length N1/2 (float2 and float4 copies)
   // and the radix-2 twiddles W_N1^k
   const int totm = two_pass ? gbdct::tw_size_p(n1 / 2, p->pmax) : 0;
   const size_t tm = two_pass ? round_up(totm + 1, 2) : 0;
-  const size_t tr = two_pass ? round_up(n1 / 2 + 1, 2) : 0;
+  const size_t tr0 = round_up(n1 / 2 + 1, 2), tr = two_pass ? (exact ? 2 : 1) * tr0 : 0;
   p->table_elems = t1 + t2 + 2 * ta + 2 * tb + tf + tx + 3 * tm + tr + 2;  // + 16 bytes for the error word
   cudaError_t e = cudaMalloc(&p->tables, p->table_elems * sizeof(float2));
   if (e != cudaSuccess) {
@@ -530,9 +548,11 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   p->fstw = four_step ? ib + tb : nullptr;
   float4* tw2x = two_item_rows ? reinterpret_cast<float4*>(ib + tb + tf) : nullptr;
   float4* fb4 = two_item_rows ? tw2x + t2 : nullptr;
+  float4* ib4 = exact ? fb4 + tb : nullptr;
   float2* twm = two_pass ? ib + tb + tf + tx : nullptr;
   float4* tw1x = two_pass ? reinterpret_cast<float4*>(ib + tb + tf + tx + tm) : nullptr;
   float2* r2w = two_pass ? ib + tb + tf + tx + 3 * tm : nullptr;
+  float2* r2r = exact ? r2w + tr0 : nullptr;
   p->err = reinterpret_cast<int*>(ib + tb + tf + tx + 3 * tm + tr);
 
   p->work_bytes = p->one_launch ? 0 : (size_t)batch * (size_t)(n1 / 2) * (size_t)n2 * sizeof(float2);
@@ -560,13 +580,16 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   }
   if (p->fstw) k_gen_fs_twiddles<<<(n1 + 255) / 256, 256>>>(p->fstw, n1, fsA, fsB);
   if (tw2x && tot2 > 0) k_expand_twiddles<<<(tot2 + 255) / 256, 256>>>(tw2, tw2x, tot2);
-  if (fb4) k_expand_twiddles<<<(n2 + 255) / 256, 256>>>(fb, fb4, n2);
+  if (exact)
+    k_gen_exact_b<<<(n2 + 255) / 256, 256>>>(fb4, ib4, n2);
+  else if (fb4)
+    k_expand_twiddles<<<(n2 + 255) / 256, 256>>>(fb, fb4, n2);
   if (two_pass) {
     if (totm > 0) {
       k_gen_stage_twiddles<<<(totm + 255) / 256, 256>>>(twm, n1 / 2, p->pmax, totm);
       k_expand_twiddles<<<(totm + 255) / 256, 256>>>(twm, tw1x, totm);
     }
-    k_gen_r2_twiddles<<<(n1 / 2 + 256) / 256, 256>>>(r2w, n1);
+    k_gen_r2_twiddles<<<(n1 / 2 + 256) / 256, 256>>>(r2w, r2r, n1);
   }
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemset(p->err, 0, 16);
@@ -590,11 +613,14 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   a.tw2x = tw2x;
   a.tw1x = tw1x;
   a.r2w = r2w;
+  a.r2r = r2r;
   a.fa = fa;
   a.fb = fb;
   a.fb4 = fb4;
   a.ia = ia;
   a.ib = ib;
+  a.ib4 = ib4;
+  a.exact = exact;
   a.fstw = p->fstw;
   a.err = p->err;
   a.step_filter = -1;

@@ -5,22 +5,34 @@
 namespace gbdct {
 namespace {
 
-template <int L, bool NARROW, bool GENERAL>
+template <int L, bool NARROW, bool GENERAL, bool EXACT>
 cudaError_t launch_k(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
   using R = TpRows<L, NARROW>;
-  const auto k = k_tp_rows_fwd<L, NARROW, GENERAL>;
+  const auto k = k_tp_rows_fwd<L, NARROW, GENERAL, EXACT>;
   if (prepare) return tp_smem_limit(reinterpret_cast<const void*>(k), R::SMEM);
   if ((a.n1 / 4) % R::NP) return cudaErrorInvalidValue;
   return pdl::launch(k, dim3(a.n1 / 4 / R::NP, 1, batch), dim3(R::THREADS), R::SMEM, s, a);
 }
 
+template <int L, bool EXACT>
+cudaError_t launch_e(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
+  const bool general = a.vkind == 1 || a.thresh > 0.f;
+  if (tp_rows_narrow<L>(a, batch))
+    return general ? launch_k<L, true, true, EXACT>(a, batch, s, prepare)
+                   : launch_k<L, true, false, EXACT>(a, batch, s, prepare);
+  return general ? launch_k<L, false, true, EXACT>(a, batch, s, prepare)
+                 : launch_k<L, false, false, EXACT>(a, batch, s, prepare);
+}
+
 // `prepare` readies the variant that a call with the same arguments runs.
 template <int L>
 cudaError_t launch(const Dct2dArgs& a, int batch, cudaStream_t s, bool prepare) {
-  const bool general = a.vkind == 1 || a.thresh > 0.f;
-  if (tp_rows_narrow<L>(a, batch))
-    return general ? launch_k<L, true, true>(a, batch, s, prepare) : launch_k<L, true, false>(a, batch, s, prepare);
-  return general ? launch_k<L, false, true>(a, batch, s, prepare) : launch_k<L, false, false>(a, batch, s, prepare);
+  if (a.exact) return launch_e<L, true>(a, batch, s, prepare);
+  if constexpr (L == 64) {
+    return cudaErrorInvalidValue;  // rows of 64 are always exact
+  } else {
+    return launch_e<L, false>(a, batch, s, prepare);
+  }
 }
 
 }  // namespace

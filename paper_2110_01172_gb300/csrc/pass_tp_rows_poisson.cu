@@ -1,37 +1,19 @@
 // pass_tp_rows_poisson.cu - inverse row pass of a Poisson solve: the three
 // inverses of one spectrum as one batch.
-#include "tp_rows_launch.cuh"
+#include "tp_rows_poisson_launch.cuh"
 
 namespace gbdct {
 namespace {
 
-template <int L, bool NARROW, bool MAPPED, bool STAGED>
-cudaError_t launch_k(const Dct2dArgs& a, const PoissonArgs& ps, int batch, cudaStream_t s, bool prepare) {
-  using R = TpRows<L, NARROW>;
-  constexpr size_t SMEM = !STAGED ? R::SMEM : tp_den_staged<L, NARROW>() ? R::SMEM_DEN : R::SMEM_STAGED;
-  const auto k = k_tp_rows_inv<L, MAPPED, STAGED, NARROW, true>;
-  if (prepare) return tp_smem_limit(reinterpret_cast<const void*>(k), SMEM);
-  if ((a.n1 / 4) % R::NP) return cudaErrorInvalidValue;
-  return pdl::launch(k, dim3(a.n1 / 4 / R::NP, 1, batch), dim3(R::THREADS), SMEM, s, a, ps);
-}
-
-template <int L, bool NARROW>
-cudaError_t launch_n(const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare) {
-  if (prepare) {
-    const cudaError_t e = launch_k<L, NARROW, true, false>(a, ps, 3, s, true);
-    return e == cudaSuccess ? launch_k<L, NARROW, true, true>(a, ps, 3, s, true) : e;
-  }
-  return a.io_dev ? launch_k<L, NARROW, true, true>(a, ps, 3, s, false) : launch_k<L, NARROW, true, false>(a, ps, 3, s, false);
-}
-
 template <int L>
 cudaError_t launch(const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare) {
-  return tp_rows_narrow<L>(a, 3) ? launch_n<L, true>(a, ps, s, prepare) : launch_n<L, false>(a, ps, s, prepare);
+  return launch_e<L, false>(a, ps, s, prepare);
 }
 
 }  // namespace
 
 cudaError_t run_tp_rows_poisson(int lg2, const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s, bool prepare) {
+  if (a.exact) return run_tp_rows_poisson_exact(lg2, a, ps, s, prepare);
   GBDCT_TP_ROWS_SWITCH(lg2, launch, a, ps, s, prepare);
 }
 

@@ -120,7 +120,7 @@ __device__ __forceinline__ int last_butterfly(int g, int q) {
 // v (output m of butterfly q at v[q R + m]).  Called once the thread has written
 // its outputs of the stage before; the barrier that follows is in here, after
 // the loads of the stage's twiddles, so that their latency passes in its wait.
-template <int L, int NS, bool INV, bool NEG>
+template <int L, int NS, bool INV, bool NEG, bool EXACT>
 __device__ __forceinline__ void stages_to_regs(float4* __restrict__ s, int g, int group,
                                                const float4* __restrict__ tw, soa::C2* v) {
   constexpr int R = stage_radix(L, NS);
@@ -140,11 +140,12 @@ __device__ __forceinline__ void stages_to_regs(float4* __restrict__ s, int g, in
   if constexpr (!LAST) group_sync<TPS>(group);
 #pragma unroll
   for (int q = 0; q < NB; ++q) {
-    soa::twiddle<R, INV>(v + q * R, w[q]);
+    const int t = LAST ? last_butterfly<L, NEG>(g, q) : g + q * TPS;
+    soa::twiddle<R, INV, EXACT>(v + q * R, w[q], tw + tw_offset(L, NS) + (t & (NS - 1)), NS);
     soa::dft<R, INV>(v + q * R);
     if constexpr (!LAST) soa::store_butterfly<L, NS, 1>(v + q * R, s, g + q * TPS);
   }
-  if constexpr (!LAST) stages_to_regs<L, NS * R, INV, NEG>(s, g, group, tw, v);
+  if constexpr (!LAST) stages_to_regs<L, NS * R, INV, NEG, EXACT>(s, g, group, tw, v);
 }
 
 // Whether any group of the calling warp is the transform's first one (the
@@ -168,7 +169,8 @@ __device__ __forceinline__ bool warp_has_first(bool first) {
 struct Outs {
   float2 lo0, lo1, hi0, hi1;  // (lane a, lane b): rows k1 and kmir at c, then at L - c
 };
-template <bool FIRST>
+// EXACT: b = (br, bi) and the rests (br, bi) that its rounding left.
+template <bool FIRST, bool EXACT>
 __device__ __forceinline__ Outs combine(soa::C2 P, soa::C2 M, float2 avr, float2 avi, float4 b, bool packed) {
   const soa::C2 aP = soa::mulw(P, avr, avi), aM = soa::mulw(M, avr, avi);
   const float2 ur = soa::add2(aP.re, aM.re), nui = soa::sub2(aM.im, aP.im);
@@ -177,8 +179,16 @@ __device__ __forceinline__ Outs combine(soa::C2 P, soa::C2 M, float2 avr, float2
     nwr.x = kRH * (P.re.x - M.re.x);
     wi.x = -kRH * (P.im.x + M.im.x);
   }
-  const float2 br = make_float2(b.x, b.y), bi = make_float2(b.z, b.w), nbi = soa::ng(bi);
   Outs o;
+  if constexpr (EXACT) {
+    const float2 br = soa::bc(b.x), bi = soa::bc(b.y), rr = soa::bc(b.z), ri = soa::bc(b.w), nwi = soa::ng(wi);
+    o.lo0 = soa::fma2(nui, bi, soa::fma2(ur, br, soa::fma2(nui, ri, soa::mul2(ur, rr))));
+    o.hi0 = soa::fma2(nui, br, soa::fma2(ur, soa::ng(bi), soa::fma2(nui, rr, soa::mul2(ur, soa::ng(ri)))));
+    o.lo1 = soa::fma2(nwi, br, soa::fma2(nwr, bi, soa::fma2(nwi, rr, soa::mul2(nwr, ri))));
+    o.hi1 = soa::fma2(wi, bi, soa::fma2(nwr, br, soa::fma2(wi, ri, soa::mul2(nwr, rr))));
+    return o;
+  }
+  const float2 br = make_float2(b.x, b.y), bi = make_float2(b.z, b.w), nbi = soa::ng(bi);
   o.lo0 = soa::fma2(nui, bi, soa::mul2(ur, br));
   o.hi0 = soa::fma2(nui, br, soa::mul2(ur, nbi));
   o.lo1 = soa::fma2(soa::ng(wi), br, soa::mul2(nwr, bi));
@@ -277,13 +287,13 @@ __device__ __forceinline__ void neg_pairs(soa::C2* v, int g, int t, int src, con
 }
 
 // Postprocess of a group's two rows from the last stage's registers.
-template <int L, bool FIRST, typename Out>
+template <int L, bool FIRST, bool EXACT, typename Out>
 __device__ __forceinline__ void fwd_post(soa::C2* v, const Out& out, float2 avr, float2 avi,
                                          const float4* __restrict__ fb4, int g, bool packed) {
   constexpr int NS = Last<L>::NS;
   neg_pairs<L>(v, g, neg_lane_butterfly<NS>(g), neg_lane_source<NS>(g),
                [&](soa::C2 P, soa::C2 M, int base, int off, bool mirror) {
-                 out.store(combine<FIRST>(P, M, avr, avi, __ldg(fb4 + base + off), packed), base, off, mirror);
+                 out.store(combine<FIRST, EXACT>(P, M, avr, avi, __ldg(fb4 + base + off), packed), base, off, mirror);
                });
 }
 
@@ -301,15 +311,17 @@ struct Quad {
 // c2, -(c3 + c4)); at the mirror the reads trade places and b_km = i conj(b_k2).
 // FIRST && packed: lane a packs rows 0 and N1/2 as the real and imaginary
 // parts of one sequence.
-template <bool FIRST>
-__device__ __forceinline__ void inv_pair_points(const Quad& qa, const Quad& qb, float2 b, float2 iaA, float2 iar,
+// EXACT: b = (br, bi) and the rests that its rounding left (else 0).
+template <bool FIRST, bool EXACT>
+__device__ __forceinline__ void inv_pair_points(const Quad& qa, const Quad& qb, float4 b4, float2 iaA, float2 iar,
                                                 float2 iai, float2 ih, bool packed, soa::C2& lo,
                                                 soa::C2& hi) {
-  const float2 br = soa::bc(b.x), bi = soa::bc(b.y);
+  const float2 b = make_float2(b4.x, b4.y), br = soa::bc(b.x), bi = soa::bc(b.y);
+  const float2 rr = soa::bc(b4.z), ri = soa::bc(b4.w);
   const soa::C2 x{make_float2(qa.c1 - qa.c2, qb.c1 - qb.c2), make_float2(-(qa.c3 + qa.c4), -(qb.c3 + qb.c4))};
-  lo = soa::mulw(soa::mulw(x, br, bi), iar, iai);
+  lo = soa::mulw(EXACT ? soa::mulw(x, br, bi, rr, ri) : soa::mulw(x, br, bi), iar, iai);
   const soa::C2 y{make_float2(qa.c2 + qa.c1, qb.c2 + qb.c1), make_float2(qa.c4 - qa.c3, qb.c4 - qb.c3)};
-  hi = soa::mulw(soa::mulwc(y, br, bi), iar, iai);
+  hi = soa::mulw(EXACT ? soa::mulw(y, br, soa::ng(bi), rr, soa::ng(ri)) : soa::mulwc(y, br, bi), iar, iai);
   if (FIRST && packed) {
     const float2 v0 = cmul(cmul(make_float2(qa.c1, -qa.c4), b), iaA);
     const float2 vh = cmul(cmul(make_float2(qa.c3 - qa.c2, -(qa.c3 + qa.c2)), b), ih);
@@ -326,18 +338,24 @@ __device__ __forceinline__ void inv_pair_points(const Quad& qa, const Quad& qb, 
 // Points t + TPS j (t the thread's first-stage butterfly, returned) of both
 // items in v.  quads(k2, km, qa, qb) reads one pair of columns of both items
 // (km = 0 past the edge for k2 = 0, where the mirror reads are zero).
-template <int L, bool FIRST, typename Quads>
-__device__ __forceinline__ int inv_pre(const Quads& quads, const float2* __restrict__ ib, float2 iaA, float2 iaB,
+template <int L, bool FIRST, bool EXACT, typename Quads>
+__device__ __forceinline__ int inv_pre(const Quads& quads, const float2* __restrict__ ib,
+                                       const float4* __restrict__ ib4, float2 iaA, float2 iaB,
                                        float2 ih, bool packed, int g, soa::C2* v) {
   constexpr int T = fft_tps(L);
   const int t = neg_lane_butterfly<T>(g), src = neg_lane_source<T>(g);
   const float2 iar = make_float2(iaA.x, iaB.x), iai = make_float2(iaA.y, iaB.y);
+  auto twiddle = [&](int k) {
+    if constexpr (EXACT) return __ldg(ib4 + k);
+    const float2 w = __ldg(ib + k);
+    return make_float4(w.x, w.y, 0.f, 0.f);
+  };
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     Quad qa, qb;
     quads(t + T * j, L - t - T * j, j == 0 && t == 0, qa, qb);
     soa::C2 hi;
-    inv_pair_points<FIRST>(qa, qb, __ldg(ib + t + T * j), iaA, iar, iai, ih, packed, v[j], hi);
+    inv_pair_points<FIRST, EXACT>(qa, qb, twiddle(t + T * j), iaA, iar, iai, ih, packed, v[j], hi);
     v[15 - j] = shfl(hi, src);  // point L - k2 belongs to the mirror butterfly, at 15 - j
   }
   if (t == 0) {  // butterfly 0 mirrors onto itself with j <-> 16 - j; point L / 2 pairs with itself
@@ -346,7 +364,7 @@ __device__ __forceinline__ int inv_pre(const Quads& quads, const float2* __restr
     Quad qa, qb;
     quads(L / 2, L / 2, false, qa, qb);
     soa::C2 hi;
-    inv_pair_points<FIRST>(qa, qb, __ldg(ib + L / 2), iaA, iar, iai, ih, packed, v[8], hi);
+    inv_pair_points<FIRST, EXACT>(qa, qb, twiddle(L / 2), iaA, iar, iai, ih, packed, v[8], hi);
   }
   return t;
 }

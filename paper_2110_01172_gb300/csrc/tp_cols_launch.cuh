@@ -35,15 +35,15 @@ bool encode_maps(const Dct2dArgs& a, const PoissonArgs& ps, int batch, bool inve
          CUDA_SUCCESS;
 }
 
-template <int M, int NP, bool INV, bool POIS>
+template <int M, int NP, bool INV, bool POIS, bool EXACT>
 cudaError_t col_launch_k(const Dct2dArgs& a, const PoissonArgs& ps, int batch, cudaStream_t s, bool prepare) {
   using G = TpColGeom<M, NP>;
   if (prepare) {
     if (G::SMEM_TMA <= 48 * 1024) return cudaSuccess;  // within the default limit
-    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_tp_cols<M, NP, INV, POIS>),
+    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_tp_cols<M, NP, INV, POIS, EXACT>),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_tp_cols_tma<M, NP, INV, POIS>),
+      e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_tp_cols_tma<M, NP, INV, POIS, EXACT>),
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM_TMA);
     return e;
   }
@@ -52,8 +52,8 @@ cudaError_t col_launch_k(const Dct2dArgs& a, const PoissonArgs& ps, int batch, c
   // host-mapped or managed buffers
   ColMaps<POIS ? 3 : 1> maps;
   if (a.io_dev && encode_maps(a, ps, batch, INV, NP, G::ZB, &maps))
-    return pdl::launch(k_tp_cols_tma<M, NP, INV, POIS>, grid, dim3(G::THREADS), G::SMEM_TMA, s, a, maps);
-  return pdl::launch(k_tp_cols<M, NP, INV, POIS>, grid, dim3(G::THREADS), G::SMEM, s, a, ps);
+    return pdl::launch(k_tp_cols_tma<M, NP, INV, POIS, EXACT>, grid, dim3(G::THREADS), G::SMEM_TMA, s, a, maps);
+  return pdl::launch(k_tp_cols<M, NP, INV, POIS, EXACT>, grid, dim3(G::THREADS), G::SMEM, s, a, ps);
 }
 
 // The strip width: the plan's choice, else the default for M, halved (down
@@ -78,7 +78,10 @@ cudaError_t col_width(const Dct2dArgs& a, const PoissonArgs& ps, int batch, cuda
     return cudaErrorInvalidValue;
   } else {
     if (!prepare && (a.n2 / 4) % NP) return cudaErrorInvalidValue;
-    return col_launch_k<M, NP, INV, POIS>(a, ps, batch, s, prepare);
+    // exact plans with M > 32 have N2 = 64 (a stage of radix 2, M = 32, is exact anyway)
+    if constexpr (M > 32 && NP <= 16 && G::POISSON)
+      if (a.exact) return col_launch_k<M, NP, INV, POIS, true>(a, ps, batch, s, prepare);
+    return a.exact && M > 32 ? cudaErrorInvalidValue : col_launch_k<M, NP, INV, POIS, false>(a, ps, batch, s, prepare);
   }
 }
 

@@ -1,5 +1,5 @@
 // tp_rows_launch.cuh - launch rules of the two-pass family's row passes, shared
-// by the translation units of the forward and the inverse row pass.
+// by the translation units of the forward, the inverse and the Poisson row pass.
 #pragma once
 
 #include "dct2d_launch.cuh"
