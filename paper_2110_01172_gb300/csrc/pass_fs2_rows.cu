@@ -31,8 +31,9 @@ cudaError_t row_launch(bool inverse, const Dct2dArgs& a, int batch, cudaStream_t
     if (inverse) return pdl::launch(k_fs2_rows_inv_x2<L, false>, grid, block, R::SMEM, s, a);
     Dct2dArgs b = a;
     b.ahead = L == 8192 && (long long)batch * a.n1 * a.n2 * 4 > a.l2 ? a.nsm : 0;
-    if (a.vkind == 1 || a.thresh > 0.f) return pdl::launch(k_fs2_rows_fwd_x2<L, true>, grid, block, R::SMEM, s, b);
-    return pdl::launch(k_fs2_rows_fwd_x2<L, false>, grid, block, R::SMEM, s, b);
+    const bool overlap = pdl::gains_from_overlap((long long)grid.x * batch, a.nsm);
+    const auto k = a.vkind == 1 || a.thresh > 0.f ? k_fs2_rows_fwd_x2<L, true> : k_fs2_rows_fwd_x2<L, false>;
+    return pdl::launch_if(overlap, k, grid, block, R::SMEM, s, b);
   } else {
     using R = RowGeom<L>;
     if (prepare) {

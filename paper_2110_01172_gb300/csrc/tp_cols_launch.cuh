@@ -48,12 +48,13 @@ cudaError_t col_launch_k(const Dct2dArgs& a, const PoissonArgs& ps, int batch, c
     return e;
   }
   const dim3 grid(a.n2 / 4 / NP, 2, batch);
+  const bool overlap = INV || pdl::gains_from_overlap(2LL * grid.x * batch, a.nsm);
   // bulk tensor copies for device buffers; per-thread loads / stores for
   // host-mapped or managed buffers
   ColMaps<POIS ? 3 : 1> maps;
   if (a.io_dev && encode_maps(a, ps, batch, INV, NP, G::ZB, &maps))
-    return pdl::launch(k_tp_cols_tma<M, NP, INV, POIS, EXACT>, grid, dim3(G::THREADS), G::SMEM_TMA, s, a, maps);
-  return pdl::launch(k_tp_cols<M, NP, INV, POIS, EXACT>, grid, dim3(G::THREADS), G::SMEM, s, a, ps);
+    return pdl::launch_if(overlap, k_tp_cols_tma<M, NP, INV, POIS, EXACT>, grid, dim3(G::THREADS), G::SMEM_TMA, s, a, maps);
+  return pdl::launch_if(overlap, k_tp_cols<M, NP, INV, POIS, EXACT>, grid, dim3(G::THREADS), G::SMEM, s, a, ps);
 }
 
 // The strip width: the plan's choice, else the default for M, halved (down
