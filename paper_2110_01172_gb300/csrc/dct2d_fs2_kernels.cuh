@@ -726,37 +726,53 @@ __device__ __forceinline__ void fwd_split_x2(const float2* __restrict__ za, cons
   }
 }
 
-// Forward postprocess of both items (rowp::fwd_post) into the output rows k1,
-// N1-k1 (lane a; rows 0 and N1/2 of the packed item) and kb, N1-kb (lane b) of
-// y, `stride` floats apart.  GENERAL: plans with the DST-II order or a magnitude
-// threshold.
+// Output rows k1, N1-k1 (lane a; rows 0 and N1/2 of the packed item) and kb, N1-kb
+// (lane b) of a group.
+struct OutRows {
+  float *a0, *a1, *b0, *b1;
+};
+// The output row of item k (mirror: its second row); DST-II (rev): output (k1, k2)
+// goes to (N1-1-k1, N2-1-k2).
+__device__ __forceinline__ int fwd_out_row(int k, bool mirror, int N1, bool rev) {
+  const int r = mirror ? row_mirror(k, N1) : k;
+  return rev ? N1 - 1 - r : r;
+}
+
+// Forward postprocess of both items (rowp::fwd_post) into their output rows.
+// GENERAL: plans with the DST-II order or a magnitude threshold.
 template <int L, bool GENERAL, bool FIRST, bool SMEM, bool EXACT>
-__device__ __forceinline__ void fwd_post_rows(soa::C2* v, const Dct2dArgs& a, float* y, long long stride, int k1,
-                                              int kb, bool packed, int g) {
-  const int N1 = a.n1;
+__device__ __forceinline__ void fwd_post_rows(soa::C2* v, const Dct2dArgs& a, const OutRows& rows, int k1, int kb,
+                                              bool packed, int g) {
   const float2 fa0 = __ldg(a.fa + k1), fa1 = __ldg(a.fa + kb);
   // 1/2 of the split folded into the a-twiddle (not for the packed item)
   const float2 avr = make_float2(packed ? 1.f : 0.5f * fa0.x, 0.5f * fa1.x);
   const float2 avi = make_float2(packed ? 0.f : 0.5f * fa0.y, 0.5f * fa1.y);
-  const bool rev = GENERAL && a.vkind == 1;  // DST-II: output (k1, k2) goes to (N1-1-k1, N2-1-k2)
-  const int kma = row_mirror(k1, N1), kmb = row_mirror(kb, N1);
   rowp::FwdOut<L, GENERAL, SMEM> out;
-  out.a0 = y + (rev ? N1 - 1 - k1 : k1) * stride;
-  out.a1 = y + (rev ? N1 - 1 - kma : kma) * stride;
-  out.b0 = y + (rev ? N1 - 1 - kb : kb) * stride;
-  out.b1 = y + (rev ? N1 - 1 - kmb : kmb) * stride;
+  out.a0 = rows.a0;
+  out.a1 = rows.a1;
+  out.b0 = rows.b0;
+  out.b1 = rows.b1;
   out.pol = l2::evict_first();  // the output is streamed out
   out.eps = a.thresh;           // magnitude threshold of Section V-A, Eq. image-compression (0: off)
-  out.rev = rev;
+  out.rev = GENERAL && a.vkind == 1;
   rowp::fwd_post<L, FIRST, EXACT>(v, out, avr, avi, a.fb4, g, packed);
 }
 template <int L, bool GENERAL, bool SMEM, bool EXACT>
-__device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, float* y, long long stride, int k1, int kb,
+__device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, const OutRows& rows, int k1, int kb,
                                             bool packed, int g) {
   if (rowp::warp_has_first<fft_tps(L)>(packed))
-    fwd_post_rows<L, GENERAL, true, SMEM, EXACT>(v, a, y, stride, k1, kb, packed, g);
+    fwd_post_rows<L, GENERAL, true, SMEM, EXACT>(v, a, rows, k1, kb, packed, g);
   else
-    fwd_post_rows<L, GENERAL, false, SMEM, EXACT>(v, a, y, stride, k1, kb, false, g);
+    fwd_post_rows<L, GENERAL, false, SMEM, EXACT>(v, a, rows, k1, kb, false, g);
+}
+// The same into rows of y, `stride` floats apart.
+template <int L, bool GENERAL, bool SMEM, bool EXACT>
+__device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, float* y, long long stride, int k1, int kb,
+                                            bool packed, int g) {
+  const bool rev = GENERAL && a.vkind == 1;
+  auto row = [&](int k, bool mirror) { return y + fwd_out_row(k, mirror, a.n1, rev) * stride; };
+  const OutRows rows{row(k1, false), row(k1, true), row(kb, false), row(kb, true)};
+  fwd_post_x2<L, GENERAL, SMEM, EXACT>(v, a, rows, k1, kb, packed, g);
 }
 
 // Row FFT of both items from registers (v: points t + TPS j of the thread's

@@ -354,8 +354,33 @@ __device__ __forceinline__ void tp_fwd_load(const float2* e1r, const float2* o1r
   }
 }
 
+// The group's finished rows gathered in its shared buffer and stored whole by the
+// CTA, for outputs that are not device memory: the registers' stores cover L/16
+// columns at a time, which L2 joins but the host link does not (device to page-locked
+// host memory, stored from registers / gathered: 64 x (512 x 64) 230 / 61 us, 64 x (512
+// x 128) 292 / 95).
+template <int L, bool NARROW, bool EXACT>
+__device__ __forceinline__ void tp_fwd_gathered(soa::C2* v, float4* smem, const Dct2dArgs& a, int c, int kb, bool first,
+                                                int g, int pi) {
+  using R = TpRows<L, NARROW>;
+  float* st = reinterpret_cast<float*>(smem + pi * R::LP);  // 4 L of its 4.25 L floats
+  rowp::group_sync<R::TPS>(pi);                             // the rows overlay the points of the last stage
+  fwd_post_x2<L, true, true, EXACT>(v, a, OutRows{st, st + L, st + 2 * L, st + 3 * L}, c, kb, first, g);
+  __syncthreads();
+  float* y = a.out + (long long)blockIdx.z * a.out_bstride;
+  const uint64_t pol = l2::evict_first();
+#pragma unroll 4
+  for (int i = 0; i < R::NP * L / R::THREADS; ++i) {
+    const int f = threadIdx.x + R::THREADS * i, row = f / (L / 4), col = f % (L / 4), slot = row & 3;
+    const int cc = blockIdx.x * R::NP + row / 4, item = slot < 2 ? cc : tp_item_b(cc, a.n1 / 2);
+    const int k = fwd_out_row(item, slot & 1, a.n1, a.vkind == 1);
+    l2::st(reinterpret_cast<float4*>(y + (long long)k * L) + col, smem[row / 4 * R::LP + slot * (L / 4) + col], pol);
+  }
+}
+
 // GENERAL: plans with the DST-II order or a magnitude threshold (row_pairs.cuh).
-template <int L, bool NARROW, bool GENERAL, bool EXACT>
+// HOST: the output is not device memory.
+template <int L, bool NARROW, bool GENERAL, bool EXACT, bool HOST>
 __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>::MINB) k_tp_rows_fwd(Dct2dArgs a) {
   using R = TpRows<L, NARROW>;
   constexpr int TPS = R::TPS;
@@ -379,7 +404,14 @@ __global__ void __launch_bounds__(TpRows<L, NARROW>::THREADS, TpRows<L, NARROW>:
     tp_fwd_load<L, true, false, EXACT>(e1r, o1r, e2r, o2r, w, first, t, v);
   else
     tp_fwd_load<L, false, false, EXACT>(e1r, o1r, e2r, o2r, w, false, t, v);
-  fwd_fft_post_x2<L, GENERAL, EXACT>(v, s, a, a.out + (long long)blockIdx.z * a.out_bstride, c, kb, first, t, g, pi);
+  if constexpr (HOST) {
+    soa::first_stage<L, false>(v, s, t);
+    rowp::stages_to_regs<L, 16, false, true, EXACT>(s, g, pi, a.tw2x, v);
+    pdl::launch_dependents();
+    tp_fwd_gathered<L, NARROW, EXACT>(v, sxt, a, c, kb, first, g, pi);
+  } else {
+    fwd_fft_post_x2<L, GENERAL, EXACT>(v, s, a, a.out + (long long)blockIdx.z * a.out_bstride, c, kb, first, t, g, pi);
+  }
 }
 
 // Inverse pairing of both items into E' / O' rows: from the row IFFT u in v,
