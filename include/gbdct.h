@@ -321,6 +321,12 @@ gbdct_status gbdct_poisson_create(gbdct_poisson_t* out, int64_t n1, int64_t n2);
 gbdct_status gbdct_poisson_solve(gbdct_poisson_t p, const void* rho, void* psi, void* xi0, void* xi1,
                                  void* stream);
 
+/* As gbdct_plan_check_device_error and gbdct_plan_set_wait_limit, for the plans of a
+ * solver: a solve whose bounded waits gave up leaves parts of its outputs unwritten
+ * and says so here (GBDCT_ERR_TIMEOUT, once). */
+gbdct_status gbdct_poisson_check_device_error(gbdct_poisson_t p);
+gbdct_status gbdct_poisson_set_wait_limit(gbdct_poisson_t p, uint32_t polls);
+
 /* Device bytes owned by the solver (workspaces, staging and tables). */
 size_t gbdct_poisson_workspace_bytes(gbdct_poisson_t p);
 

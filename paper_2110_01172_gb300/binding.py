@@ -84,6 +84,8 @@ def load(path: str | None = None, build_if_missing: bool = True) -> ctypes.CDLL:
             "gbdct_poisson_create": (ctypes.c_int, [ctypes.POINTER(plan_p), ctypes.c_int64, ctypes.c_int64]),
             "gbdct_poisson_solve": (ctypes.c_int, [plan_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                                    ctypes.c_void_p, ctypes.c_void_p]),
+            "gbdct_poisson_check_device_error": (ctypes.c_int, [plan_p]),
+            "gbdct_poisson_set_wait_limit": (ctypes.c_int, [plan_p, ctypes.c_uint32]),
             "gbdct_poisson_workspace_bytes": (ctypes.c_size_t, [plan_p]),
             "gbdct_poisson_destroy": (ctypes.c_int, [plan_p]),
             "gbdct_dct2d_forward_noalloc": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64,
@@ -417,6 +419,15 @@ class PoissonSolver:
         _check(self._lib.gbdct_poisson_solve(self._h, rho.data_ptr(), psi.data_ptr(), xi0.data_ptr(), xi1.data_ptr(),
                                              _stream_handle(stream, rho.device)), "gbdct_poisson_solve")
         return psi, xi0, xi1
+
+    def check_device_error(self) -> int:
+        """Status of the solver's device error words (OK, or ERR_TIMEOUT after a bounded wait gave up)."""
+        return int(self._lib.gbdct_poisson_check_device_error(self._h))
+
+    def set_wait_limit(self, polls: int):
+        """Bound of the solver's device-side waits in polls (0: the default)."""
+        _check(self._lib.gbdct_poisson_set_wait_limit(self._h, int(polls)), "gbdct_poisson_set_wait_limit")
+        return self
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:

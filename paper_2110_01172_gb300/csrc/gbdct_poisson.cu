@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
 #include <new>
 
 #include "../../include/gbdct.h"
@@ -151,6 +152,24 @@ gbdct_status gbdct_poisson_solve(gbdct_poisson_t p, const void* rho, void* psi, 
   if (st == GBDCT_OK) st = gbdct_exec_inverse(p->fld0, xi0, xi0, stream);
   if (st == GBDCT_OK) st = gbdct_exec_inverse(p->fld1, xi1, xi1, stream);
   return st;
+}
+
+gbdct_status gbdct_poisson_check_device_error(gbdct_poisson_t p) {
+  if (!p) return GBDCT_ERR_INVALID_ARG;
+  gbdct_status st = GBDCT_OK;
+  for (gbdct_plan_t plan : {p->fused, p->fwd, p->fld0, p->fld1}) {
+    if (!plan) continue;
+    const gbdct_status one = gbdct_plan_check_device_error(plan);  // clears every plan's word
+    if (st == GBDCT_OK) st = one;
+  }
+  return st;
+}
+
+gbdct_status gbdct_poisson_set_wait_limit(gbdct_poisson_t p, uint32_t polls) {
+  if (!p) return GBDCT_ERR_INVALID_ARG;
+  for (gbdct_plan_t plan : {p->fused, p->fwd, p->fld0, p->fld1})
+    if (plan) gbdct_plan_set_wait_limit(plan, polls);
+  return GBDCT_OK;
 }
 
 size_t gbdct_poisson_workspace_bytes(gbdct_poisson_t p) {
