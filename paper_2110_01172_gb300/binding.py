@@ -155,6 +155,28 @@ def _stream_handle(stream, device):
     return _current_stream(device.index)
 
 
+def _contiguous(x, stream, device):
+    """x, or a contiguous copy of it on the device that a call on `stream` (None: the
+    current one) may read although the caller never sees it.
+
+    The copy is made on the current stream, so another stream waits for it, and the
+    allocator learns that the stream uses it.  Page-locked memory is copied to the
+    device as well: a host copy would be pageable and gone before the kernels read it.
+    """
+    if x.is_contiguous():
+        return x
+    torch = _torch()
+    x = x.contiguous() if x.is_cuda else x.to(device).contiguous()
+    if stream is not None:
+        current = torch.cuda.current_stream(x.device)
+        if stream.cuda_stream != current.cuda_stream:
+            if not isinstance(stream, torch.cuda.Stream):
+                stream = torch.cuda.ExternalStream(stream.cuda_stream, device=x.device)
+            stream.wait_stream(current)
+            x.record_stream(stream)
+    return x
+
+
 class Plan:
     """A transform plan: twiddle tables and workspace resident on one GPU.
 
@@ -219,7 +241,7 @@ class Plan:
         """Kernel launches of one forward call (an inverse one differs in the split-BF16 mode only)."""
         return int(self._lib.gbdct_plan_launches_per_exec(self._h))
 
-    def _prep(self, x, out):
+    def _prep(self, x, out, stream=None):
         """x and out: CUDA float32 tensors, or page-locked CPU float32 tensors
         (read/written by the kernels over the host link, no staging copy)."""
         torch = _torch()
@@ -238,22 +260,21 @@ class Plan:
             raise TypeError("expected a CUDA or page-locked CPU float32 tensor")
         if tuple(x.shape) != want:
             raise ValueError(f"expected shape {want}, got {tuple(x.shape)}")
-        if not x.is_contiguous():
-            x = x.contiguous()
         if out is None:
-            out = torch.empty_like(x) if x.is_cuda else torch.empty(want, dtype=torch.float32, pin_memory=True)
+            out = (torch.empty(want, dtype=torch.float32, device=x.device) if x.is_cuda
+                   else torch.empty(want, dtype=torch.float32, pin_memory=True))
         elif tuple(out.shape) != want or not usable(out) or not out.is_contiguous():
             raise ValueError("out must be a contiguous CUDA or page-locked float32 tensor of the input's shape")
-        return x, out
+        return _contiguous(x, stream, self.device), out
 
     def forward(self, x, out=None, stream=None):
-        x, out = self._prep(x, out)
+        x, out = self._prep(x, out, stream)
         _check(self._lib.gbdct_exec_forward(self._h, x.data_ptr(), out.data_ptr(),
                                             _stream_handle(stream, self.device)), "gbdct_exec_forward")
         return out
 
     def inverse(self, x, out=None, stream=None):
-        x, out = self._prep(x, out)
+        x, out = self._prep(x, out, stream)
         _check(self._lib.gbdct_exec_inverse(self._h, x.data_ptr(), out.data_ptr(),
                                             _stream_handle(stream, self.device)), "gbdct_exec_inverse")
         return out
@@ -412,7 +433,7 @@ class PoissonSolver:
         torch = _torch()
         if rho.dtype != torch.float32 or not rho.is_cuda or tuple(rho.shape) != self.shape:
             raise ValueError(f"expected a CUDA float32 tensor of shape {self.shape}")
-        rho = rho.contiguous()
+        rho = _contiguous(rho, stream, self.device)
         psi = torch.empty_like(rho) if psi is None else psi
         xi0 = torch.empty_like(rho) if xi0 is None else xi0
         xi1 = torch.empty_like(rho) if xi1 is None else xi1
