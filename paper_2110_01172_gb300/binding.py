@@ -177,6 +177,13 @@ def _contiguous(x, stream, device):
     return x
 
 
+def _check_out(out, numel, what):
+    """The kernels write `numel` float32 values through the pointer, whatever the tensor says."""
+    if not (out.dtype is _torch().float32 and out.numel() == numel and out.is_contiguous()
+            and (out.is_cuda or out.is_pinned())):
+        raise ValueError(f"{what} must be a contiguous CUDA or page-locked float32 tensor of {numel} values")
+
+
 class Plan:
     """A transform plan: twiddle tables and workspace resident on one GPU.
 
@@ -387,7 +394,10 @@ class MultiPlan:
         torch = _torch()
         if x.dtype != torch.float32 or not x.is_cuda or x.numel() != self.total or not x.is_contiguous():
             raise ValueError(f"expected a contiguous CUDA float32 buffer of {self.total} values")
-        out = torch.empty_like(x) if out is None else out
+        if out is None:
+            out = torch.empty_like(x)
+        else:
+            _check_out(out, self.total, "out")
         _check(self._lib.gbdct_multi_exec(self._h, int(inverse), x.data_ptr(), out.data_ptr(),
                                           _stream_handle(stream, self.device)), "gbdct_multi_exec")
         return out
@@ -434,9 +444,13 @@ class PoissonSolver:
         if rho.dtype != torch.float32 or not rho.is_cuda or tuple(rho.shape) != self.shape:
             raise ValueError(f"expected a CUDA float32 tensor of shape {self.shape}")
         rho = _contiguous(rho, stream, self.device)
-        psi = torch.empty_like(rho) if psi is None else psi
-        xi0 = torch.empty_like(rho) if xi0 is None else xi0
-        xi1 = torch.empty_like(rho) if xi1 is None else xi1
+        outs = [psi, xi0, xi1]
+        for i, out in enumerate(outs):
+            if out is None:
+                outs[i] = torch.empty_like(rho)
+            else:
+                _check_out(out, self.shape[0] * self.shape[1], "psi, xi0 and xi1")
+        psi, xi0, xi1 = outs
         _check(self._lib.gbdct_poisson_solve(self._h, rho.data_ptr(), psi.data_ptr(), xi0.data_ptr(), xi1.data_ptr(),
                                              _stream_handle(stream, rho.device)), "gbdct_poisson_solve")
         return psi, xi0, xi1
@@ -607,6 +621,8 @@ def dct2_noalloc(x, out=None, stream=None):
         raise TypeError("expected a contiguous 2D CUDA float32 tensor")
     if out is None:
         out = torch.empty_like(x)
+    else:
+        _check_out(out, x.numel(), "out")
     n1, n2 = x.shape
     _check(lib.gbdct_dct2d_forward_noalloc(ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(out.data_ptr()),
                                            n1, n2, _stream_handle(stream, x.device)),
