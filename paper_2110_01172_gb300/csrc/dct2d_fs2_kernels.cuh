@@ -738,16 +738,17 @@ __device__ __forceinline__ int fwd_out_row(int k, bool mirror, int N1, bool rev)
   return rev ? N1 - 1 - r : r;
 }
 
-// Forward postprocess of both items (rowp::fwd_post) into their output rows.
-// GENERAL: plans with the DST-II order or a magnitude threshold.
-template <int L, bool GENERAL, bool FIRST, bool SMEM, bool EXACT>
-__device__ __forceinline__ void fwd_post_rows(soa::C2* v, const Dct2dArgs& a, const OutRows& rows, int k1, int kb,
+// Forward postprocess of both items (rowp::fwd_post) into their output rows,
+// rows_of().  GENERAL: plans with the DST-II order or a magnitude threshold.
+template <int L, bool GENERAL, bool FIRST, bool SMEM, bool EXACT, typename Rows>
+__device__ __forceinline__ void fwd_post_rows(soa::C2* v, const Dct2dArgs& a, const Rows& rows_of, int k1, int kb,
                                               bool packed, int g) {
   const float2 fa0 = __ldg(a.fa + k1), fa1 = __ldg(a.fa + kb);
   // 1/2 of the split folded into the a-twiddle (not for the packed item)
   const float2 avr = make_float2(packed ? 1.f : 0.5f * fa0.x, 0.5f * fa1.x);
   const float2 avi = make_float2(packed ? 0.f : 0.5f * fa0.y, 0.5f * fa1.y);
   rowp::FwdOut<L, GENERAL, SMEM> out;
+  const OutRows rows = rows_of();
   out.a0 = rows.a0;
   out.a1 = rows.a1;
   out.b0 = rows.b0;
@@ -757,13 +758,13 @@ __device__ __forceinline__ void fwd_post_rows(soa::C2* v, const Dct2dArgs& a, co
   out.rev = GENERAL && a.vkind == 1;
   rowp::fwd_post<L, FIRST, EXACT>(v, out, avr, avi, a.fb4, g, packed);
 }
-template <int L, bool GENERAL, bool SMEM, bool EXACT>
-__device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, const OutRows& rows, int k1, int kb,
+template <int L, bool GENERAL, bool SMEM, bool EXACT, typename Rows>
+__device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, const Rows& rows_of, int k1, int kb,
                                             bool packed, int g) {
   if (rowp::warp_has_first<fft_tps(L)>(packed))
-    fwd_post_rows<L, GENERAL, true, SMEM, EXACT>(v, a, rows, k1, kb, packed, g);
+    fwd_post_rows<L, GENERAL, true, SMEM, EXACT>(v, a, rows_of, k1, kb, packed, g);
   else
-    fwd_post_rows<L, GENERAL, false, SMEM, EXACT>(v, a, rows, k1, kb, false, g);
+    fwd_post_rows<L, GENERAL, false, SMEM, EXACT>(v, a, rows_of, k1, kb, false, g);
 }
 // The same into rows of y, `stride` floats apart.
 template <int L, bool GENERAL, bool SMEM, bool EXACT>
@@ -771,8 +772,8 @@ __device__ __forceinline__ void fwd_post_x2(soa::C2* v, const Dct2dArgs& a, floa
                                             bool packed, int g) {
   const bool rev = GENERAL && a.vkind == 1;
   auto row = [&](int k, bool mirror) { return y + fwd_out_row(k, mirror, a.n1, rev) * stride; };
-  const OutRows rows{row(k1, false), row(k1, true), row(kb, false), row(kb, true)};
-  fwd_post_x2<L, GENERAL, SMEM, EXACT>(v, a, rows, k1, kb, packed, g);
+  fwd_post_x2<L, GENERAL, SMEM, EXACT>(
+      v, a, [&] { return OutRows{row(k1, false), row(k1, true), row(kb, false), row(kb, true)}; }, k1, kb, packed, g);
 }
 
 // Row FFT of both items from registers (v: points t + TPS j of the thread's

@@ -365,7 +365,8 @@ __device__ __forceinline__ void tp_fwd_gathered(soa::C2* v, float4* smem, const 
   using R = TpRows<L, NARROW>;
   float* st = reinterpret_cast<float*>(smem + pi * R::LP);  // 4 L of its 4.25 L floats
   rowp::group_sync<R::TPS>(pi);                             // the rows overlay the points of the last stage
-  fwd_post_x2<L, true, true, EXACT>(v, a, OutRows{st, st + L, st + 2 * L, st + 3 * L}, c, kb, first, g);
+  fwd_post_x2<L, true, true, EXACT>(
+      v, a, [&] { return OutRows{st, st + L, st + 2 * L, st + 3 * L}; }, c, kb, first, g);
   __syncthreads();
   float* y = a.out + (long long)blockIdx.z * a.out_bstride;
   const uint64_t pol = l2::evict_first();
