@@ -50,10 +50,10 @@ FALLBACK_HBM_GBS = 6800.0
 # launches, so the workspace stays in L2 as it does here).  Valid only for the
 # kernel sources with this digest; otherwise reported as null.
 TRAFFIC = {
-    "sources_sha256": "5fb873179485872c29c9a19aab0e2b700e5d23236e86beb6e7f6d406c5b9849b",
+    "sources_sha256": "cb1c426922a94bd6e65bbf95b115e1c9272c48ed798a4395422aaddb31d77181",
     "family": "tp",
-    "forward_bytes": 157930240,
-    "inverse_bytes": 151274496,
+    "forward_bytes": 158042112,
+    "inverse_bytes": 150663680,
 }
 
 
@@ -144,8 +144,8 @@ def measured_peaks():
 # TRAFFIC is valid only while these are unchanged).
 KERNEL_SOURCES = ("dct2d_tp_kernels.cuh", "dct2d_fs2_kernels.cuh", "dct2d_kernels.cuh", "dct2d_launch.cuh",
                   "fft_core.cuh", "fft_soa.cuh", "l2_hint.cuh", "tma_util.cuh", "launch_dep.cuh", "row_pairs.cuh",
-                  "tp_cols_launch.cuh", "tp_rows_launch.cuh", "pass_tp.cu", "pass_tp_cols_fwd.cu",
-                  "pass_tp_cols_inv.cu", "pass_tp_rows_fwd.cu", "pass_tp_rows_inv.cu")
+                  "tp_cols_launch.cuh", "tp_rows_launch.cuh", "tp_rows_inv_launch.cuh", "pass_tp.cu",
+                  "pass_tp_cols_fwd.cu", "pass_tp_cols_inv.cu", "pass_tp_rows_fwd.cu", "pass_tp_rows_inv.cu")
 
 
 def sources_digest() -> str:

@@ -177,11 +177,11 @@ int gbdct_plan_launches_per_exec(gbdct_plan_t plan);
 const char* gbdct_plan_kernel_family(gbdct_plan_t plan);
 
 /* Reports (and clears) a failure recorded on the device by the plan's
- * kernels: the pipelined tensor-core kernels of the split-BF16 mode bound every
- * wait on an asynchronous copy or MMA, and a wait that gives up records it
- * here instead of hanging the GPU (the kernel then waits for the work it has
- * already issued and leaves its output tile unwritten, so the transform's
- * output is invalid).  Synchronises with the device.  Returns GBDCT_OK,
+ * kernels: the two-pass kernels bound their waits for bulk copies, and the
+ * tensor-core kernels of the split-BF16 mode every wait on an asynchronous copy
+ * or MMA.  A wait that gives up records it here instead of hanging the GPU (the
+ * kernel then waits for the work it has already issued and leaves its part of
+ * the output unwritten, so the transform's output is invalid).  Synchronises with the device.  Returns GBDCT_OK,
  * GBDCT_ERR_TIMEOUT, GBDCT_ERR_INVALID_ARG (NULL plan) or GBDCT_ERR_CUDA. */
 gbdct_status gbdct_plan_check_device_error(gbdct_plan_t plan);
 
@@ -225,7 +225,8 @@ gbdct_status gbdct_plan_create_family(gbdct_plan_t* out, int ndim, const int64_t
  * process and, when the environment variable GBDCT_TUNE_CACHE names a file,
  * appended to that file ("key family microseconds" lines) and read back by
  * later processes, which then create the plan without timing.  family_out
- * (optional, family_cap bytes) receives the chosen candidate's name.
+ * (optional, family_cap bytes) receives the chosen candidate's name; the default
+ * plan goes by its family's, here and in the file.
  * Synchronises the device.  Errors as gbdct_plan_create_batched.
  */
 gbdct_status gbdct_plan_create_tuned(gbdct_plan_t* out, int ndim, const int64_t* dims, int64_t batch, int kind,

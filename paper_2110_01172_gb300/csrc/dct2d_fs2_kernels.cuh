@@ -1,27 +1,24 @@
 // dct2d_fs2_kernels.cuh - four-step column FFTs + row passes, occupancy-first.
 //
-// Same method and data flow as dct2d_fs_kernels.cuh (arXiv 2110.01172,
-// Algorithm 2 with the fused pre/postprocess of Section III; the column FFT of
-// length N1 = A*B split the four-step way so that every global access is a
-// contiguous row segment), with kernels shaped for occupancy:
+// Method: arXiv 2110.01172, Algorithm 2 with the fused pre/postprocess of Section
+// III; the column FFT of length N1 = A*B is split the four-step way so that every
+// global access is a contiguous row segment.  Kernels shaped for occupancy:
 //
 //  * column steps: a CTA owns a slab of S rows (S = A or B) x a block of
 //    complex columns; Q threads share a column group and each holds T = S/Q
 //    points of it, so a DFT_S is a DFT_T in registers, a twiddle W_S^{q m},
 //    an exchange through shared memory and DFT_Qs
-//    (W_S^{(q+Qj)(m+Tp)} = W_S^{qm} W_Q^{qp} W_T^{jm}).  The default vector
-//    form (k_fs2_colv) gives each thread two adjacent columns (16-byte
-//    accesses; Q = 4 or 8, S up to 128); the scalar form (k_fs2_col) one
-//    column with Q = 4;
-//  * row passes: one sequence per 16-point thread group (float2), the radix-16
-//    Stockham engine of fft_core.cuh, ~64 registers per thread.
+//    (W_S^{(q+Qj)(m+Tp)} = W_S^{qm} W_Q^{qp} W_T^{jm}).  A thread has two adjacent
+//    columns (16-byte accesses; Q = 4 or 8), one at S = 128;
+//  * row passes: two items per thread group on the two-lane engine of fft_soa.cuh
+//    (N2 <= 8192), or one sequence per group (float2, the radix-16 Stockham engine
+//    of fft_core.cuh, ~64 registers per thread) at N2 = 16384.
 //
-// Workspace layout as in dct2d_fs_kernels.cuh: N1 rows of N2/2 complex, row
-// k1 of the column spectrum at physical row (k1 % B) * A + k1 / B.
+// Workspace: N1 rows of N2/2 complex, row k1 of the column spectrum at physical row
+// (k1 % B) * A + k1 / B.
 // Launches overlap through programmatic dependent launch (8192 x 4096 forward /
 // inverse 153.8 / 148.6 -> 147.0 / 142.6 us).
-// Supported: N1 in {256, ..., 8192} (8192 with the vector column steps only),
-// N2 in {256, ..., 16384}.
+// Supported: N1 in {256, ..., 8192}, N2 in {256, ..., 16384}.
 //
 // The other kinds are index/sign maps around the DCT-II (Section V-B, Eq.
 // idxst; DST-II per axis), folded into the first loads and last stores
@@ -900,10 +897,10 @@ __device__ __forceinline__ int inv_pre_x2(const Dct2dArgs& a, const Reads& A, co
                                         __ldg(a.ia + a.n1 / 2), packed, g, v);
 }
 
-// Inverse pairing of both items: row IFFT u in s -> workspace rows k1 and its
-// mirror: Z(k1, p) = u(p) + i u(L-1-p), Z(kmir, p) = conj(u(p)) + i conj(u(L-1-p)),
-// one column p per thread and iteration; packed lane a: the real and imaginary
-// parts go to rows 0 and N1/2.
+// Inverse pairing of both items: row IFFT u in the registers of the last stage ->
+// workspace rows k1 and its mirror: Z(k1, p) = u(p) + i u(L-1-p), Z(kmir, p) =
+// conj(u(p)) + i conj(u(L-1-p)), the pairs of points p and L-1-p as rowp::inv_pairs
+// joins them; packed lane a: the real and imaginary parts go to rows 0 and N1/2.
 template <int L>
 __device__ __forceinline__ void inv_pair_x2(const soa::C2* v, const Dct2dArgs& a, float2* Zw, int k1, bool packed,
                                             int g) {

@@ -72,7 +72,7 @@ struct Dct2dArgs {
   int nsm;            // host side only: multiprocessors of the device
   long long l2;       // host side only: bytes of L2
   int stream_work;    // two-pass workspace written evict-first (batches of plans larger than L2)
-  int exact;          // host side only: every stage twiddle from the table, b_k2 with its rest (row_pairs.cuh)
+  int exact;          // host side only: every stage twiddle from the table, b_k2 with its rest (side_exact)
   int ahead;          // row groups ahead whose rows a CTA sends for into L2 (0: none; fs2 forward rows)
 };
 
@@ -86,7 +86,7 @@ struct Dct2dArgs {
 // 1.38 / 1.31, 32 x 256 1.39 / 1.48 / 1.37, 512 x 64 1.48 / 1.60 / 1.46, 64 x 2048
 // 1.57 / 1.71 / 1.57; a Poisson solve's potential 512 x 64 1.48 / 1.77 / 1.58.  Time,
 // products -> exact: 203 x 64^2 forward / inverse 5.4 / 6.5 -> 5.9 / 6.8 us (two-sequence
-// 12.7 / 15.8), 2048 x 64 7.4 / 8.2 -> 7.8 / 8.4 (14.5 / 16.9).  Larger sides keep the
+// 12.3 / 15.9), 2048 x 64 7.3 / 7.9 -> 7.7 / 8.0 (14.1 / 17.2).  Larger sides keep the
 // products: they read 4 of 15 twiddles (exact at 4096^2: forward + inverse 12 % slower).
 constexpr bool side_exact(int lg1, int lg2) { return lg1 < 7 || lg2 < 7; }
 

@@ -74,7 +74,7 @@ cudaError_t run_tp_rows_poisson_exact(int lg2, const Dct2dArgs& a, const Poisson
 // and the column pass once each, over a workspace of three entries).
 cudaError_t run_tp_poisson(int log2N1, int log2N2, const Dct2dArgs& a, const PoissonArgs& ps, cudaStream_t s,
                            bool prepare);
-constexpr int kTpPoissonMinLog2 = 6;  // a solve's sides also go down to 64
+constexpr int kTpPoissonMinLog2 = 6;  // sides of solves and of default plans go down to 64
 constexpr int kTpMinLog2N1 = 7, kTpMaxLog2N1 = 13, kTpMinLog2N2 = 7, kTpMaxLog2N2 = 13;
 // Strip widths NP (column pairs per CTA) the two-pass column pass is built
 // for at half-length M: 64 to 512 threads (M/16 per pair), the strip's

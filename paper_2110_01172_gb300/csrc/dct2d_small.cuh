@@ -8,9 +8,10 @@
 // latency when single, and by the extra pass over the workspace in batches;
 // larger ones do not fit the registers of one CTA (64 values per thread, 256
 // threads at 128 registers).  Measured, pair family -> one launch, forward /
-// inverse: 64^2 8.7 / 10.7 -> 3.9 / 4.7 us, 203 x 64^2 12.6 / 15.8 -> 5.4 / 6.3,
-// 2048 x 64^2 75 / 95 -> 16.0 / 18.0, 2048 x (64 x 256) 118 / 143 -> 74 / 75;
-// two-pass family -> one launch: 2048 x 128^2 103 / 101 -> 73 / 75.
+// inverse: 64^2 8.2 / 10.6 -> 3.9 / 4.5 us, 203 x 64^2 12.3 / 15.9 -> 5.9 / 6.8,
+// 2048 x 64^2 74 / 96 -> 18.3 / 19.2, 2048 x (64 x 256) 117 / 143 -> 78 / 80;
+// two-pass family -> one launch: 2048 x 128^2 102 / 98 -> 72 / 76.  All but 128 x 128
+// run exact (Dct2dArgs::exact), which costs 0.5 us of 203 x 64^2 forward.
 //
 // Shared memory of one transform is used in turn as the column FFTs' points
 // (padded, the N2/4 float4 columns interleaved), the workspace rows E, O (E', O'),

@@ -25,8 +25,9 @@
 // Eq. (2d_idct_post).
 //
 // Workspace: N1 rows of N2/2 complex; rows [0, M) hold E (E'), rows [M, N1) O (O').
-// Supported: N1 in {128, ..., 8192}, N2 in {128, ..., 8192}; the solves of
-// gbdct_poisson.cu also run sides of 64.
+// Supported: N1 in {128, ..., 8192}, N2 in {128, ..., 8192}; default plans (above 16384
+// values) and the solves of gbdct_poisson.cu also run sides of 64, with exact kernels
+// (Dct2dArgs::exact).
 #pragma once
 
 #include "dct2d_fs2_kernels.cuh"
@@ -357,8 +358,8 @@ __device__ __forceinline__ void tp_fwd_load(const float2* e1r, const float2* o1r
 // The group's finished rows gathered in its shared buffer and stored whole by the
 // CTA, for outputs that are not device memory: the registers' stores cover L/16
 // columns at a time, which L2 joins but the host link does not (device to page-locked
-// host memory, stored from registers / gathered: 64 x (512 x 64) 230 / 61 us, 64 x (512
-// x 128) 292 / 95).
+// host memory, stored from registers / gathered: 64 x (512 x 64) 230 / 53 us, 64 x (512
+// x 128) 292 / 98).
 template <int L, bool NARROW, bool EXACT>
 __device__ __forceinline__ void tp_fwd_gathered(soa::C2* v, float4* smem, const Dct2dArgs& a, int c, int kb, bool first,
                                                 int g, int pi) {

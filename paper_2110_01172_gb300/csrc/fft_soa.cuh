@@ -176,7 +176,7 @@ __device__ __forceinline__ C2 apply(C2 u, C2 w) {
 // products of at most three of them (a few ulp from the exactly rounded
 // values), which keeps the table reads (and registers) low.  EXACT reads them from
 // the table too: for shapes whose transforms are short enough that the products'
-// error shows in the result (row_pairs.cuh).
+// error shows in the result (side_exact in dct2d_kernels.cuh).
 template <int R>
 struct Tw {
   static constexpr int N = R == 16 ? 4 : R == 8 ? 3 : R == 4 ? 2 : 1;

@@ -55,7 +55,7 @@ namespace {
 // Kernel families (all compute the same transform; chosen by size):
 //   FAM_TP   two passes per direction: half-length column FFTs on strips +
 //            row passes with the radix-2 column step folded in,
-//            N1 in {512..8192}, N2 in {256..8192}
+//            N1, N2 in {128..8192}
 //   FAM_FS2  four-step column steps + two-item row passes (three passes),
 //            N1 in {256..8192}, N2 in {256..16384}
 //   FAM_PAIR two interleaved sequences per thread, 16 <= N1, N2 <= 8192
@@ -491,10 +491,12 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
   }
   // Small shapes of a default plan (no family asked for) run in one launch
   // whatever their family; a forced family keeps its own kernels.  Where the
-  // two-pass family applies (128 x 128) its many CTAs per transform are faster
-  // until there is a transform for half of the SMs (forward, two-pass vs one
-  // launch: batch 1 5.3 vs 6.4 us, 16 5.5 vs 6.4, 203 13.5 vs 10.8, 2048 103 vs 73);
-  // against the pair family one launch won at every batch.
+  // two-pass family applies (128 x 128) its many CTAs per transform are faster for
+  // few transforms; one launch is taken from half an SM count of them on (152 SMs: 76).
+  // Forward, two-pass / one launch: batch 1 5.4 / 6.3 us, 16 5.6 / 6.3, 32 6.4 / 6.4,
+  // 48 7.6 / 6.4, 76 8.9 / 6.5, 152 11.8 / 7.6, 203 13.8 / 10.8, 2048 102 / 72 (inverse
+  // 1 5.9 / 6.9, 32 7.2 / 7.1, 76 8.7 / 7.3, 2048 98 / 76): the break-even is at 32.
+  // Against the pair family one launch won at every batch.
   if (cudaDeviceGetAttribute(&p->nsm, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
     delete p;
     return GBDCT_ERR_CUDA;
@@ -503,7 +505,7 @@ static gbdct_status create_impl(gbdct_plan_t* out, int ndim, const int64_t* dims
                   p->lg1 + p->lg2 <= gbdct::kSmallMaxLog2 && (!tp || 2 * batch >= p->nsm);
   // Default plans with a side of 64 that the pair family would run: the two-pass
   // kernels reach down to 64 as well and are faster (forward, pair -> two-pass: 64 x
-  // 512 11.5 -> 6.0 us, 2048 x 64 14.8 -> 7.4, 128 x (64 x 2048) 69 -> 50, 8192 x 64 23 -> 15).
+  // 512 10.6 -> 5.9 us, 2048 x 64 14.1 -> 7.7, 128 x (64 x 2048) 69 -> 53, 8192 x 64 23.0 -> 15.6).
   p->tp64 = !fname && !poisson && !p->one_launch && p->family == FAM_PAIR && p->lg1 >= gbdct::kTpPoissonMinLog2 &&
             p->lg1 <= gbdct::kTpMaxLog2N1 && p->lg2 >= gbdct::kTpPoissonMinLog2 && p->lg2 <= gbdct::kTpMaxLog2N2;
   const bool exact = p->one_launch ? gbdct::side_exact(p->lg1, p->lg2)

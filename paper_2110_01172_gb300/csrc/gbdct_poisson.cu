@@ -11,10 +11,10 @@
 // and one column pass over the three inverses as a batch, the spectral scalings
 // applied to the spectrum as the row pass reads it.  Small solves are bound by
 // launches and by too few CTAs per launch (512^2: 128 per inverse), large ones
-// by the array passes; separate transforms take nine launches (13 with a side
-// of 64, whose default family is not folded) and the scaling seven more passes
-// over the array.  GPU time per solve, separate -> fused: 64^2 48.5 -> 15.8 us,
-// 64 x 2048 62.5 -> 16.1, 512^2 32.7 -> 16.9, 1024^2 41.4 -> 24.0, 2048^2 92.7 -> 74.1.
+// by the array passes; separate transforms take nine launches and the scaling
+// seven more passes over the array.  GPU time per solve, separate -> fused (separate
+// sides of 64 on the pair family, 13 launches): 64^2 48.5 -> 15.4 us, 64 x 2048
+// 62.5 -> 16.3, 512^2 32.7 -> 16.7, 1024^2 41.4 -> 23.9, 2048^2 92.7 -> 73.6.
 // Other shapes run the library's own plans around one scaling kernel.
 // The eigenvalue denominators 1 / (wu^2 + wv^2) are evaluated in FP64 once,
 // when the solver is created, and rounded once into an FP32 table that every

@@ -7,8 +7,10 @@
 // instead of one: the even frequencies from the sums x_j + x_{N-1-j}, the odd
 // ones from the differences (the inverse: the sum and difference of the two
 // products).  Over both axes a transform is four quadrants (parity p1, p2) and
-// half of the operations and operand bytes of the full products, which is what
-// bounds them: the tiles' operands, through L2.
+// half of the operations and operand bytes of the full products.  What bounds the
+// products at 1024^2 is latency: 128 tiles for 152 SMs, eight blocks of K each, the
+// epilogue behind the last of them (11.4 us a product by ncu; tensor pipe 22 % of a
+// busy SM's cycles, L2 throughput 9 %, warps waiting for tensor memory and stores).
 //
 // Every operand v is split into bf16 parts hi = bf16(v), lo = bf16(v - hi), and
 // each product A B is accumulated in FP32 as hi_A hi_B + hi_A lo_B + lo_A hi_B +

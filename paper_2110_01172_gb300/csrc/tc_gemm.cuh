@@ -6,12 +6,12 @@
 //   D = Ah Bh^T + Ah Bl^T + Al Bh^T + Al Bl^T,
 // all four products accumulated into the same FP32 accumulator in tensor
 // memory.  K advances in blocks of 64 elements: the four operand tiles of a
-// block (128 x 64 and BN x 64 bf16, 128-byte rows with the 128-byte swizzle) arrive by tiled tensor loads into a ring of NST
-// shared-memory stages; one thread issues the loads and the MMAs (K = 16 per
-// instruction) and releases a stage with tcgen05.commit when the MMAs that
-// read it are done.  The four warps then read the accumulator rows back with
-// tcgen05.ld (warp w owns lanes 32w .. 32w+31, lane = tile row) and apply the
-// epilogue:
+// block (128 x 64 and BN x 64 bf16, 128-byte rows with the 128-byte swizzle)
+// arrive by tiled tensor loads into a ring of NST shared-memory stages; one thread
+// issues the loads and the MMAs (K = 16 per instruction) and releases a stage with
+// tcgen05.commit when the MMAs that read it are done.  The four warps then read
+// the accumulator rows back with tcgen05.ld (warp w owns lanes 32w .. 32w+31, lane =
+// tile row) and apply the epilogue:
 //   EPI_SPLIT_T   first product: row (b, p1, i1) of A, column j2 of parity
 //                 p2 = blockIdx.z; stored split and transposed,
 //                 Th/Tl[p1][b][p2][j2][i1], as the K-major operand of the second

@@ -90,7 +90,8 @@ class _Resources:
         graph_pool = 0
         if graph:
             # The whole solve (forward DCT-II, spectral divide, three inverse
-            # transforms: 13 kernel launches) as one CUDA graph, replayed per request.
+            # transforms: four launches where it is fused) as one CUDA graph,
+            # replayed per request.
             side = torch.cuda.Stream(device)
             side.wait_stream(torch.cuda.current_stream(device))
             with torch.cuda.stream(side):
